@@ -63,195 +63,287 @@ __global__ void validate_kernel(uint32_t n, uint32_t w, const uint32_t *__restri
     }
 }
 
-// Maximum-degree-first order.  The block stages the rows in shared memory
-// (when they fit) and computes all degrees; then warp 0 runs the n rounds
-// with the keys in registers: lane l owns the vertices of words
-// [l*JW, l*JW + JW), key = (degree + 1) << 12 | (4095 - u) while u is not
-// placed (0 once placed), so the maximum key is the highest remaining degree
-// with the smallest label.  A round takes the warp's two largest keys,
-// places the first vertex and, when the second is not adjacent to it, the
-// second too (its key is then unchanged while every other key can only
-// fall, so it is the next pick), and decrements the keys of the placed
-// vertices' remaining neighbours.
-template <int JW>
-__device__ __forceinline__ void order_body(uint32_t n, uint32_t w, const uint32_t *__restrict__ rows,
-                                           uint32_t *__restrict__ order, int rows_in_smem, uint32_t *sm)
+// Maximum-degree-first order (Section 4.2) by one block of T threads: highest
+// remaining degree first, smallest label on ties.
+//
+// The order is sequential by definition, but most of a pick's cost is finding
+// the maximum over all vertices and reading rows.  So vertices are placed in
+// rounds.  A round gathers the up to 128 vertices of highest remaining degree
+// (whole degree classes, by a histogram below the maximum), their 128 x 128
+// adjacency bits, and lets one warp pick from them alone, four candidates a
+// lane: a pick is one max-reduction and the removal of one row of bits.  It
+// is the right pick as long as it beats every vertex outside, and those can
+// only fall: the warp stops when the best candidate has fallen to the
+// highest degree outside.  (When the highest degree alone has more than 128
+// vertices, the candidates are the 128 of smallest label, and the first one
+// left out is the one to beat.)  Then all degrees are lowered by the picks'
+// rows at once.  G(1000, 0.3) takes 46 rounds of 22 picks, G(3000, 0.1) 97 of
+// 31, a graph of up to 128 vertices one round.  What bounds it is the chain of
+// picks, about 0.1 us each (max-reduction, one broadcast load, four
+// subtractions), and 3 to 5 us of gathering and barriers a round.  A search of
+// all vertices for one or two picks a round took, per launch (G(n, p), now in
+// brackets): n = 100 24 us (16), 300 85 (57), 500 146 (121), 1000 383 (253),
+// 3000 4345 (756; rows in L2, two dependent reads a round).
+constexpr unsigned kOrderCand = 128;
+
+struct OrderShared {
+    uint32_t adj[kOrderCand][4];   // adjacency among the candidates
+    uint32_t hist[kOrderCand];     // vertices by (maximum degree - degree)
+    uint32_t chunk[4096 / 32];     // vertices of maximum degree by 32 labels (crowded rounds)
+    uint16_t label[kOrderCand];    // the candidates
+    uint16_t placed[kOrderCand];   // this round's picks
+    uint32_t cands, picks, top, beat;
+};
+
+// Bit j of lane i becomes bit i of lane j.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, uint32_t lane)
 {
-    uint32_t *sdeg = sm;                                  // n keys
-    uint32_t *srows = sm + ((n + 3u) & ~3u);              // n * w words (optional)
-    const uint32_t *R = rows;
-    if (rows_in_smem) {
-        for (uint32_t i = threadIdx.x; i < n * w; i += blockDim.x) srows[i] = rows[i];
-        R = srows;
+    const uint32_t mask[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        const uint32_t d = 16u >> s;
+        const uint32_t y = __shfl_xor_sync(FULLM, x, (int)d);
+        x = (lane & d) ? ((x & ~mask[s]) | ((y >> d) & mask[s])) : ((x & mask[s]) | ((y << d) & ~mask[s]));
+    }
+    return x;
+}
+
+// deg[u] = remaining degree + 1, 0 once placed (n entries in shared memory).
+// Rows that are not a simple graph's (flagged by the validation) give some
+// order and stay in bounds: degrees are clamped and never fall below 1.
+template <unsigned T>
+__device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint32_t *R, uint32_t *__restrict__ order,
+                                             uint16_t *deg, OrderShared &sh)
+{
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    constexpr uint32_t NW = T / 32u;
+    const uint32_t chunks = (n + 31u) / 32u;
+    if (t == 0) sh.top = 0u;
+    for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[i] = 0u;
+    __syncthreads();
+    {
+        uint32_t mx = 0u;
+        for (uint32_t u = t; u < n; u += T) {
+            uint32_t d = 0;
+#pragma unroll 4
+            for (uint32_t j = 0; j < w; ++j) d += (uint32_t)__popc(R[(size_t)u * w + j]);
+            d = (d < 4095u ? d : 4095u) + 1u;
+            deg[u] = (uint16_t)d;
+            mx = d > mx ? d : mx;
+        }
+        mx = __reduce_max_sync(FULLM, mx);
+        if (lane == 0) atomicMax(&sh.top, mx);
     }
     __syncthreads();
-    for (uint32_t u = threadIdx.x; u < n; u += blockDim.x) {
-        uint32_t deg = 0;
-        for (uint32_t j = 0; j < w; ++j) deg += __popc(R[(size_t)u * w + j]);
-        sdeg[u] = ((deg + 1u) << 12) | (4095u - u);
-    }
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-
-    const uint32_t lane = threadIdx.x;
-    uint32_t key[32 * JW];
-#pragma unroll
-    for (int q = 0; q < JW; ++q)
-#pragma unroll
-        for (int b = 0; b < 32; ++b) {
-            const uint32_t u = (lane * JW + q) * 32u + b;
-            key[q * 32 + b] = u < n ? sdeg[u] : 0u;
+    for (uint32_t done = 0; done < n;) {
+        const uint32_t M = sh.top;
+        if (t == 0) {
+            sh.cands = 0u;
+            sh.beat = 0u;
         }
-
-    for (uint32_t i = 0; i < n;) {
-        uint32_t a1 = 0u, a2 = 0u;
+        for (uint32_t u = t; u < n; u += T) {
+            const uint32_t d = deg[u];
+            if (d != 0u && M - d < kOrderCand) atomicAdd(&sh.hist[M - d], 1u);
+        }
+        __syncthreads();
+        // degree classes M, M - 1, ... that fit together (every warp computes
+        // the same number)
+        uint32_t classes;
+        {
+            const uint4 h = *reinterpret_cast<const uint4 *>(&sh.hist[4u * lane]);
+            const uint32_t s4 = h.x + h.y + h.z + h.w;
+            uint32_t incl = s4;
 #pragma unroll
-        for (int t = 0; t < 32 * JW; ++t) {
-            const uint32_t k = key[t];
-            if (k > a1) {
-                a2 = a1;
-                a1 = k;
-            } else if (k > a2) {
-                a2 = k;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULLM, incl, o);
+                incl += (int)lane >= o ? y : 0u;
+            }
+            const uint32_t e = incl - s4, c0 = e + h.x, c1 = c0 + h.y, c2 = c1 + h.z, c3 = c2 + h.w;
+            classes = (c0 <= kOrderCand) + (c1 <= kOrderCand) + (c2 <= kOrderCand) + (c3 <= kOrderCand);
+            classes = __reduce_add_sync(FULLM, classes);
+        }
+        if (classes != 0u) {
+            for (uint32_t c = warp; c < chunks; c += NW) {
+                const uint32_t u = c * 32u + lane, d = u < n ? deg[u] : 0u;
+                const uint32_t in = __ballot_sync(FULLM, d != 0u && M - d < classes);
+                if (in == 0u) continue;
+                uint32_t at = 0u;
+                if (lane == 0) at = atomicAdd(&sh.cands, (uint32_t)__popc(in));
+                at = __shfl_sync(FULLM, at, 0) + (uint32_t)__popc(in & ((1u << lane) - 1u));
+                if ((in >> lane) & 1u) sh.label[at] = (uint16_t)u;
+            }
+        } else {  // more than 128 vertices of the maximum degree: the smallest labels
+            for (uint32_t c = warp; c < chunks; c += NW) {
+                const uint32_t u = c * 32u + lane;
+                const uint32_t b = __ballot_sync(FULLM, u < n && deg[u] == M);
+                if (lane == 0) sh.chunk[c] = (uint32_t)__popc(b);
+            }
+            __syncthreads();
+            for (uint32_t c = warp; c < chunks; c += NW) {
+                uint32_t before = 0u;
+                for (uint32_t x = lane; x < c; x += 32u) before += sh.chunk[x];
+                before = __reduce_add_sync(FULLM, before);
+                const uint32_t u = c * 32u + lane;
+                const bool in = u < n && deg[u] == M;
+                const uint32_t at = before + (uint32_t)__popc(__ballot_sync(FULLM, in) & ((1u << lane) - 1u));
+                if (in && at < kOrderCand) sh.label[at] = (uint16_t)u;
+                if (in && at == kOrderCand) sh.beat = (M << 12) | (4095u - u);
+            }
+            if (t == 0) sh.cands = kOrderCand;
+        }
+        __syncthreads();
+        const uint32_t m = sh.cands;
+        // their adjacency, four rows a warp at a time (16 loads in flight)
+        {
+            uint32_t wd[4], sf[4];  // word and bit of this lane's columns
+            bool on[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t c = lane + 32u * k;
+                on[k] = c < m;
+                const uint32_t u = on[k] ? sh.label[c] : 0u;
+                wd[k] = u >> 5;
+                sf[k] = u & 31u;
+            }
+            for (uint32_t r0 = warp * 4u; r0 < m; r0 += NW * 4u) {
+                uint32_t x[4][4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t *row = R + (size_t)sh.label[r0 + q < m ? r0 + q : 0u] * w;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) x[q][k] = row[wd[k]];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t b[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) b[k] = __ballot_sync(FULLM, on[k] && ((x[q][k] >> sf[k]) & 1u));
+                    if (lane == 0 && r0 + q < m)
+                        *reinterpret_cast<uint4 *>(sh.adj[r0 + q]) = make_uint4(b[0], b[1], b[2], b[3]);
+                }
             }
         }
-        const uint32_t b1 = __reduce_max_sync(FULLM, a1);
-        const uint32_t b2 = __reduce_max_sync(FULLM, a1 == b1 ? a2 : a1);
-        const uint32_t v = 4095u - (b1 & 4095u);
-        const uint32_t v2 = 4095u - (b2 & 4095u);
-        const uint32_t *rv = R + (size_t)v * w;
-        const bool two = b2 != 0u && !((rv[v2 >> 5] >> (v2 & 31u)) & 1u);
-        const uint32_t *rv2 = R + (size_t)v2 * w;
-        if (lane == 0) {
-            order[i] = v;
-            if (two) order[i + 1] = v2;
-        }
+        __syncthreads();
+        if (warp == 0) {
+            // key: degree + 1 (13 bits) | 4095 - label (12) | candidate (7)
+            uint32_t key[4], open[4];  // open: 1 until the candidate is picked
 #pragma unroll
-        for (int q = 0; q < JW; ++q) {
-            const uint32_t wi = lane * JW + q;
-            const uint32_t word = wi < w ? rv[wi] : 0u;
-            const uint32_t word2 = (two && wi < w) ? rv2[wi] : 0u;
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t c = lane + 32u * k;
+                const uint32_t u = c < m ? sh.label[c] : 0u;
+                open[k] = c < m ? 1u : 0u;
+                key[k] = c < m ? ((uint32_t)deg[u] << 19) | ((4095u - u) << 7) | c : 0u;
+            }
+            // the (degree + 1, 4095 - label) to beat; whole classes: any
+            // degree above the classes taken
+            const uint32_t beat = classes != 0u ? ((M - classes < M ? M - classes : 0u) << 12) | 4095u : sh.beat;
+            // (a row that is not a simple graph's can take a degree field below
+            // zero: the candidate is then picked out of turn, and nothing else)
+            uint32_t picks = 0u, floor_key = 0u;  // the first pick always stands
+#pragma unroll 2
+            for (; picks < m; ++picks) {
+                const uint32_t a = key[0] > key[1] ? key[0] : key[1], b = key[2] > key[3] ? key[2] : key[3];
+                const uint32_t best = __reduce_max_sync(FULLM, a > b ? a : b);
+                if (best <= floor_key) break;
+                floor_key = (beat << 7) | 127u;
+                const uint4 row = *reinterpret_cast<const uint4 *>(sh.adj[best & 127u]);
+                if (lane == 0) sh.placed[picks] = (uint16_t)(4095u - ((best >> 7) & 4095u));
+                const uint32_t rw[4] = {row.x, row.y, row.z, row.w};
 #pragma unroll
-            for (int b = 0; b < 32; ++b) {
-                uint32_t k = key[q * 32 + b];
-                const uint32_t u = wi * 32u + b;
-                if (u == v || (two && u == v2)) k = 0u;
-                else if (k) k -= (((word >> b) & 1u) + ((word2 >> b) & 1u)) << 12;
-                key[q * 32 + b] = k;
+                for (int k = 0; k < 4; ++k) {
+                    const bool own = key[k] == best;
+                    const uint32_t lower = key[k] - (((rw[k] >> lane) & open[k]) << 19);
+                    key[k] = own ? 0u : lower;
+                    open[k] = own ? 0u : open[k];
+                }
+            }
+            __syncwarp();
+            for (uint32_t x = lane; x < picks; x += 32u) {
+                const uint32_t u = sh.placed[x];
+                order[done + x] = u;
+                deg[u] = 0u;
+            }
+            if (lane == 0) {
+                sh.picks = picks;
+                sh.top = 0u;
             }
         }
-        i += two ? 2u : 1u;
+        __syncthreads();
+        const uint32_t picks = sh.picks;
+        done += picks;
+        // lower the degrees: lane j reads its pick's word for 32 vertices (four
+        // such words in flight), a transposition gives lane i the picks'
+        // bits of vertex i, and their population count is its loss
+        uint32_t mx = 0u;
+        for (uint32_t c0 = warp; c0 < chunks; c0 += NW * 4u) {
+            uint32_t dec[4] = {0u, 0u, 0u, 0u};
+            for (uint32_t p0 = 0; p0 < picks; p0 += 32u) {
+                const bool on = p0 + lane < picks;
+                const uint32_t *row = R + (size_t)sh.placed[on ? p0 + lane : 0u] * w;
+                uint32_t x[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[q] = on && c0 + q * NW < chunks ? row[c0 + q * NW] : 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) dec[q] += (uint32_t)__popc(transpose_bits(x[q], lane));
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t u = (c0 + q * NW) * 32u + lane;
+                uint32_t d = u < n ? deg[u] : 0u;
+                if (d != 0u) {
+                    d = d > dec[q] + 1u ? d - dec[q] : 1u;
+                    deg[u] = (uint16_t)d;
+                }
+                mx = d > mx ? d : mx;
+            }
+        }
+        mx = __reduce_max_sync(FULLM, mx);
+        if (lane == 0) atomicMax(&sh.top, mx);
+        for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[i] = 0u;
+        __syncthreads();
     }
 }
 
-// The same order for one graph with the whole block (eight warps): thread t
-// owns the keys of vertices t, t + 256, ... (KP of them).  A round finds the
-// two largest keys of the block (each warp's two largest by two
-// __reduce_max_sync, the block's through a double-buffered pair of slots
-// per warp in shared memory: one barrier per round -- a warp cannot reach
-// round r + 2's write before every warp has passed round r + 1's barrier,
-// after its reads of round r), places the first vertex v1, and places the
-// second one v2 in the same round when v2 is not adjacent to v1: then v2's
-// key is unchanged by placing v1 while every other key can only fall, so v2
-// is exactly the next maximum-degree vertex (labels make keys distinct).  On
-// G(n, 0.3) about two vertices in three rounds go in pairs.  Finally the keys
-// of the placed vertices' remaining neighbours are decremented.
-template <int KP>
-__global__ void __launch_bounds__(256) order_kernel(uint32_t n, uint32_t w, const uint32_t *__restrict__ rows,
-                                                   uint32_t *__restrict__ order, int rows_in_smem)
+// Shared memory of an ordering block: its state, the degrees, and the rows
+// when they fit.
+__host__ __device__ inline size_t order_fixed_bytes(uint32_t n)
 {
-    extern __shared__ __align__(16) uint32_t sm[];
-    uint32_t *mx = sm;              // [2 rounds][8 warps][2 keys]
-    uint32_t *srows = sm + 32;      // n * w words (optional)
-    const uint32_t *R = rows;
+    return (sizeof(OrderShared) + 15) / 16 * 16 + ((size_t)n * 2 + 15) / 16 * 16;
+}
+
+template <unsigned T>
+__device__ __forceinline__ void order_block(uint32_t n, uint32_t w, const uint32_t *__restrict__ rows,
+                                            uint32_t *__restrict__ order, bool rows_in_smem, unsigned char *sm)
+{
+    OrderShared &sh = *reinterpret_cast<OrderShared *>(sm);
+    uint16_t *deg = reinterpret_cast<uint16_t *>(sm + (sizeof(OrderShared) + 15) / 16 * 16);
     if (rows_in_smem) {
-        for (uint32_t i = threadIdx.x; i < n * w; i += blockDim.x) srows[i] = rows[i];
-        R = srows;
-    }
-    __syncthreads();
-    const uint32_t t = threadIdx.x;
-    uint32_t key[KP];
-#pragma unroll
-    for (int q = 0; q < KP; ++q) {
-        const uint32_t u = t + 256u * q;
-        uint32_t k = 0u;
-        if (u < n) {
-            uint32_t deg = 0;
-            for (uint32_t j = 0; j < w; ++j) deg += __popc(R[(size_t)u * w + j]);
-            k = ((deg + 1u) << 12) | (4095u - u);
-        }
-        key[q] = k;
-    }
-    uint32_t i = 0, rd = 0;
-    while (i < n) {
-        uint32_t a1 = 0u, a2 = 0u;  // this thread's two largest keys
-#pragma unroll
-        for (int q = 0; q < KP; ++q) {
-            const uint32_t k = key[q];
-            if (k > a1) {
-                a2 = a1;
-                a1 = k;
-            } else if (k > a2) {
-                a2 = k;
-            }
-        }
-        const uint32_t w1 = __reduce_max_sync(FULLM, a1);
-        const uint32_t w2 = __reduce_max_sync(FULLM, a1 == w1 ? a2 : a1);
-        volatile uint32_t *slot = mx + (rd & 1u) * 16u;
-        if ((t & 31u) == 0u) {
-            slot[2u * (t >> 5)] = w1;
-            slot[2u * (t >> 5) + 1u] = w2;
-        }
+        uint32_t *srows = reinterpret_cast<uint32_t *>(sm + order_fixed_bytes(n));
+#pragma unroll 8
+        for (uint32_t i = threadIdx.x; i < n * w; i += T) srows[i] = rows[i];
         __syncthreads();
-        uint32_t b1 = 0u, b2 = 0u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t x1 = slot[2 * j], x2 = slot[2 * j + 1];
-            if (x1 > b1) {
-                b2 = x2 > b1 ? x2 : b1;
-                b1 = x1;
-            } else if (x1 > b2) {
-                b2 = x1;
-            }
-        }
-        const uint32_t v1 = 4095u - (b1 & 4095u);
-        const uint32_t v2 = 4095u - (b2 & 4095u);
-        const uint32_t *r1 = R + (size_t)v1 * w;
-        const bool two = b2 != 0u && !((r1[v2 >> 5] >> (v2 & 31u)) & 1u);
-        const uint32_t *r2 = R + (size_t)v2 * w;
-        if (t == 0) {
-            order[i] = v1;
-            if (two) order[i + 1] = v2;
-        }
-#pragma unroll
-        for (int q = 0; q < KP; ++q) {
-            const uint32_t u = t + 256u * q;
-            if (u < n) {
-                uint32_t k = key[q];
-                if (u == v1 || (two && u == v2)) {
-                    k = 0u;
-                } else if (k) {
-                    uint32_t dec = (r1[u >> 5] >> (u & 31u)) & 1u;
-                    if (two) dec += (r2[u >> 5] >> (u & 31u)) & 1u;
-                    k -= dec << 12;
-                }
-                key[q] = k;
-            }
-        }
-        i += two ? 2u : 1u;
-        ++rd;
+        order_rounds<T>(n, w, srows, order, deg, sh);
+    } else {
+        order_rounds<T>(n, w, rows, order, deg, sh);
     }
+}
+
+template <unsigned T>
+__global__ void __launch_bounds__(T) order_kernel(uint32_t n, uint32_t w, const uint32_t *__restrict__ rows,
+                                                  uint32_t *__restrict__ order, int rows_in_smem)
+{
+    extern __shared__ __align__(16) unsigned char osm[];
+    order_block<T>(n, w, rows, order, rows_in_smem != 0, osm);
 }
 
 // One block per graph of a batch; the rows go to shared memory when they fit
 // in the launch's dynamic shared memory.
-template <int JW>
 __global__ void __launch_bounds__(256) order_batch_kernel(const BatchGraph *__restrict__ graphs, size_t smem_bytes)
 {
-    extern __shared__ __align__(16) uint32_t sm[];
+    extern __shared__ __align__(16) unsigned char osm[];
     const BatchGraph gd = graphs[blockIdx.x];
-    const size_t need = (size_t)((gd.n + 3u) & ~3u) * 4 + (size_t)gd.n * gd.w * 4;
-    order_body<JW>(gd.n, gd.w, gd.rows, gd.order, need <= smem_bytes, sm);
+    const size_t need = order_fixed_bytes(gd.n) + (size_t)gd.n * gd.w * 4;
+    order_block<256>(gd.n, gd.w, gd.rows, gd.order, need <= smem_bytes, osm);
 }
 
 __global__ void identity_kernel(uint32_t n, uint32_t *order)
@@ -330,20 +422,19 @@ cudaError_t launch_validate_rows(uint32_t n, uint32_t w, const uint32_t *rows, u
 cudaError_t launch_order(uint32_t n, uint32_t w, const uint32_t *rows, uint32_t *order, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    const size_t rbytes = (size_t)n * w * 4;
-    const int in_smem = (128 + rbytes) <= 200u * 1024u;
-    const size_t smem = 128 + (in_smem ? rbytes : 0);
-    const void *k = nullptr;
-    void (*f)(uint32_t, uint32_t, const uint32_t *, uint32_t *, int) = nullptr;
-    if (n <= 256) f = order_kernel<1>;
-    else if (n <= 512) f = order_kernel<2>;
-    else if (n <= 1024) f = order_kernel<4>;
-    else if (n <= 2048) f = order_kernel<8>;
-    else f = order_kernel<16>;
-    k = (const void *)f;
-    cudaError_t e = kernel_smem_setup(k);
+    // rows in shared memory up to 200 KB; more threads where there are more
+    // vertices to look at, fewer where barriers cost more than they save (256 /
+    // 512 / 1024 threads: n = 500 122 / 121 / 127 us, 1000 266 / 253 / 278, 3000
+    // 961 / 812 / 756)
+    const size_t fixed = order_fixed_bytes(n), rbytes = (size_t)n * w * 4;
+    const int in_smem = fixed + rbytes <= 200u * 1024u;
+    const size_t smem = fixed + (in_smem ? rbytes : 0);
+    const unsigned threads = n <= 128 ? 128u : (n <= 1024 ? 512u : 1024u);
+    void (*f)(uint32_t, uint32_t, const uint32_t *, uint32_t *, int) =
+        threads == 128u ? order_kernel<128> : (threads == 512u ? order_kernel<512> : order_kernel<1024>);
+    cudaError_t e = kernel_smem_setup((const void *)f);
     if (e != cudaSuccess) return e;
-    f<<<1, 256, smem, s>>>(n, w, rows, order, in_smem);
+    f<<<1, threads, smem, s>>>(n, w, rows, order, in_smem);
     return cudaGetLastError();
 }
 
@@ -389,24 +480,16 @@ cudaError_t kernel_smem_setup(const void *func)
 
 cudaError_t prepare_order_batch(uint32_t max_n, uint32_t max_w, size_t *smem)
 {
-    const size_t keys = ((max_n + 3u) & ~3u) * sizeof(uint32_t);
-    const size_t rbytes = (size_t)max_n * max_w * 4;
-    *smem = keys + ((keys + rbytes) <= 200u * 1024u ? rbytes : 0);
-    const uint32_t words = (max_n + 31) / 32;
-    cudaError_t e;
-    if (words <= 32) e = cudaFuncSetAttribute(order_batch_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-    else if (words <= 64) e = cudaFuncSetAttribute(order_batch_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-    else e = cudaFuncSetAttribute(order_batch_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-    return e;
+    const size_t fixed = order_fixed_bytes(max_n), rbytes = (size_t)max_n * max_w * 4;
+    *smem = fixed + (fixed + rbytes <= 200u * 1024u ? rbytes : 0);
+    return kernel_smem_setup((const void *)order_batch_kernel);
 }
 
 cudaError_t launch_order_batch(const BatchGraph *graphs, uint32_t count, uint32_t max_n, size_t smem, cudaStream_t s)
 {
+    (void)max_n;
     if (count == 0) return cudaSuccess;
-    const uint32_t words = (max_n + 31) / 32;
-    if (words <= 32) order_batch_kernel<1><<<count, 256, smem, s>>>(graphs, smem);
-    else if (words <= 64) order_batch_kernel<2><<<count, 256, smem, s>>>(graphs, smem);
-    else order_batch_kernel<4><<<count, 256, smem, s>>>(graphs, smem);
+    order_batch_kernel<<<count, 256, smem, s>>>(graphs, smem);
     return cudaGetLastError();
 }
 
