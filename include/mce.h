@@ -125,13 +125,14 @@ extern "C" {
 typedef struct {
     uint32_t pivot_mode;        /* MCE_PIVOT_*                                */
     uint32_t flags;             /* MCE_ORDER_IDENTITY | MCE_LIST | ...        */
-    uint32_t lanes_per_subtree; /* lanes of a warp that share one search
-                                   subtree: 1,2,4,8,16,32; 0 = autotuned       */
-    uint32_t words_per_lane;    /* 32-bit words of each set a lane holds:
-                                   1,2,4; 0 = autotuned                       */
+    uint32_t lanes_per_subtree; /* lanes that hold a row of the adjacency:
+                                   1,2,4,8,16,32; 0 = by n (a whole warp
+                                   searches a subtree in any case)            */
+    uint32_t words_per_lane;    /* 32-bit words of a row a lane holds:
+                                   1,2,4; 0 = by n                            */
     uint32_t blocks;            /* persistent grid size; 0 = one wave         */
-    uint32_t threads_per_block; /* 0 = autotuned; a multiple of 32, at most
-                                   512 (else MCE_EINVAL)                      */
+    uint32_t threads_per_block; /* 0 = 768 or fewer; a multiple of 32, at
+                                   most 512 (else MCE_EINVAL)                 */
     uint64_t timeout_ns;        /* device-side wait budget: a search whose
                                    idle warps see no progress for this long
                                    stops with MCE_ETIMEOUT; 0 = 60 s          */
@@ -139,8 +140,7 @@ typedef struct {
                                    frames spill to the device work queue,
                                    1..64; 0 = 64                              */
     uint32_t queue_log2;        /* log2 of the device work-queue slots, <= 24;
-                                   0 = auto (at least four times the subtree
-                                   groups).  mce_enumerate retries a search
+                                   0 = auto (at least four times the warps).  mce_enumerate retries a search
                                    that overflowed with a 16x larger queue.   */
     uint32_t split_min_p;       /* a new subtree whose candidate set P has at
                                    least this many vertices is published to
@@ -165,9 +165,9 @@ typedef struct {
 #define MCE_OUT_DONATIONS  7   /* work frames handed between warps           */
 #define MCE_OUT_STEALS     8   /* frames taken from a work queue (any level) */
 #define MCE_OUT_GLOBAL     9   /* ... of which from the device-wide queue    */
-#define MCE_OUT_BUSY_NS   10   /* subtree-group time spent holding a frame:
+#define MCE_OUT_BUSY_NS   10   /* warp time spent holding a frame:
                                   utilisation = busy / (groups x duration)   */
-#define MCE_OUT_GROUPS    11   /* subtree groups of the launch               */
+#define MCE_OUT_GROUPS    11   /* warps of the launch                        */
 #define MCE_OUT_GPUSH     12   /* frames published to the device-wide queue  */
 #define MCE_OUT_GTRY      13   /* claims of frames from it (one fetch-and-add
                                   each, for up to four frames)              */
@@ -175,9 +175,9 @@ typedef struct {
                                   counters (block-private rings of the
                                   batched form; the device-wide queue
                                   takes tickets by fetch-and-add)           */
-#define MCE_OUT_LANE_TASKS 15  /* subtrees handed to single lanes (frames
-                                  whose P u X has at most 32 vertices,
-                                  searched with 32-bit local sets)          */
+#define MCE_OUT_LANE_TASKS 15  /* subtrees handed to the warp tier (frames
+                                  whose P u X has at most 128 vertices,
+                                  searched a node per lane)                 */
 #define MCE_OUT_HIST       16
 #define MCE_OUT_WORDS(n)   (MCE_OUT_HIST + (uint64_t)(n) + 1)
 
@@ -394,9 +394,9 @@ int mce_batch_create(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count,
  * classed by words per row (1, 2, 4, ..., 128).  Classes with a choice cached
  * in the context (per class and pivot rule) take it; the others, if they hold
  * at least 16 graphs of the batch, are tuned by coordinate descent in
- * decreasing order of expected work: every candidate for the class -- 1, 2
- * or 4 words per lane with the fewest lanes that hold a row, 128 / 256 / 512
- * threads per block, then the best with the breadth-first split off -- is
+ * decreasing order of expected work: every candidate for the class -- 128 /
+ * 256 / 512 threads per block, then the best with the breadth-first split
+ * off -- is
  * timed as one captured launch of the whole batch (up to 4096 of its graphs,
  * sampled evenly) with the other classes at their current choice, and the
  * fastest is kept and cached.  Classes with fewer graphs use the built-in
@@ -476,10 +476,9 @@ uint64_t mce_ctx_mem_used(const mce_ctx *ctx);
  * caller-owned, zeroed by the caller) is split evenly between the launch's
  * blocks; each block appends 16-byte records whenever it refreshes its view
  * of the device-wide queue (about every 2 us while it runs):
- *   uint64 globaltimer ns, uint16 busy groups of the block, uint16 lanes of
- *   the block holding a lane-tier subproblem (frames whose P u X has at most
- *   32 vertices), uint16 frames in the device-wide queue (saturating),
- *   uint16 starving blocks (saturating).
+ *   uint64 globaltimer ns, uint16 busy warps of the block, uint16 0,
+ *   uint16 frames in the device-wide queue (saturating), uint16 idle warps of
+ *   the whole launch (saturating).
  * Records past a block's share are dropped. */
 int mce_trace_enable(void *d_buf, uint64_t bytes);
 

@@ -81,18 +81,16 @@ __attribute__((constructor)) void fault_from_env()
 // Launch configuration
 
 struct Config {
-    int G = 32, K = 1;
+    int G = 32, K = 1;  // the caller's shape: rows of G * K words
     bool smem = false;
     unsigned threads = 0, blocks = 0;
-    uint32_t stack_levels = 0, stack_offset = 0;
     size_t smem_bytes = 0;
     uint32_t wp = 32;
     uint32_t qcap = 1024, fs = 0;
     uint32_t total_groups = 0;
     int pivot = 0;
     bool list = false;  // frames carry R (clique listing)
-    uint32_t t2_offset = 0, t2_levels = 0, t2_max_p = 0;  // lane tier (t2_max_p 0: off)
-    bool seed = false;  // start from the root's children
+    uint32_t t2_offset = 0, pool_bytes = 0, t2_max_p = 0, direct_offset = 0;  // warp tier (t2_max_p 0: off)
     uint32_t local_slots = kLocalSlots;  // block ring slots
     SearchImpl impl{nullptr, nullptr, nullptr, nullptr};
 };
@@ -108,22 +106,21 @@ mce_options defaults(const mce_options *o)
     return d;
 }
 
-SearchImpl impl_for(int G, int K, bool smem, int pivot, bool list = false)
+// The search kernels for sets of `words` 32-bit words: one, two or four words
+// per lane of a warp.
+SearchImpl impl_for(uint32_t words, bool smem, int pivot, bool list = false)
 {
     if (pivot == MCE_PIVOT_GREEDY_NX) pivot = MCE_PIVOT_GREEDY_TX;  // the TX kernels, early exit on
-#define MCE_IMPL_CASE(g, k)                                                                                \
-    case g * 8 + k:                                                                                        \
-        return list ? search_list_impl_##g##_##k(smem, pivot) : search_impl_##g##_##k(smem, pivot);
-    switch (G * 8 + K) {
-        MCE_IMPL_CASE(1, 1) MCE_IMPL_CASE(1, 2) MCE_IMPL_CASE(1, 4)
-        MCE_IMPL_CASE(2, 1) MCE_IMPL_CASE(2, 2) MCE_IMPL_CASE(2, 4)
-        MCE_IMPL_CASE(4, 1) MCE_IMPL_CASE(4, 2) MCE_IMPL_CASE(4, 4)
-        MCE_IMPL_CASE(8, 1) MCE_IMPL_CASE(8, 2) MCE_IMPL_CASE(8, 4)
-        MCE_IMPL_CASE(16, 1) MCE_IMPL_CASE(16, 2) MCE_IMPL_CASE(16, 4)
-        MCE_IMPL_CASE(32, 1) MCE_IMPL_CASE(32, 2) MCE_IMPL_CASE(32, 4)
-    default: return {nullptr, nullptr, nullptr, nullptr};
-    }
-#undef MCE_IMPL_CASE
+    if (words <= 32) return list ? search_list_impl_1(smem, pivot) : search_impl_1(smem, pivot);
+    if (words <= 64) return list ? search_list_impl_2(smem, pivot) : search_impl_2(smem, pivot);
+    if (words <= 128) return list ? search_list_impl_4(smem, pivot) : search_impl_4(smem, pivot);
+    return {nullptr, nullptr, nullptr, nullptr};
+}
+
+// Shapes a caller may ask for.
+bool shape_known(int G, int K)
+{
+    return (G == 1 || G == 2 || G == 4 || G == 8 || G == 16 || G == 32) && (K == 1 || K == 2 || K == 4);
 }
 
 uint32_t next_pow2(uint64_t x)
@@ -140,29 +137,16 @@ size_t search_smem(uint32_t n, uint32_t wp, bool rows_in_smem, bool list = false
 
 constexpr uint32_t kListFlags = MCE_LIST | MCE_LIST_SORTED;
 
-// Shared-memory stack: as many levels (up to kStackSmemMax) as fit between
-// `base` (rows, hash terms, histogram, block ring) and `limit`.
-void plan_stack_for(uint32_t base, int G, int K, unsigned threads, size_t limit, uint32_t &levels, uint32_t &offset,
-                    size_t &total)
+// Bytes of a warp's region of the warp tier: its share of the shared memory
+// between `base` and `limit`.
+uint32_t plan_pool(size_t base, unsigned threads, size_t limit)
 {
-    offset = (uint32_t)round_up(base, 16);
-    const size_t per_level = (size_t)(threads / 32) * stack_level_words(G, K) * 32 * 4;
-    const size_t avail = limit > offset ? limit - offset : 0;
-    levels = (uint32_t)std::min<size_t>(kStackSmemMax, avail / per_level);
-    total = offset + (size_t)levels * per_level;
+    const size_t each = limit > base ? (limit - base) / (threads / 32) / 16 * 16 : 0;
+    return (uint32_t)std::min<size_t>(kPoolBytesMax, std::max<size_t>(kPoolBytesMin, each));
 }
 
-// Default subtree shape (lanes G x words per lane K).  With the lane tier
-// taking the small subproblems, one word per lane and as many lanes as the
-// row has words won up to 24 words per row: measured on one graph of each
-// size, whole path (old four-word shapes in brackets), G(45) Moon-Moser 1.33
-// (1.48) ms, G(100, 0.5) 0.27 (0.29), G(128, 0.7) 1.29 (1.84), G(200, 0.55)
-// 1.36 (2.10), G(256, 0.5) 1.44 (2.52), G(300, 0.5) 2.11 (2.96), G(700, 0.3)
-// 1.55 (1.66) ms.  At 13-16 words two words per lane led (G(500, 0.4): 2.63
-// against 2.76 with one and 3.15 with four), at 25-32 four (G(1000, 0.3):
-// 7.28 against 7.96 with two and 8.97 with one: 32 one-word lanes per
-// subtree leave a block too few subtrees), above 32 two (G(1500, 0.15) and
-// G(2000, 0.1): 2.53 / 2.60 against 2.59 / 2.67 with four).
+// Default row width of n vertices, as lanes x words per lane: the smallest
+// power of two that holds them, a whole warp's above 16 words.
 void default_shape(uint32_t n, int &G, int &K)
 {
     const uint32_t W = std::max<uint32_t>(1, (n + 31) / 32);
@@ -192,27 +176,20 @@ void pick_shape(uint32_t n, const mce_options &o, int &G, int &K)
     }
 }
 
-// The search kernels are built for at most kMaxThreads threads per block
-// (128 registers per thread: the group state of four-word lanes, and no
-// spills for the narrower shapes), and the plain form launches that many.
-// On graphs of up to 128 vertices 512 threads beat 256 wherever the search
-// has real work (0.65-0.89x the time) and lost 3-9 % on the smallest,
-// launch-bound ones.
+// Most threads per block a caller may ask for; the library's own choice is
+// kLaunchThreads (24 warps, 80 registers per thread: the warp tier's loop
+// needs no more, and more warps hide its shared-memory latencies).
 constexpr unsigned kMaxThreads = 512u;
 
-// stack_cap: most shared memory for the explicit stack per block (the served
-// form keeps blocks small so that several requests share an SM).
-int choose(uint32_t n, const mce_options &o, Config &c, size_t stack_cap = ~(size_t)0)
+int choose(uint32_t n, const mce_options &o, Config &c)
 {
     if (o.pivot_mode > MCE_PIVOT_GREEDY_NX || o.stack_levels > (uint32_t)kStackDepth || o.queue_log2 > 24)
         return MCE_EINVAL;
     const uint32_t W = std::max<uint32_t>(1, (n + 31) / 32);
     int G, K;
     pick_shape(n, o, G, K);
-    if ((uint32_t)(G * K) < W) return MCE_EINVAL;
+    if ((uint32_t)(G * K) < W || !shape_known(G, K)) return MCE_EINVAL;
     c.list = (o.flags & kListFlags) != 0u;
-    c.impl = impl_for(G, K, false, (int)o.pivot_mode, c.list);
-    if (!c.impl.run) return MCE_EINVAL;
     c.G = G;
     c.K = K;
     c.wp = (uint32_t)(G * K);
@@ -224,72 +201,29 @@ int choose(uint32_t n, const mce_options &o, Config &c, size_t stack_cap = ~(siz
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return MCE_ECUDA;
     const size_t limit = (size_t)optin - 1024;  // static shared memory + slack
 
-    c.threads = o.threads_per_block ? o.threads_per_block : kMaxThreads;
-    if (c.threads % 32 || c.threads > kMaxThreads) return MCE_EINVAL;
+    c.threads = o.threads_per_block ? o.threads_per_block : kLaunchThreads;
+    if (c.threads % 32 || (o.threads_per_block && c.threads > kMaxThreads)) return MCE_EINVAL;
 
-    // The lane tier (counting kernels, groups of two or more lanes; in the
-    // served form, whose stack is capped so that requests share SMs, when
-    // serve_t2 is set) needs t2_warp_bytes per warp.  Rows stay in shared
-    // memory when they fit beside it; otherwise, with t2_smem_rows, the block
-    // gets fewer warps so that they fit, or they are read from L2.
+    // Shared memory: rows of up to t2_smem_words words, and a region per warp
+    // for the warp tier; fewer warps where the regions do not fit.
     const Tuning tu = default_tuning();
-    const bool t2 = !c.list && G >= 2 && tu.t2_p != 0 && (stack_cap == ~(size_t)0 || tu.serve_t2);
-    uint32_t t2_levels = tu.t2_levels;
-    size_t t2w = t2 ? t2_warp_bytes(t2_levels, o.pivot_mode != MCE_PIVOT_GREEDY) : 0;
-    auto fits = [&](bool rows_smem, unsigned threads) {
-        return round_up(search_smem(n, c.wp, rows_smem, c.list, c.local_slots), 16) + (size_t)(threads / 32) * t2w <=
-               limit;
+    const uint32_t direct = n <= 128u ? kDirectBytes : 0u;
+    auto base_of = [&](bool rows_smem) {
+        return round_up(search_smem(n, c.wp, rows_smem, c.list, c.local_slots), 16) + direct;
     };
-    c.smem = c.wp <= 32 && fits(true, c.threads);
-    if (!c.smem && t2 && tu.t2_smem_rows && c.wp <= 32 && !o.threads_per_block) {
-        // rows in shared memory with as many warps as fit beside them (one
-        // warp at a time), with fewer lane-tier stack levels in shared memory
-        // (deeper levels go to local memory) and then a half-size block ring
-        // when that buys warps; G(1000, 0.3): 8 warps with four levels, 9
-        // with three, 10 with two, 11 with one, 12 with one and 16 ring
-        // slots (6.2 -> 5.85 ms from 11 to 12)
-        auto most = [&]() {
-            unsigned th = c.threads;
-            while (th >= 128 && !fits(true, th)) th -= 32;
-            return th >= 128 ? th : 0u;
-        };
-        unsigned best = 0;
-        uint32_t best_levels = t2_levels, best_slots = kLocalSlots;
-        for (uint32_t slots : {(uint32_t)kLocalSlots, (uint32_t)kLocalSlotsSmall}) {
-            c.local_slots = slots;
-            for (uint32_t lv = t2_levels; lv >= 1; --lv) {
-                t2w = t2_warp_bytes(lv, o.pivot_mode != MCE_PIVOT_GREEDY);
-                const unsigned th = most();
-                if (th > best) {
-                    best = th;
-                    best_levels = lv;
-                    best_slots = slots;
-                }
-            }
-        }
-        c.local_slots = best_slots;
-        t2_levels = best_levels;
-        t2w = t2_warp_bytes(t2_levels, o.pivot_mode != MCE_PIVOT_GREEDY);
-        if (best) {
-            c.threads = best;
-            c.smem = true;
-        }
-    }
-    if (t2 && !fits(c.smem, c.threads) && !o.threads_per_block)
-        while (c.threads > 128 && !fits(c.smem, c.threads)) c.threads -= 64;
-    const bool t2_on = t2 && fits(c.smem, c.threads);
-    if (c.smem) c.impl = impl_for(G, K, true, (int)o.pivot_mode, c.list);
-    if (search_smem(n, c.wp, c.smem, c.list, c.local_slots) > limit) return MCE_EINVAL;
-
-    size_t base = search_smem(n, c.wp, c.smem, c.list, c.local_slots);
-    if (t2_on) {
-        c.t2_offset = (uint32_t)round_up(base, 16);
-        c.t2_levels = t2_levels;
-        c.t2_max_p = tu.t2_p;
-        base = c.t2_offset + (size_t)(c.threads / 32) * t2w;
-    }
-    const size_t cap = stack_cap < limit - base ? base + stack_cap : limit;
-    plan_stack_for((uint32_t)base, c.G, c.K, c.threads, cap, c.stack_levels, c.stack_offset, c.smem_bytes);
+    auto fits = [&](bool rows_smem, unsigned threads) {
+        return base_of(rows_smem) + (size_t)(threads / 32) * kPoolBytesMin <= limit;
+    };
+    c.smem = W <= 32 && c.wp <= tu.t2_smem_words && fits(true, c.threads);
+    while (c.threads > 32 && !fits(c.smem, c.threads)) c.threads -= 32;
+    if (!fits(c.smem, c.threads)) return MCE_EINVAL;
+    c.impl = impl_for(W, c.smem, (int)o.pivot_mode, c.list);
+    if (!c.impl.run) return MCE_EINVAL;
+    c.t2_offset = (uint32_t)base_of(c.smem);
+    c.direct_offset = c.t2_offset - direct;
+    c.pool_bytes = plan_pool(c.t2_offset, c.threads, limit);
+    c.t2_max_p = c.list ? 0u : tu.t2_p;
+    c.smem_bytes = c.t2_offset + (size_t)(c.threads / 32) * c.pool_bytes;
     if (o.blocks) {
         c.blocks = o.blocks;
     } else {
@@ -298,10 +232,9 @@ int choose(uint32_t n, const mce_options &o, Config &c, size_t stack_cap = ~(siz
         if (per_sm < 1) return MCE_ENOMEM;
         c.blocks = (unsigned)(per_sm * sms);
     }
-    c.total_groups = c.blocks * (c.threads / 32) * (32 / G);
+    c.total_groups = c.blocks * (c.threads / 32);
     c.qcap = next_pow2(std::max<uint64_t>(1024, 4ull * c.total_groups + 256));
-    c.seed = tu.seed != 0;
-    if (c.seed) c.qcap = std::max<uint32_t>(c.qcap, next_pow2(2ull * n + 256));  // every root child queued at once
+    c.qcap = std::max<uint32_t>(c.qcap, next_pow2(2ull * n + 256));  // every root child queued at once
     if (o.queue_log2) c.qcap = std::max<uint32_t>(c.qcap, 1u << o.queue_log2);
     c.fs = (uint32_t)frame_words(c.wp, c.list);
     return MCE_OK;
@@ -341,16 +274,24 @@ int cuda_code(cudaError_t e) { return e == cudaSuccess ? MCE_OK : (e == cudaErro
 Tuning mce::default_tuning()
 {
     static const Tuning t = [] {
-        // block-ring checks every 8 and device-wide checks every 16 group
-        // iterations of a busy warp: with fetch-and-add ring tickets the
-        // checks are cheap enough that checking more often than every 16 /
-        // 64 iterations paid (G(1000, 0.3): 7.8 -> 7.4 ms; G(700, 0.3): 2.2
-        // -> 1.7 ms).  Served form: a request alone gets a block per 20,000
-        // expected maximal cliques, and requests expecting up to 10^6 share
+        Tuning d{};  // 0: thresholds by density
+        d.local_check = d.global_check = 1u;
+        d.refresh_ns = 2000u;
+        // Served form: a request alone gets a block per 20,000 expected
+        // maximal cliques, and requests expecting up to 10^6 share
         // micro-batches (on the served workload, 10,400 -> 11,300 requests/s
         // closed loop and p99 6.3 -> 3.9 ms at 0.7x that load, against one
         // block per 50,000 and micro-batches up to 10^5)
-        Tuning d{0u, 0u, 8u, 16u, 2000u, 20000u, 16384u, 32u, 16384u, 32u, 4u, 1u, 1u, 1u, 1u, 4u, 1000u, 1u};  // 0: thresholds by density
+        d.serve_cpb = 20000u;
+        d.serve_bcost = 1000u;
+        d.pop_tries = 16384u;
+        // (2 us -> 1 us took 1 to 3 % off searches of up to 2 ms, G(106, 0.7)
+        // 0.472 -> 0.456 ms, and nothing off longer ones)
+        d.idle_sleep_ns = 1024u;
+        d.t2_p = (uint32_t)kPoolMaxP;
+        d.t2_smem_words = 0u;
+        d.batch_split = 4u;
+        d.give_steps = 16u;
         if (const char *env = std::getenv("MCE_TUNE")) {
             const char *p = env;
             while (*p) {
@@ -365,17 +306,15 @@ Tuning mce::default_tuning()
                 else if (!std::strcmp(key, "refresh_ns")) d.refresh_ns = val;
                 else if (!std::strcmp(key, "serve_cpb") && val) d.serve_cpb = val;
                 else if (!std::strcmp(key, "pop_tries") && val) d.pop_tries = val;
-                else if (!std::strcmp(key, "share_tail") && val) d.share_tail = val;
                 else if (!std::strcmp(key, "idle_sleep_ns") && val) d.idle_sleep_ns = val;
-                else if (!std::strcmp(key, "t2_p")) d.t2_p = std::min(val, 32u);
-                else if (!std::strcmp(key, "t2_levels")) d.t2_levels = std::min(val, 31u);
-                else if (!std::strcmp(key, "t2_smem_rows")) d.t2_smem_rows = val;
-                else if (!std::strcmp(key, "seed")) d.seed = val;
-                else if (!std::strcmp(key, "serve_t2")) d.serve_t2 = val;
-                else if (!std::strcmp(key, "batch_wide")) d.batch_wide = val;
+                else if (!std::strcmp(key, "t2_p")) d.t2_p = std::min(val, (uint32_t)kPoolMaxP);
+                else if (!std::strcmp(key, "t2_smem_words")) d.t2_smem_words = val;
                 else if (!std::strcmp(key, "batch_split")) d.batch_split = val;
                 else if (!std::strcmp(key, "serve_bcost")) d.serve_bcost = val;
-                else if (!std::strcmp(key, "small_split")) d.small_split = val;
+                else if (!std::strcmp(key, "t2_task")) d.t2_task = val;
+                else if (!std::strcmp(key, "give_p")) d.give_p = val;
+                else if (!std::strcmp(key, "give_steps") && val) d.give_steps = pow2_ceil(val);
+                else if (!std::strcmp(key, "t2_cls")) d.t2_cls = val;
                 p += used;
                 if (*p == ',') ++p;
             }
@@ -410,13 +349,10 @@ SearchParams params(uint32_t n, const Config &c, const Layout &L, unsigned char 
     p.stack_levels = o.stack_levels ? std::min<uint32_t>(o.stack_levels, kStackDepth) : kStackDepth;
     p.split_min_p = o.split_min_p;  // 0: by density
     p.split_target = c.qcap / 2;
-    p.stack_smem_levels = c.stack_levels;
-    p.stack_offset = c.stack_offset;
     p.tune = default_tuning();
     // the breadth-first split of small graphs from 20 vertices pays in a
     // full-wave launch of one graph; a grid sized for one served request
     // (o.blocks) ran slower with it (10,800 -> 10,300 requests/s)
-    if (o.blocks) p.tune.small_split = 0u;
     p.trace = nullptr;
     p.trace_per_block = 0;
     if (g_trace && c.blocks) {
@@ -428,9 +364,9 @@ SearchParams params(uint32_t n, const Config &c, const Layout &L, unsigned char 
     p.part_k = 0;
     p.count_root = 1;
     p.t2_offset = c.t2_offset;
-    p.t2_levels = c.t2_levels;
+    p.pool_bytes = c.pool_bytes;
     p.t2_max_p = c.t2_max_p;
-    p.seed_children = c.seed ? 1u : 0u;
+    p.direct_offset = c.direct_offset;
     p.local_slots = c.local_slots;
     return p;
 }
@@ -1413,11 +1349,11 @@ struct Bucket {
     std::vector<uint32_t> graphs;
     std::vector<uint32_t> items;  // work items: graph | part << 16 | parts << 24
     uint32_t split_graphs = 0;
-    SearchImpl impl{nullptr, nullptr, nullptr, nullptr};
+    SearchImpl plain{nullptr, nullptr, nullptr, nullptr}, impl{nullptr, nullptr, nullptr, nullptr};
     LaunchShape shape{};
     uint32_t qcap = 0, fs = 0, groups = 0;
-    uint32_t stack_levels = 0, stack_offset = 0;
-    uint32_t t2_offset = 0, t2_levels = 0, t2_max_p = 0;  // lane tier (t2_max_p 0: off)
+    uint32_t t2_offset = 0, pool_bytes = 0, t2_max_p = 0, direct_offset = 0;  // warp tier (t2_max_p 0: off)
+    uint32_t cls = 1;  // its words per set, for all graphs of the bucket
     size_t qstride = 0, list_off = 0, region_off = 0, next_off = 0;
 };
 
@@ -1478,8 +1414,8 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
             k = (uint32_t)std::min(cap, std::ceil(cost[i] / target));
         }
         for (uint32_t j = 0; j < k; ++j) items.push_back({cost[i] / k, i | (j << 16) | (k << 24)});
+        if (!g->root) frames = std::max(frames, (g->n + k - 1) / k + 1);
         if (k >= 2) {
-            frames = std::max(frames, (g->n + k - 1) / k + 1);
             ++bk.split_graphs;
         }
     }
@@ -1493,35 +1429,25 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
 }
 
 // Launch choice of a batched graph without a tuned one: forced shapes as
-// given; otherwise 512 threads and subtrees of at most two words per lane
-// (one up to 128 vertices), the pattern the autotuner settled on for every
-// words class of the mixed 4,096-graph workload (more, narrower subtrees per
-// block than the plain form's shapes: a batched graph has no device-wide ring
-// to spread its work, so a block needs many subtrees of its own).
+// given, otherwise the most threads a block can have (a batched graph has no
+// device-wide ring to spread its work: one block with all of the SM's warps);
+// 256 for the outer loop's subproblems, most of which have fewer children than
+// that block has warps.
 TuneChoice default_choice(uint32_t n, const mce_options &o, bool wide)
 {
     TuneChoice t;
     pick_shape(n, o, t.G, t.K);
     t.threads = o.threads_per_block ? o.threads_per_block : 256u;
-    if (wide && default_tuning().batch_wide && !o.lanes_per_subtree && !o.words_per_lane) {
-        const uint32_t W = std::max<uint32_t>(1, (n + 31) / 32);
-        t.K = W <= 4 ? 1 : (W <= 64 ? 2 : 4);
-        t.G = 1;
-        while ((uint32_t)(t.G * t.K) < W) t.G <<= 1;
-        if (!o.threads_per_block) t.threads = kMaxThreads;
-    }
+    if (wide && !o.lanes_per_subtree && !o.words_per_lane && !o.threads_per_block)
+        t.threads = kLaunchThreads;
     t.split = o.split_min_p;
     return t;
 }
 
 // Plan and capture a batch with the launch choice of every words class
 // given in `choice` (classes not in it: the defaults).
-// subproblems: a batch of the outer loop's many small subproblems (Alg. 3):
-// untuned graphs take the plain form's shapes instead of default_choice's
-// wide ones, and no lane tier (on G(10000, p) with p = 0.01 / 0.03 the lane
-// tier made the batch 5.8 / 19.5 ms against 3.9 / 17.1 ms without it: a
-// subproblem's frames are small from the start, and the tier's region costs
-// the block its stack levels in shared memory).
+// subproblems: a batch of the outer loop's many small subproblems (Alg. 3),
+// searched by smaller blocks (see default_choice).
 int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, const mce_options &o,
                       const std::map<uint32_t, TuneChoice> &choice, mce_batch **out,
                       cudaStream_t stream = nullptr, bool subproblems = false);
@@ -1578,18 +1504,12 @@ void tune_batch(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, const mc
                 best = t;
             }
         };
-        for (int K : {1, 2, 4}) {
-            uint32_t G = 1;
-            while (G * (uint32_t)K < W) G <<= 1;
-            if (G > 32) continue;
-            for (unsigned threads : {128u, 256u, 512u}) {
-                TuneChoice t;
-                t.G = (int)G;
-                t.K = K;
-                t.threads = threads;
-                t.split = o.split_min_p;
-                consider(t);
-            }
+        for (unsigned threads : {128u, 256u, 512u}) {
+            TuneChoice t;
+            default_shape(32u * W, t.G, t.K);
+            t.threads = threads;
+            t.split = o.split_min_p;
+            consider(t);
         }
         if (best_ms < 0.0) continue;
         TuneChoice t = best;
@@ -1681,22 +1601,27 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         auto it = choice.find(wc);
         const TuneChoice t = it != choice.end() ? it->second : default_choice(g->n, o, !subproblems);
         const int G = t.G, K = t.K;
-        if ((uint32_t)(G * K) < W || !impl_for(G, K, false, (int)o.pivot_mode).run) { delete b; return MCE_EINVAL; }
+        const SearchImpl plain = impl_for(W, false, (int)o.pivot_mode);
+        if ((uint32_t)(G * K) < W || !shape_known(G, K) || !plain.run) { delete b; return MCE_EINVAL; }
+        const bool smem = W <= 32 && (uint32_t)(G * K) <= default_tuning().t2_smem_words;
         size_t bi = 0;
-        while (bi < buckets.size() && !(buckets[bi].G == G && buckets[bi].K == K && buckets[bi].threads == t.threads &&
-                                        buckets[bi].split == t.split))
+        while (bi < buckets.size() && !(buckets[bi].plain.run == plain.run && buckets[bi].smem == smem &&
+                                        buckets[bi].threads == t.threads && buckets[bi].split == t.split))
             ++bi;
         if (bi == buckets.size()) {
             Bucket nb;
-            nb.G = G;
-            nb.K = K;
+            nb.plain = plain;
             nb.threads = t.threads;
             nb.split = t.split;
             nb.wclass = wc;
             nb.tuned = t.tuned;
             nb.tuned_ms = t.ms_per_graph;
-            nb.smem = G * K <= 32;
+            nb.smem = smem;
             buckets.push_back(nb);
+        }
+        if (G * K > buckets[bi].G * buckets[bi].K) {  // the bucket reports its widest rows
+            buckets[bi].G = G;
+            buckets[bi].K = K;
         }
         buckets[bi].wclass = std::max(buckets[bi].wclass, wc);
         buckets[bi].graphs.push_back(i);
@@ -1728,37 +1653,36 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
     int rc = MCE_OK;
     for (Bucket &bk : buckets) {
         std::stable_sort(bk.graphs.begin(), bk.graphs.end(), [&](uint32_t a, uint32_t c2) { return cost[a] > cost[c2]; });
-        bk.impl = impl_for(bk.G, bk.K, bk.smem, (int)o.pivot_mode);
+        uint32_t words = 1;
         size_t base = 0;
-        for (uint32_t i : bk.graphs) base = std::max(base, search_smem(b->n[i], (uint32_t)(bk.G * bk.K), bk.smem));
-        const unsigned threads = bk.threads;
-        if (threads % 32 || threads > kMaxThreads) { rc = MCE_EINVAL; break; }
-        // the lane tier's region (groups of two or more lanes) when it fits,
-        // then at most 56 KB of stack per block, so that several blocks share
-        // an SM
-        const Tuning tu = default_tuning();
-        if (bk.G >= 2 && tu.t2_p != 0u && !subproblems) {
-            const size_t off = round_up(base, 16), t2b = (size_t)(threads / 32) * t2_warp_bytes(tu.t2_levels, o.pivot_mode != MCE_PIVOT_GREEDY);
-            if (off + t2b <= slimit) {
-                bk.t2_offset = (uint32_t)off;
-                bk.t2_levels = tu.t2_levels;
-                bk.t2_max_p = tu.t2_p;
-                base = off + t2b;
-            }
+        for (uint32_t i : bk.graphs) {
+            words = std::max(words, (b->n[i] + 31) / 32);
+            base = std::max(base, search_smem(b->n[i], wp_of[i], bk.smem));
         }
-        size_t smem = 0;
-        plan_stack_for((uint32_t)base, bk.G, bk.K, threads, std::min<size_t>(slimit, base + 56 * 1024),
-                       bk.stack_levels, bk.stack_offset, smem);
+        bk.impl = impl_for(words, bk.smem, (int)o.pivot_mode);
+        unsigned threads = bk.threads;
+        if (threads % 32 || threads > (o.threads_per_block ? kMaxThreads : kLaunchThreads)) { rc = MCE_EINVAL; break; }
+        // the whole-graph layout and the warp tier's regions; fewer warps where
+        // they do not fit
+        base = round_up(base, 16);
+        bk.direct_offset = (uint32_t)base;
+        bk.t2_offset = (uint32_t)(base + kDirectBytes);
+        while (threads > 32 && bk.t2_offset + (threads / 32) * kPoolBytesMin > slimit) threads -= 32;
+        bk.threads = threads;
+        bk.pool_bytes = plan_pool(bk.t2_offset, threads, std::max<size_t>((slimit + 2048) * threads / kLaunchThreads - 2048, bk.t2_offset));
+        bk.t2_max_p = default_tuning().t2_p;
+        bk.cls = std::min<uint32_t>(words, kPoolMaxP / 32);
+        const size_t smem = bk.t2_offset + (threads / 32) * bk.pool_bytes;
         int per_sm = 0;
         if (bk.impl.batch_occupancy((int)threads, smem, &per_sm) != cudaSuccess || per_sm < 1) { rc = MCE_EINVAL; break; }
         unsigned blocks = o.blocks ? o.blocks : (unsigned)(per_sm * sms);
         const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, blocks, default_tuning().batch_split);
         blocks = std::min<unsigned>(blocks, (unsigned)bk.items.size());
         bk.shape = LaunchShape{blocks, threads, smem, bk.smem};
-        bk.groups = threads / 32 * (32 / bk.G);
+        bk.groups = threads / 32;
         bk.qcap = next_pow2(std::max<uint64_t>(256, 4ull * bk.groups + 64 + part_frames));
         if (o.queue_log2) bk.qcap = std::max<uint32_t>(bk.qcap, 1u << o.queue_log2);
-        bk.fs = (uint32_t)frame_words((uint32_t)(bk.G * bk.K));
+        bk.fs = (uint32_t)frame_words((uint32_t)(bk.G * bk.K));  // the widest rows' frames
         bk.qstride = batch_region_bytes(bk.qcap, bk.fs);
         bk.list_off = take(bk.items.size() * 4, 16);
         bk.next_off = take(4, 128);
@@ -1854,13 +1778,12 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
             bp.groups_per_block = bk.groups;
             bp.split_min_p = bk.split;
             bp.split_target = bk.qcap / 2;
-            bp.stack_smem_levels = bk.stack_levels;
-            bp.stack_offset = bk.stack_offset;
             bp.tune = default_tuning();
-            bp.tune.small_split = 0u;  // the batched form ran 6 % slower with it
             bp.t2_offset = bk.t2_offset;
-            bp.t2_levels = bk.t2_levels;
+            bp.pool_bytes = bk.pool_bytes;
+            bp.direct_offset = bk.direct_offset;
             bp.t2_max_p = bk.t2_max_p;
+            bp.cls = bk.cls;
             ce = cudaStreamWaitEvent(b->side[i], b->events[0], 0);
             if (ce == cudaSuccess) ce = bk.impl.run_batch(bp, bk.shape, b->side[i]);
             if (ce == cudaSuccess) ce = cudaEventRecord(b->events[i + 1], b->side[i]);
@@ -2099,7 +2022,6 @@ extern "C" int mce_enumerate_batch(mce_ctx *ctx, mce_graph *const *graphs, uint3
 namespace {
 
 constexpr int kServeSlots = 128;
-constexpr size_t kServeStackBytes = 56 * 1024;  // shared-memory stack per block
 // Micro-batches: while at least kBatchMin requests that can share a launch
 // wait, up to kBatchMax of them (each expecting at most serve_bcost
 // thousand maximal cliques) run as one batched launch on one stream slot.
@@ -2441,7 +2363,7 @@ extern "C" int mce_submit(mce_ctx *ctx, mce_graph *g, const mce_options *opts, m
     r->g = g;
     r->o = o;
     r->batchable = batchable;
-    int rc = g->n > MCE_NMAX ? MCE_EINVAL : choose(g->n, o, r->c, kServeStackBytes);
+    int rc = g->n > MCE_NMAX ? MCE_EINVAL : choose(g->n, o, r->c);
     if (rc) { delete r; return rc; }
     r->L = layout(g->n, r->c);
     r->scratch_bytes = r->L.total;

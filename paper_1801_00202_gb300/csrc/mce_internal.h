@@ -28,7 +28,7 @@ struct Ctl {
     unsigned head;     unsigned pad0[31];  // global queue consumer ticket
     unsigned tail;     unsigned pad1[31];  // global queue producer ticket
     unsigned pending;  unsigned pad2[31];  // frames in the global ring + active blocks
-    unsigned starving; unsigned pad3[31];  // blocks with idle groups and no local frame
+    unsigned starving; unsigned pad3[31];  // warps without a frame; pad3[0]: the degree sum
     unsigned abort;    unsigned pad4[31];  // set on error: every warp stops
 };
 
@@ -37,13 +37,12 @@ struct Ctl {
 // slots = kLocalSlots, or kLocalSlotsSmall where halving the ring buys a
 // warp of a plain search block (the planner decides).
 constexpr int kLocalSlots = 32;
-constexpr int kLocalSlotsSmall = 16;
 struct LocalHdr {
     unsigned head, tail;  // ring tickets
-    unsigned idle;        // groups of this block without a frame
-    unsigned bwork;       // busy groups + frames in the ring; the block holds
+    unsigned idle;        // warps of this block without a frame
+    unsigned bwork;       // busy warps + frames in the ring; the block holds
                           // one unit of Ctl::pending while this is non-zero
-    unsigned starving;    // this block is counted in Ctl::starving
+    unsigned spare0;      // unused
     unsigned poller;      // a warp of this block is polling the global ring
     unsigned done;        // the search is over (1) or aborted (2)
     unsigned refreshing;  // a warp is refreshing the cached global state
@@ -52,7 +51,14 @@ struct LocalHdr {
     unsigned spare;       // unused (keeps the stamp 8-byte aligned)
     unsigned long long stamp;
     unsigned trace_n;     // timeline records written by this block
-    unsigned t2_busy;     // lanes of the block holding a lane-tier subproblem
+    unsigned give_p;      // warp tier: smallest |P| of a frame that is given away
+    // the device-wide ring and the frame shape, for frames given away by the
+    // warp tier
+    Ctl *ctl;
+    unsigned *gseq;
+    uint32_t *gframes;
+    unsigned qcap, fs, margin, wp, slots, n;
+    unsigned give_mask, total;
     // work-distribution diagnostics of the block (rare events, shared-memory
     // atomics; added to the result array once the block is done)
     unsigned long long diag[8];
@@ -94,36 +100,38 @@ struct Tuning {
     uint32_t refresh_ns;    // age of a block's cached view of the global ring
     uint32_t serve_cpb;     // served form: expected maximal cliques per block
     uint32_t pop_tries;     // ticket attempts of one take from the device-wide ring
-    uint32_t share_tail;    // smallest |P| shared once half the groups/blocks are idle
     uint32_t idle_sleep_ns; // longest back-off of an idle warp that is not polling
-    uint32_t t2_p;          // lane tier: largest |P| of a subproblem handed to one lane (0: off)
-    uint32_t t2_levels;     // lane tier: explicit-stack levels per lane in shared memory
-    uint32_t t2_smem_rows;  // lane tier on: keep the rows in shared memory (fewer warps) when 1
-    uint32_t seed;          // start from every root child as its own queued frame (1) or the root (0)
-    uint32_t serve_t2;      // served requests use the lane tier too (its region beside the capped stack)
-    uint32_t batch_wide;    // batched form by default: 512 threads, at most two words per lane (1), or the plain shapes (0)
+    uint32_t t2_p;          // warp tier: largest |P| of a subproblem (0: off, at most kPoolMaxP)
+    uint32_t t2_smem_words; // warp tier on: rows of up to this many words are kept in shared memory
     uint32_t batch_split;   // batched form: parts of about 1/(blocks * batch_split) of a bucket's cost (0: no split)
     uint32_t serve_bcost;   // served form: largest expected maximal cliques (thousands) of a micro-batched request
-    uint32_t small_split;   // small graphs of density <= 0.75 split breadth first from 20 vertices (1) or by density (0)
+    uint32_t t2_task;       // largest |P u X| of a subproblem (0: by density and size)
+    uint32_t t2_cls;        // words per set of a subproblem (0: by density and size)
+    uint32_t give_p;        // smallest |P| a warp tier gives away (0: by density)
+    uint32_t give_steps;    // warp tier: steps between looks for idle warps (a power of two)
 };
 
-// The lane tier (second search tier): a frame whose P u X has at most 32
-// vertices is relabelled 0..u-1 in order and searched by one lane with 32-bit
-// sets.  Per warp in shared memory: the 32 lanes' local adjacency rows
-// A[row][lane] (u32), the positions of their local vertices pos[v][lane]
-// (u16), and t2_levels explicit-stack levels of six words per lane
-// [level][field][lane] (P, X, L, |R|, S low, S high).
-// After them, for the pivot rules that score candidates (GreedyBBTX/NX,
-// TomitaBB), 512 bytes of scratch for the group search's parallel pivot
-// scoring (each lane's words of P'); GreedyBB needs none, so its blocks keep
-// that room (on 1,000 vertices with rows in shared memory: a quarter more
-// warps).
-constexpr int kT2Fields = 6;
-constexpr int kPivotScratchWords = 128;
-__host__ __device__ inline size_t t2_warp_bytes(uint32_t levels, bool scoring)
-{
-    return 32 * 32 * 4 + 32 * 32 * 2 + (size_t)levels * kT2Fields * 32 * 4 + (scoring ? kPivotScratchWords * 4 : 0);
-}
+// The warp tier (second search tier): a frame whose P u X has at most 128
+// vertices is relabelled 0..u-1 in order and searched by its whole warp, each
+// lane expanding a node per step.  Per warp in shared memory: the local
+// adjacency rows (u rows of ceil(u/32) words; several small subproblems side
+// by side), the hash terms of the local vertices, a buffer of leaves, and the
+// stack of frames the 32 lanes share.
+constexpr int kPoolLeafBytes = 63 * 12 + 12;  // 31 leaves waiting and 32 new ones, three words each
+constexpr int kPoolFixedBytes = 5456;   // the most that precedes a stack in the region
+constexpr int kPoolMaxP = 128;          // largest |P| of a subproblem
+// A warp's region: at least 64 frames of any set size (a stack that is paged
+// out at fewer than 32 free frames must hold 32 to page), at most about 256 of
+// four words.
+constexpr uint32_t kPoolBytesMin = 7248, kPoolBytesMax = 15360;
+
+// Graphs of at most 128 vertices: the whole graph in the warp tier's layout,
+// once per block (rows, hash terms, positions).
+constexpr int kDirectRows = 512, kDirectVerts = 128;
+constexpr uint32_t kDirectBytes = kDirectRows * 4 + kDirectVerts * 10;
+
+// Most threads of a search block (the register bound of the kernels).
+constexpr unsigned kLaunchThreads = 768u;
 
 struct SearchParams {
     uint32_t n;             // vertices
@@ -142,8 +150,6 @@ struct SearchParams {
     uint32_t stack_levels;  // <= kStackDepth
     uint32_t split_min_p;   // publish new subtrees with |P| >= this ...
     uint32_t split_target;  // ... while the global ring holds fewer frames
-    uint32_t stack_smem_levels;  // explicit-stack levels kept in shared memory
-    uint32_t stack_offset;       // byte offset of the stack region in shared memory
     unsigned long long *trace;   // optional timeline (2 words per record)
     uint32_t trace_per_block;    // records per block
     Tuning tune;
@@ -155,13 +161,10 @@ struct SearchParams {
     const uint32_t *part;
     uint32_t part_k;
     uint32_t count_root;
-    // lane tier: byte offset of its shared-memory region (t2_warp_bytes per
-    // warp), stack levels kept there, and the largest |P| handed to a lane
-    // (0: the tier is off)
-    uint32_t t2_offset, t2_levels, t2_max_p;
-    // start from the root's children, each its own queued frame, instead of
-    // the root frame (the root is still counted once)
-    uint32_t seed_children;
+    // warp tier: byte offset of its shared memory, the bytes of a warp's region
+    // (a multiple of 16) and the largest |P| of a subproblem (0: the tier is off)
+    uint32_t t2_offset, pool_bytes, t2_max_p;
+    uint32_t direct_offset;  // byte offset of the whole-graph layout (n <= 128)
     uint32_t local_slots;   // slots of the block ring (kLocalSlots or kLocalSlotsSmall)
 };
 
@@ -219,9 +222,9 @@ struct BatchParams {
     uint64_t timeout_ns;
     uint32_t pivot_mode, stack_levels, groups_per_block;
     uint32_t split_min_p, split_target;
-    uint32_t stack_smem_levels, stack_offset;
     Tuning tune;
-    uint32_t t2_offset, t2_levels, t2_max_p;  // lane tier (as in SearchParams)
+    uint32_t t2_offset, pool_bytes, t2_max_p, direct_offset;  // warp tier (as in SearchParams)
+    uint32_t cls;            // words per set of the warp tier, for all graphs of the bucket
 };
 
 // Per-block queue region of the batched search: [Ctl | seq | frames]
@@ -249,43 +252,13 @@ struct SearchImpl {
     cudaError_t (*run_batch)(const BatchParams &, const LaunchShape &, cudaStream_t);
     cudaError_t (*batch_occupancy)(int threads, size_t smem, int *blocks_per_sm);
 };
-SearchImpl search_impl_1_1(bool smem, int pivot);
-SearchImpl search_impl_1_2(bool smem, int pivot);
-SearchImpl search_impl_1_4(bool smem, int pivot);
-SearchImpl search_impl_2_1(bool smem, int pivot);
-SearchImpl search_impl_2_2(bool smem, int pivot);
-SearchImpl search_impl_2_4(bool smem, int pivot);
-SearchImpl search_impl_4_1(bool smem, int pivot);
-SearchImpl search_impl_4_2(bool smem, int pivot);
-SearchImpl search_impl_4_4(bool smem, int pivot);
-SearchImpl search_impl_8_1(bool smem, int pivot);
-SearchImpl search_impl_8_2(bool smem, int pivot);
-SearchImpl search_impl_8_4(bool smem, int pivot);
-SearchImpl search_impl_16_1(bool smem, int pivot);
-SearchImpl search_impl_16_2(bool smem, int pivot);
-SearchImpl search_impl_16_4(bool smem, int pivot);
-SearchImpl search_impl_32_1(bool smem, int pivot);
-SearchImpl search_impl_32_2(bool smem, int pivot);
-SearchImpl search_impl_32_4(bool smem, int pivot);
+SearchImpl search_impl_1(bool smem, int pivot);
+SearchImpl search_impl_2(bool smem, int pivot);
+SearchImpl search_impl_4(bool smem, int pivot);
 // Listing variants (run/occupancy only; no batched form).
-SearchImpl search_list_impl_1_1(bool smem, int pivot);
-SearchImpl search_list_impl_1_2(bool smem, int pivot);
-SearchImpl search_list_impl_1_4(bool smem, int pivot);
-SearchImpl search_list_impl_2_1(bool smem, int pivot);
-SearchImpl search_list_impl_2_2(bool smem, int pivot);
-SearchImpl search_list_impl_2_4(bool smem, int pivot);
-SearchImpl search_list_impl_4_1(bool smem, int pivot);
-SearchImpl search_list_impl_4_2(bool smem, int pivot);
-SearchImpl search_list_impl_4_4(bool smem, int pivot);
-SearchImpl search_list_impl_8_1(bool smem, int pivot);
-SearchImpl search_list_impl_8_2(bool smem, int pivot);
-SearchImpl search_list_impl_8_4(bool smem, int pivot);
-SearchImpl search_list_impl_16_1(bool smem, int pivot);
-SearchImpl search_list_impl_16_2(bool smem, int pivot);
-SearchImpl search_list_impl_16_4(bool smem, int pivot);
-SearchImpl search_list_impl_32_1(bool smem, int pivot);
-SearchImpl search_list_impl_32_2(bool smem, int pivot);
-SearchImpl search_list_impl_32_4(bool smem, int pivot);
+SearchImpl search_list_impl_1(bool smem, int pivot);
+SearchImpl search_list_impl_2(bool smem, int pivot);
+SearchImpl search_list_impl_4(bool smem, int pivot);
 
 
 // The root's children as independent subtrees (split.cu).  The root's
@@ -354,31 +327,19 @@ cudaError_t list_build(const ListJob &j, cudaStream_t s);
 Tuning default_tuning();
 
 // Shared-memory layout of the search kernels:
-//   [rows (when staged), padded to 16 B][hv: n x u64][hk: (n + 1) x u64]
-//   [hist: (n + 1) x u32, padded to 16 B][local frame ring][stack]
+//   [rows (when staged), padded to 16 B][hist: (n + 1) x u32, padded to 16 B]
+//   [local frame ring][whole-graph layout (n <= 128)][warp regions]
 __host__ __device__ inline size_t smem_rows_bytes(uint32_t n, uint32_t wp, bool rows_in_smem)
 {
     return rows_in_smem ? ((size_t)n * wp * 4 + 15) / 16 * 16 : 0;
 }
 __host__ __device__ inline size_t smem_local_offset(uint32_t n, uint32_t wp, bool rows_in_smem)
 {
-    return smem_rows_bytes(n, wp, rows_in_smem) + (size_t)n * 8 +
-           (((size_t)n + 1) * 4 + 15) / 16 * 16;
+    return smem_rows_bytes(n, wp, rows_in_smem) + (((size_t)n + 1) * 4 + 15) / 16 * 16;
 }
 __host__ __device__ inline size_t search_smem_bytes(uint32_t n, uint32_t wp, bool rows_in_smem, bool list = false,
                                                    uint32_t slots = kLocalSlots)
 {
     return smem_local_offset(n, wp, rows_in_smem) + local_queue_bytes(wp, list, slots);
 }
-// Explicit-stack words per lane per level for groups of `lanes` lanes with
-// `words` words per lane: P, X and the level's scalars (one word when the
-// group has four or more lanes to spread them over, else four).
-__host__ __device__ inline uint32_t stack_level_words(int lanes, int words)
-{
-    return 2u * (uint32_t)words + (lanes >= 4 ? 1u : 4u);
-}
-// Most levels worth keeping in shared memory (deeper ones use local memory).
-constexpr int kStackSmemMax = 24;
-
-
 }  // namespace mce

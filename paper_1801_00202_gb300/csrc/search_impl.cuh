@@ -1,35 +1,29 @@
 // Bit-parallel Bron-Kerbosch search (Alg. 4, BKPivotOrdered with
 // ChoosePivotOrdered) as a persistent, work-stealing CUDA kernel for sm_103a.
 //
-// Mapping (Section 4.1 describes the CPU bitset encoding this replaces):
-//  * A *group* of G lanes of one warp owns one search subtree.  Lane l of the
-//    group holds words [l*K, l*K + K) of every set, so a set of n vertices
-//    takes WP = G*K 32-bit words spread over the group.  32/G groups share a
-//    warp and advance in lock step: every warp-wide collective (ballot,
-//    shuffle) is executed by all 32 lanes, and group-specific decisions are
-//    data predicates.
+// Two tiers (Section 4.1 describes the CPU bitset encoding this replaces):
+//  * The top of the search tree: a warp owns one frame (P, X, pivot, end, |R|,
+//    S(R)), which stands for "expand the children v in L = P & ~N(pivot) &
+//    [0, end) in increasing position".  Lane l holds words [l*K, l*K + K) of
+//    every set; the current frame lives in registers, its ancestors on an
+//    explicit stack in local memory (no recursion).  A frame is pushed only
+//    while it has children left, so single-child chains (e.g. a complete
+//    graph) do not grow the stack.
+//  * The warp tier, where nearly all nodes are: subtrees of at most 128
+//    vertices, compressed to small sets and searched a child per lane (see
+//    "The warp tier" below).
 //  * The renumbered adjacency (Section 4.2) is staged in shared memory by a
-//    1-D bulk-copy (TMA) when it fits, else read from L2 through the
-//    read-only path with 64/128-bit loads.
-//  * A frame (P, X, pivot, end, |R|, S(R)) stands for "expand the children
-//    v in L = P & ~N(pivot) & [0, end) in increasing position": the current
-//    frame lives in registers, its ancestors on a per-group explicit stack in
-//    local memory (no recursion).  A frame is pushed only while it has
-//    children left, so single-child chains (e.g. a complete graph) do not
-//    grow the stack.
-//  * Work moves at two levels.  Idle groups take frames from their block's
-//    ring in shared memory, which busy groups of the block refill by giving
-//    away the front half of their shallowest branching set; blocks whose
-//    groups are idle with an empty ring count as starving, one idle warp per
-//    block polls the global ring (a bounded MPMC ring in global memory whose
-//    tickets are taken by fetch-and-add at both ends, never by a contended
-//    compare-and-swap), and busy groups feed that ring while starving blocks
-//    outnumber its frames.
+//    1-D bulk-copy (TMA) when it is small, else read from L2.
+//  * Work moves at two levels.  Idle warps take frames from their block's
+//    ring in shared memory or from the device-wide ring (a bounded MPMC ring
+//    in global memory whose tickets are taken by fetch-and-add at both ends);
+//    busy warps refill the block's ring while it has more idle warps than
+//    queued frames, and the device-wide ring while the GPU has.
 //    Cutting a branching set L into a front part L1 (given) and the rest as
 //    (P, X, end = first kept element) and (P \ L1, X u L1, end) reproduces
 //    exactly the sequential P/X updates of Alg. 4, so node counts do not
 //    depend on how the work was split.
-//  * Leaves update per-group register counters; sizes go to a shared-memory
+//  * Leaves update per-lane register counters; sizes go to a shared-memory
 //    histogram; everything is integer arithmetic modulo 2^64, so the
 //    reduction order does not matter and results are bit-exact.
 //
@@ -68,52 +62,93 @@ __constant__ unsigned short kSplitByDensity[39] = {1363, 907, 651, 515, 433, 376
                                                    65,   61,  58,  55,  52,  50,  48,  46,  45,  44,  43,  45,  51};
 
 struct Thresholds {
-    unsigned share_local, share_global, split;
+    unsigned share;        // smallest |P| of a frame given to the block's idle warps
+    unsigned share_far;    // smallest |P| of a frame given to the device-wide ring
+    unsigned split;        // smallest |P| of a new subtree that is published breadth-first
+    unsigned task;         // warp tier: largest |P| of a subproblem
+    unsigned cls;          // warp tier: words per set (P u X of at most 32 cls vertices)
 };
 
-// Thresholds for a block's graph from the density of its rows; non-zero
-// caller values win.  Whole block (barriers inside); every thread gets the
-// same values.
-__device__ __forceinline__ Thresholds density_thresholds(const uint32_t *rows, uint32_t n, uint32_t wp,
-                                                         unsigned fixed_local, unsigned fixed_global,
-                                                         unsigned fixed_split, unsigned *scratch_u32,
-                                                         bool small_split)
+// Thresholds from the graph's edge density (deg_sum = twice the edges);
+// non-zero caller values win.  batch_cls != 0: one of a batch's graphs, which
+// share sets of that size.
+__device__ __forceinline__ Thresholds density_thresholds(unsigned deg_sum, uint32_t n, const Tuning &tune,
+                                                         unsigned fixed_split, unsigned batch_cls = 0u)
 {
-    if (threadIdx.x == 0) *scratch_u32 = 0u;
-    __syncthreads();
-    unsigned mine = 0;
-    for (uint32_t i = threadIdx.x; i < n * wp; i += blockDim.x) mine += __popc(rows[i]);
-    atomicAdd(scratch_u32, mine);
-    __syncthreads();
-    const unsigned deg_sum = *scratch_u32;
-    __syncthreads();
-    Thresholds t{0xffffffffu, 0xffffffffu, 0xffffffffu};
-    if (n >= 2) {
-        const double pd = (double)deg_sum / ((double)n * (double)(n - 1));
-        int i = (int)(pd * 40.0 + 0.5);
+    Thresholds t{0xffffffffu, 0xffffffffu, 0xffffffffu, 128u, max(batch_cls, 1u)};
+    if (n >= 2u) {
+        const float pd = (float)deg_sum / ((float)n * (float)(n - 1u));
+        int i = (int)(pd * 40.0f + 0.5f);
         i = i < 1 ? 1 : (i > 39 ? 39 : i);
-        // The tables assume random graphs; a structured graph (Moon-Moser:
-        // every branching set has three vertices) keeps big subtrees at
-        // much smaller |P|, so a candidate set holding a good share of the
-        // graph also counts as big.
-        t.share_local = min((unsigned)kShareLocalByDensity[i - 1], max(16u, n / 8u));
-        t.share_global = min((unsigned)kShareGlobalByDensity[i - 1], max(20u, n / 4u));
+        t.share = kShareLocalByDensity[i - 1];
+        t.share_far = t.share;
         // dense structured graphs (Moon-Moser: every child keeps all but three
         // vertices) would never reach the density's split size; cap it at
-        // half of n (Moon-Moser 45: 1.37 -> 0.90 ms against two thirds).
-        // With small_split (full-wave launches of one graph), small graphs
-        // of density up to 0.75 split from 20 vertices: their whole tree is
-        // too small for the density's split size, and only frames that move
-        // keep the GPU busy (measured, whole path: G(100, 0.5) 0.28 -> 0.21
-        // ms, G(100, 0.7) 0.95 -> 0.50, G(128, 0.5) 0.36 -> 0.24, G(200,
-        // 0.5) 0.83 -> 0.54, G(256, 0.4) 0.72 -> 0.51; G(100, 0.8) would
-        // lose: 1.27 -> 2.2 ms)
+        // half of n
         t.split = min((unsigned)kSplitByDensity[i - 1], max(20u, n / 2u));
-        if (small_split && n <= 256u && i <= 30) t.split = min(t.split, 20u);
+        // Largest subproblem of the warp tier: about a 4,096th of the whole
+        // search (log2 of its expected maximal cliques continued from the
+        // table on a log-log line), so that every warp gets some before
+        // frames have to be given away; the whole graph when that is small
+        // (fewer than 50,000: handing out the parts takes longer than it
+        // saves).  In dense graphs, where a subtree can hold far more cliques
+        // than a random graph's (Moon-Moser), a third of the vertices.
+        // Measured with limits of 24 / 32 / 48 / 64 / 128 vertices, ms:
+        // G(106, 0.71) 0.40 / 0.43 / 0.49 / - / 0.57, G(100, 0.8) 1.5 / 1.1 /
+        // 1.5 / 1.8 / 1.4, G(300, 0.5) 3.7 / 2.5 / 1.5 / 1.3 / 1.4, G(100, 0.5)
+        // 0.20 / 0.18 / 0.19 / 0.16 / 0.16; Moon-Moser 45 with 16 / 20 / 24 /
+        // 32: 0.69 / 0.63 / 0.77 / 1.06.
+        const float k2 = (float)kShareGlobalByDensity[i - 1], k3 = (float)kSplitByDensity[i - 1];
+        const float size = 14.0f + 3.0f * __logf((float)n / k3) / __logf(k3 / k2);
+        if (i >= 30) t.task = min((unsigned)kShareGlobalByDensity[i - 1], max(20u, n / 3u));
+        else if (n > 128u) t.task = min((unsigned)kSplitByDensity[i - 1], max(48u, 3u * n / 10u));
+        else if (size >= 15.6f || (size >= 12.5f && i >= 24))
+            t.task = size < 21.5f ? kShareLocalByDensity[i - 1]
+                                  : (size < 24.5f ? kShareGlobalByDensity[i - 1] : kSplitByDensity[i - 1]);
+        // Set size of the warp tier: k levels below the root P u X has about
+        // n p^k vertices.  The first level of at most 112 (128 in a long
+        // search, which has frames enough beside the larger half) gets the tier, or
+        // the one below where the children of the root would hold more than
+        // about 600 cliques each (then they are too few and too uneven).
+        // Room for all of the level's frames: three standard deviations for
+        // the children of the root, two below; none in dense graphs, where
+        // one level further down still holds enough work per frame.  One
+        // size for the whole search keeps one instance of the tier's code in
+        // the instruction caches: with all four sizes in use the SM's
+        // instruction fetches were what bounded the search.
+        float sz = (float)n, pk = 1.0f;
+        const float pf = pd < 0.95f ? pd : 0.95f;
+        int level = 0;
+        const float most = size < 22.5f ? 112.0f : 128.0f;
+        while (sz > most || (level == 1 && size - __log2f((float)n) > 9.3f)) {
+            sz *= pf;
+            pk *= pf;
+            ++level;
+        }
+        if (level <= 1) sz += 3.0f * sqrtf(sz * (1.0f - pk));
+        else if (pf < 0.48f) sz += 2.0f * sqrtf(sz * (1.0f - pk));
+        t.cls = n <= 128u ? (n + 31u) / 32u : (unsigned)((sz + 32.0f) * (1.0f / 32.0f));
+        t.cls = min(max(t.cls, 1u), 4u);
+        // A batch has work for every warp without cutting subtrees small, and
+        // one set size for all of its graphs keeps to one instance of the
+        // code: 512 graphs of 32 to 512 vertices took 17.7 ms with the limits
+        // of a graph searched alone, 13.0 with 128 vertices as the limit and
+        // four words above 128 vertices, 12.5 with four words throughout.
+        if (batch_cls) {
+            t.cls = batch_cls;
+            if (i < 30) t.task = 128u;
+        }
     }
-    if (fixed_local) t.share_local = fixed_local;
-    if (fixed_global) t.share_global = fixed_global;
-    if (fixed_split) t.split = fixed_split;
+    if (tune.share_local) t.share = tune.share_local;
+    if (tune.share_global) t.share_far = tune.share_global;
+    if (fixed_split) {
+        // (a caller's split size is honoured: larger subtrees are published,
+        // not searched by the warp tier)
+        t.split = fixed_split;
+        t.task = min(t.task, fixed_split - 1u);
+    }
+    if (tune.t2_task) t.task = min(t.task, tune.t2_task);
+    if (tune.t2_cls && n > 128u) t.cls = min(tune.t2_cls, 4u);
     return t;
 }
 
@@ -179,6 +214,7 @@ __device__ __forceinline__ bool q_reserve_push(Ctl *ctl, unsigned *seq, unsigned
     const unsigned hd = ld_relaxed(&ctl->head), tl = ld_relaxed(&ctl->tail);
     if ((int)(tl - hd) >= (int)(mask + 1u) - (int)margin) return false;
     const unsigned tk = atomicAdd(&ctl->tail, 1u);
+#pragma unroll 1
     for (unsigned t = 0; ld_acquire(&seq[tk & mask]) != tk; ++t) {
         if (t >= (kCasTries << 8) || ld_relaxed(&ctl->abort)) return false;
         __nanosleep(32);
@@ -194,6 +230,7 @@ __device__ __forceinline__ bool q_reserve_pop(Ctl *ctl, unsigned *seq, unsigned 
                                               unsigned long long *fails, unsigned tries = kCasTries)
 {
     unsigned pos = ld_relaxed(&ctl->head);
+#pragma unroll 1
     for (unsigned t = 0; t < tries; ++t) {
         unsigned s = ld_acquire(&seq[pos & mask]);
         int dif = (int)(s - (pos + 1));
@@ -212,14 +249,13 @@ __device__ __forceinline__ bool q_reserve_pop(Ctl *ctl, unsigned *seq, unsigned 
 }
 
 // Room kept free in a frame ring for producers that reserve at once: every
-// group of the launch on the device-wide ring (the plain form sizes the ring
-// at four frames per group and more), the block's groups on a block-private
+// warp of the launch on the device-wide ring (the plain form sizes the ring
+// at four frames per warp and more), the block's warps on a block-private
 // ring (batched form).
-template <int G>
 __device__ __forceinline__ unsigned push_margin(const SearchParams &prm)
 {
-    const unsigned block_groups = (blockDim.x >> 5) * (32u / G);
-    return (prm.total_groups > block_groups ? prm.total_groups : block_groups) + 32u;
+    const unsigned block_warps = blockDim.x >> 5;
+    return (prm.total_groups > block_warps ? prm.total_groups : block_warps) + 32u;
 }
 
 // Claim up to `want` consecutive consumer tickets of the device-wide ring
@@ -243,154 +279,61 @@ __device__ __forceinline__ unsigned q_claim(Ctl *ctl, unsigned want, unsigned &f
 }
 
 // ---------------------------------------------------------------------------
-// Group-wide set primitives.  All collectives use the full warp mask and must
-// be reached by all 32 lanes: call them only as standalone statements in
-// warp-uniform code, never behind a short-circuit && / || or a ?: whose
-// condition differs between lanes.
+// Warp-wide set primitives: lane l holds words [l*K, l*K + K) of a set.  All
+// are reached by all 32 lanes in warp-uniform control flow.
 
-template <int G, int K>
-struct Grp {
-    static constexpr int WP = G * K;
-    unsigned lane, gl, gbase, gmask;
-
-    __device__ __forceinline__ void init()
-    {
-        lane = threadIdx.x & 31u;
-        gl = lane & (unsigned)(G - 1);
-        gbase = lane - gl;
-        gmask = (G == 32) ? FULL : (((1u << G) - 1u) << gbase);
-    }
-    __device__ __forceinline__ bool leader() const { return gl == 0; }
-
-    __device__ __forceinline__ bool anyp(bool p) const
-    {
-        if (G == 1) return p;
-        return (__ballot_sync(FULL, p) & gmask) != 0u;
-    }
-    __device__ __forceinline__ bool any(const uint32_t (&s)[K]) const
-    {
-        uint32_t o = 0;
+// Position of the lowest set bit (= the vertex first in the order), or -1.
+template <int K>
+__device__ __forceinline__ int set_first(const uint32_t (&s)[K], unsigned lane)
+{
+    int loc = -1;
 #pragma unroll
-        for (int k = 0; k < K; ++k) o |= s[k];
-        return anyp(o != 0u);
-    }
-    // Position of the lowest set bit of the group's set (= the vertex first
-    // in the order), or -1 if the set is empty.  A whole-warp group takes
-    // one min-reduction; narrower groups a ballot and a shuffle.
-    __device__ __forceinline__ int first(const uint32_t (&s)[K]) const
-    {
-        int loc = -1;
+    for (int k = K - 1; k >= 0; --k)
+        if (s[k]) loc = (int)((lane * K + k) * 32u) + __ffs(s[k]) - 1;
+    return (int)__reduce_min_sync(FULL, (unsigned)loc);
+}
+template <int K>
+__device__ __forceinline__ uint32_t set_or(const uint32_t (&s)[K])
+{
+    uint32_t o = s[0];
 #pragma unroll
-        for (int k = K - 1; k >= 0; --k)
-            if (s[k]) loc = (int)((gl * K + k) * 32u) + __ffs(s[k]) - 1;
-        if (G == 1) return loc;
-        if (G == 32) return (int)__reduce_min_sync(FULL, (unsigned)loc);
-        unsigned b = __ballot_sync(FULL, loc >= 0) & gmask;
-        int src = b ? (__ffs(b) - 1) : (int)lane;
-        int r = __shfl_sync(FULL, loc, src);
-        return b ? r : -1;
-    }
-    // Emptiness of sets a and b, and the first element of a when a is
-    // non-empty, else of b (-1 when both are empty).
-    __device__ __forceinline__ int first_either(const uint32_t (&a)[K], const uint32_t (&b)[K], bool &na,
-                                                bool &nb) const
-    {
-        uint32_t oa = 0, ob = 0;
+    for (int k = 1; k < K; ++k) o |= s[k];
+    return o;
+}
+template <int K>
+__device__ __forceinline__ unsigned set_count(const uint32_t (&s)[K])
+{
+    unsigned c = 0;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            oa |= a[k];
-            ob |= b[k];
-        }
-        unsigned ba = 0u, bb = 0u;
-        if (G == 1) {
-            na = oa != 0u;
-            nb = ob != 0u;
-        } else {
-            ba = __ballot_sync(FULL, oa != 0u) & gmask;
-            bb = __ballot_sync(FULL, ob != 0u) & gmask;
-            na = ba != 0u;
-            nb = bb != 0u;
-        }
-        int loc = -1;
+    for (int k = 0; k < K; ++k) c += (unsigned)__popc(s[k]);
+    return c;
+}
+// Bits [0, end) of this lane's k-th word.
+template <int K>
+__device__ __forceinline__ uint32_t set_below(int k, unsigned end, unsigned lane)
+{
+    const unsigned base = (lane * K + k) * 32u;
+    if (end >= base + 32u) return FULL;
+    if (end <= base) return 0u;
+    return (1u << (end - base)) - 1u;
+}
+// The bit of vertex v in this lane's k-th word.
+template <int K>
+__device__ __forceinline__ uint32_t set_bit(int k, unsigned v, unsigned lane)
+{
+    return (v >> 5) == lane * K + k ? 1u << (v & 31u) : 0u;
+}
+// Elements in lower lanes.
+__device__ __forceinline__ unsigned lanes_below_sum(unsigned x, unsigned lane)
+{
+    unsigned incl = x;
 #pragma unroll
-        for (int k = K - 1; k >= 0; --k) {
-            const uint32_t w = na ? a[k] : b[k];
-            if (w) loc = (int)((gl * K + k) * 32u) + __ffs(w) - 1;
-        }
-        if (G == 1) return loc;
-        if (G == 32) return (int)__reduce_min_sync(FULL, (unsigned)loc);
-        const unsigned m = na ? ba : bb;
-        const int src = m ? (__ffs(m) - 1) : (int)lane;
-        const int r = __shfl_sync(FULL, loc, src);
-        return m ? r : -1;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(FULL, incl, o);
+        incl += (int)lane >= o ? y : 0u;
     }
-    // Emptiness of two sets at once.
-    __device__ __forceinline__ void any2(const uint32_t (&a)[K], const uint32_t (&b)[K], bool &ra, bool &rb) const
-    {
-        uint32_t oa = 0, ob = 0;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            oa |= a[k];
-            ob |= b[k];
-        }
-        if (G == 1) {
-            ra = oa != 0u;
-            rb = ob != 0u;
-        } else if (G == 32) {
-            const unsigned m = __reduce_or_sync(FULL, (oa != 0u ? 1u : 0u) | (ob != 0u ? 2u : 0u));
-            ra = (m & 1u) != 0u;
-            rb = (m & 2u) != 0u;
-        } else {
-            const unsigned ba = __ballot_sync(FULL, oa != 0u), bb = __ballot_sync(FULL, ob != 0u);
-            ra = (ba & gmask) != 0u;
-            rb = (bb & gmask) != 0u;
-        }
-    }
-    __device__ __forceinline__ int sum(int x) const
-    {
-        if (G == 32) return (int)__reduce_add_sync(FULL, (unsigned)x);
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-        return x;
-    }
-    __device__ __forceinline__ int excl_scan(int x) const
-    {
-        int incl = x;
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            int y = __shfl_up_sync(FULL, incl, o, G);
-            if ((int)gl >= o) incl += y;
-        }
-        return incl - x;
-    }
-    __device__ __forceinline__ unsigned from_leader(unsigned x) const
-    {
-        if (G == 1) return x;
-        return __shfl_sync(FULL, x, gbase);
-    }
-    // Bits [0, end) of this lane's k-th word.
-    __device__ __forceinline__ uint32_t below(int k, unsigned end) const
-    {
-        unsigned base = (gl * K + k) * 32u;
-        if (end >= base + 32u) return FULL;
-        if (end <= base) return 0u;
-        return (1u << (end - base)) - 1u;
-    }
-    __device__ __forceinline__ void clear(uint32_t (&s)[K], int v) const
-    {
-        unsigned w = (unsigned)v >> 5;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-            if (w == gl * K + k) s[k] &= ~(1u << (v & 31));
-    }
-    __device__ __forceinline__ void set(uint32_t (&s)[K], int v) const
-    {
-        unsigned w = (unsigned)v >> 5;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-            if (w == gl * K + k) s[k] |= 1u << (v & 31);
-    }
-};
+    return incl - x;
+}
 
 template <int K, bool SMEM>
 __device__ __forceinline__ void load_row(uint32_t (&r)[K], const uint32_t *p)
@@ -420,6 +363,7 @@ __device__ __forceinline__ void vst(unsigned *p, unsigned v) { *reinterpret_cast
 __device__ __forceinline__ bool lq_reserve_push(LocalHdr *h, unsigned *seq, unsigned mask, unsigned &ticket)
 {
     unsigned pos = vld(&h->tail);
+#pragma unroll 1
     for (unsigned t = 0; t < 256; ++t) {
         const unsigned s = vld(&seq[pos & mask]);
         const int dif = (int)(s - pos);
@@ -439,6 +383,7 @@ __device__ __forceinline__ bool lq_reserve_push(LocalHdr *h, unsigned *seq, unsi
 __device__ __forceinline__ bool lq_reserve_pop(LocalHdr *h, unsigned *seq, unsigned mask, unsigned &ticket)
 {
     unsigned pos = vld(&h->head);
+#pragma unroll 1
     for (unsigned t = 0; t < 256; ++t) {
         const unsigned s = vld(&seq[pos & mask]);
         const int dif = (int)(s - (pos + 1));
@@ -474,15 +419,15 @@ __device__ __forceinline__ LocalQ local_queue_at(unsigned char *base, uint32_t w
 }
 
 // Reset the block's ring (whole block; a barrier must follow).
-__device__ __forceinline__ void local_queue_reset(const LocalQ &q, unsigned groups)
+__device__ __forceinline__ void local_queue_reset(const LocalQ &q, unsigned warps)
 {
+#pragma unroll 1
     for (unsigned i = threadIdx.x; i <= q.mask; i += blockDim.x) q.seq[i] = i;
     if (threadIdx.x == 0) {
         q.h->head = 0u;
         q.h->tail = 0u;
-        q.h->idle = groups;
+        q.h->idle = warps;
         q.h->bwork = 0u;
-        q.h->starving = 0u;
         q.h->poller = 0u;
         q.h->done = 0u;
         q.h->refreshing = 0u;
@@ -491,7 +436,6 @@ __device__ __forceinline__ void local_queue_reset(const LocalQ &q, unsigned grou
         q.h->g_starving = 0u;
         q.h->stamp = 0ull;
         q.h->trace_n = 0u;
-        q.h->t2_busy = 0u;
         for (int i = 0; i < kDiagCount; ++i) q.h->diag[i] = 0ull;
     }
 }
@@ -505,130 +449,6 @@ struct Counters {
     unsigned long long *diag = nullptr;
     __device__ __forceinline__ void note(int i, unsigned long long v = 1ull) const { atomicAdd(diag + i, v); }
 };
-
-// ---------------------------------------------------------------------------
-// Give away the front of a frame's branching set L (c elements, in order).
-// The taker gets L1 = the first `give` elements as the frame
-// (P, X, pivot, end = first kept element); the giver keeps the rest as
-// (P \ L1, X u L1, pivot, end).  Walking L1 then the rest is exactly the
-// sequential loop of Alg. 4 (each child sees P minus, and X plus, every
-// earlier sibling), so the search tree is the same however often it is cut.
-// give = floor(c/2) for c >= 2; with c == 1 the whole frame goes only when
-// `allow_whole`.  A frame whose candidate set has fewer than `min_p` vertices
-// is kept.  Returns true when a frame was handed over; the giver then applies
-// (P, X, L) &= ~L1 / |= L1 through the returned mask l1 (its own words).
-
-template <int G, int K, bool LOCAL>
-__device__ __forceinline__ bool donate_front(const Grp<G, K> &g, const SearchParams &prm, const LocalQ &lq,
-                                             bool pred, bool allow_whole, int min_p, const uint32_t (&P)[K],
-                                             const uint32_t (&X)[K], const uint32_t (&L)[K], unsigned pe,
-                                             unsigned rs, uint64_t S, bool list, const uint32_t (&R)[K],
-                                             uint32_t (&l1)[K], bool &whole, Counters &cn)
-{
-    constexpr int WP = G * K;
-    int cl = 0, cp = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        cl += __popc(L[k]);
-        cp += __popc(P[k]);
-    }
-    const int c = g.sum(cl);
-    const int np = g.sum(cp);
-    const int give = (c >= 2) ? c / 2 : ((c == 1 && allow_whole) ? 1 : 0);
-    const bool ok = pred && give > 0 && np >= min_p;
-    // split = position of element #give of L (the first one kept), or the
-    // frame's end when everything goes
-    const int pre = g.excl_scan(cl);
-    int pos = -1;
-    if (ok && give < c && pre <= give && give < pre + cl) {
-        int r = give - pre;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int cw = __popc(L[k]);
-            if (pos < 0) {
-                if (r < cw) {
-                    uint32_t w = L[k];
-                    for (int j = 0; j < r; ++j) w &= w - 1u;
-                    pos = (int)((g.gl * K + k) * 32u) + __ffs(w) - 1;
-                } else {
-                    r -= cw;
-                }
-            }
-        }
-    }
-    int split = pos;
-    if (G > 1) {
-        const unsigned b = __ballot_sync(FULL, pos >= 0) & g.gmask;
-        split = __shfl_sync(FULL, pos, b ? (__ffs(b) - 1) : (int)g.lane);
-    }
-    if (give >= c) split = (int)(pe >> 16);
-
-    // A frame in the block ring is block work (the giver keeps the block
-    // active); a frame in the global ring is one unit of global pending.
-    unsigned ticket = 0, got = 0;
-    if (ok && g.leader()) {
-        if (LOCAL) {
-            atomicAdd(&lq.h->bwork, 1u);
-            got = lq_reserve_push(lq.h, lq.seq, lq.mask, ticket) ? 1u : 0u;
-            if (!got) atomicSub(&lq.h->bwork, 1u);
-        } else {
-            atomicAdd(&prm.ctl->pending, 1u);
-            got = q_reserve_push(prm.ctl, prm.seq, prm.qcap - 1u, ticket, push_margin<G>(prm)) ? 1u : 0u;
-            if (got) cn.note(kDiagGpush);
-            if (!got) atomicSub(&prm.ctl->pending, 1u);
-        }
-    }
-    got = g.from_leader(got);
-    ticket = g.from_leader(ticket);
-    const unsigned npe = (pe & 0xffffu) | ((unsigned)split << 16);
-#pragma unroll
-    for (int k = 0; k < K; ++k) l1[k] = got ? (L[k] & g.below(k, (unsigned)split)) : 0u;
-    if (got) {
-        if (LOCAL) {
-            volatile uint32_t *fr = lq.frames + (size_t)(ticket & lq.mask) * frame_words(WP, list);
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                fr[kFrameHdr + g.gl * K + k] = P[k];
-                fr[kFrameHdr + WP + g.gl * K + k] = X[k];
-                if (list) fr[kFrameHdr + 2 * WP + g.gl * K + k] = R[k];
-            }
-            if (g.leader()) {
-                fr[0] = npe;
-                fr[1] = rs;
-                fr[2] = (uint32_t)S;
-                fr[3] = (uint32_t)(S >> 32);
-            }
-            __threadfence_block();
-        } else {
-            uint32_t *fr = prm.frames + (size_t)(ticket & (prm.qcap - 1u)) * prm.fs;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                __stcg(fr + kFrameHdr + g.gl * K + k, P[k]);
-                __stcg(fr + kFrameHdr + WP + g.gl * K + k, X[k]);
-                if (list) __stcg(fr + kFrameHdr + 2 * WP + g.gl * K + k, R[k]);
-            }
-            if (g.leader()) {
-                __stcg(fr + 0, npe);
-                __stcg(fr + 1, rs);
-                __stcg(fr + 2, (uint32_t)S);
-                __stcg(fr + 3, (uint32_t)(S >> 32));
-            }
-            __threadfence();
-        }
-    }
-    __syncwarp();
-    if (got && g.leader()) {
-        if (LOCAL) {
-            __threadfence_block();
-            vst(&lq.seq[ticket & lq.mask], ticket + 1u);
-        } else {
-            st_release(&prm.seq[ticket & (prm.qcap - 1u)], ticket + 1u);
-        }
-        cn.note(kDiagDonations);
-    }
-    whole = give >= c;
-    return got != 0u;
-}
 
 // Warp-reduce the counters and add them to out[] (one atomic per counter per
 // warp).  Called by all 32 lanes.
@@ -682,6 +502,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t mb, uint32_t parity)
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mb, uint32_t parity)
 {
     const uint64_t t0 = global_ns();
+#pragma unroll 1
     for (unsigned t = 0;; ++t) {
         if (mbar_try_wait(mb, parity)) return true;
         if ((t & 63u) == 63u && global_ns() - t0 > 2000000000ull) return false;
@@ -724,330 +545,767 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Explicit per-group stack of frames.  Levels [0, SL) live in this warp's
-// slice of shared memory, laid out [level][word][lane] so every lane has its
-// own bank; deeper levels live in local memory.  Per level a lane keeps its
-// K words of P and of X plus M "meta" words: with four or more lanes per
-// group, lane j < 4 of the group keeps field j of (pivot|end, |R|, S low,
-// S high) and the fields come back by shuffles; narrower groups keep all
-// four fields in every lane.  |R| and S are the same in every lane.
-template <int G, int K>
-struct Stack {
-    static constexpr int M = (G >= 4) ? 1 : 4;
-    static constexpr int LW = 2 * K + M;
-    uint32_t *sm;  // the warp's slice of shared memory (kept in a register)
-    unsigned ln;   // this lane
-    int SL;
-    uint32_t (*lw)[LW];  // local-memory levels, indexed by the absolute level
-
-    __device__ __forceinline__ static uint32_t pick(unsigned pe, unsigned rs, uint64_t S, unsigned j)
-    {
-        return j == 0u ? pe : (j == 1u ? rs : (j == 2u ? (uint32_t)S : (uint32_t)(S >> 32)));
-    }
-    // A shared-memory level: P of all 32 lanes (K words each, lane-major, so
-    // one vector access per lane), then X likewise, then M meta words per
-    // lane (word-major).  The region starts 16-byte aligned and a level is
-    // 128 * LW bytes, so every vector is aligned.
-    __device__ __forceinline__ static void st_vec(uint32_t *p, const uint32_t (&v)[K])
-    {
-        if (K == 1) {
-            p[0] = v[0];
-        } else if (K == 2) {
-            *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
-        } else {
-            *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], v[3]);
-        }
-    }
-    __device__ __forceinline__ static void ld_vec(const uint32_t *p, uint32_t (&v)[K])
-    {
-        if (K == 1) {
-            v[0] = p[0];
-        } else if (K == 2) {
-            const uint2 t = *reinterpret_cast<const uint2 *>(p);
-            v[0] = t.x;
-            v[1] = t.y;
-        } else {
-            const uint4 t = *reinterpret_cast<const uint4 *>(p);
-            v[0] = t.x;
-            v[1] = t.y;
-            v[2] = t.z;
-            v[3] = t.w;
-        }
-    }
-    __device__ __forceinline__ void put(int d, unsigned gl, const uint32_t (&P)[K], const uint32_t (&X)[K],
-                                        unsigned pe, unsigned rs, uint64_t S)
-    {
-        if (d < SL) {
-            uint32_t *w = sm + (size_t)d * LW * 32;
-            st_vec(w + ln * K, P);
-            st_vec(w + 32 * K + ln * K, X);
-            if (M == 1) {
-                if (gl < 4u) w[2 * K * 32 + ln] = pick(pe, rs, S, gl);
-            } else {
-#pragma unroll
-                for (int j = 0; j < M; ++j) w[(2 * K + j) * 32 + ln] = pick(pe, rs, S, (unsigned)j);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                lw[d][k] = P[k];
-                lw[d][K + k] = X[k];
-            }
-            if (M == 1) {
-                lw[d][2 * K] = pick(pe, rs, S, gl < 4u ? gl : 0u);
-            } else {
-#pragma unroll
-                for (int j = 0; j < M; ++j) lw[d][2 * K + j] = pick(pe, rs, S, (unsigned)j);
-            }
-        }
-    }
-    __device__ __forceinline__ void put_px(int d, const uint32_t (&P)[K], const uint32_t (&X)[K])
-    {
-        if (d < SL) {
-            uint32_t *w = sm + (size_t)d * LW * 32;
-            st_vec(w + ln * K, P);
-            st_vec(w + 32 * K + ln * K, X);
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                lw[d][k] = P[k];
-                lw[d][K + k] = X[k];
-            }
-        }
-    }
-    __device__ __forceinline__ void get(int d, uint32_t (&P)[K], uint32_t (&X)[K], uint32_t (&mr)[M])
-    {
-        if (d < SL) {
-            const uint32_t *w = sm + (size_t)d * LW * 32;
-            ld_vec(w + ln * K, P);
-            ld_vec(w + 32 * K + ln * K, X);
-#pragma unroll
-            for (int j = 0; j < M; ++j) mr[j] = w[(2 * K + j) * 32 + ln];
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                P[k] = lw[d][k];
-                X[k] = lw[d][K + k];
-            }
-#pragma unroll
-            for (int j = 0; j < M; ++j) mr[j] = lw[d][2 * K + j];
-        }
-    }
-};
-
-// Fields of a stack level from the meta words get() returned.  Warp-uniform
-// call (shuffles when the fields are spread over the group's lanes).
-template <int G, int K>
-__device__ __forceinline__ void meta_unpack(const Grp<G, K> &g, const uint32_t (&mr)[Stack<G, K>::M], unsigned &pe,
-                                            unsigned &rs, uint64_t &S)
-{
-    if (Stack<G, K>::M == 1) {
-        pe = __shfl_sync(FULL, mr[0], (int)g.gbase);
-        rs = __shfl_sync(FULL, mr[0], (int)g.gbase + 1);
-        const uint32_t lo = __shfl_sync(FULL, mr[0], (int)g.gbase + 2);
-        const uint32_t hi = __shfl_sync(FULL, mr[0], (int)g.gbase + 3);
-        S = (uint64_t)lo | ((uint64_t)hi << 32);
-    } else {
-        pe = mr[0];
-        rs = mr[Stack<G, K>::M > 1 ? 1 : 0];
-        S = (uint64_t)mr[Stack<G, K>::M > 2 ? 2 : 0] | ((uint64_t)mr[Stack<G, K>::M > 3 ? 3 : 0] << 32);
-    }
-}
-
-// Publish a frame (P, X, pivot|end, |R|, S, and R itself when listing) as it
-// stands to the global ring (one unit of global pending).  Warp-uniform call;
-// true where it went.
-template <int G, int K>
-__device__ __forceinline__ bool push_global(const Grp<G, K> &g, const SearchParams &prm, bool pred,
-                                            const uint32_t (&P)[K], const uint32_t (&X)[K], unsigned pe, unsigned rs,
-                                            uint64_t S, bool list, const uint32_t (&R)[K], Counters &cn)
-{
-    constexpr int WP = G * K;
-    const unsigned qmask = prm.qcap - 1u;
-    unsigned ticket = 0, got = 0;
-    if (pred && g.leader()) {
-        atomicAdd(&prm.ctl->pending, 1u);
-        got = q_reserve_push(prm.ctl, prm.seq, qmask, ticket, push_margin<G>(prm)) ? 1u : 0u;
-        if (got) cn.note(kDiagGpush);
-        if (!got) atomicSub(&prm.ctl->pending, 1u);
-    }
-    got = g.from_leader(got);
-    ticket = g.from_leader(ticket);
-    if (got) {
-        uint32_t *fr = prm.frames + (size_t)(ticket & qmask) * prm.fs;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            __stcg(fr + kFrameHdr + g.gl * K + k, P[k]);
-            __stcg(fr + kFrameHdr + WP + g.gl * K + k, X[k]);
-            if (list) __stcg(fr + kFrameHdr + 2 * WP + g.gl * K + k, R[k]);
-        }
-        if (g.leader()) {
-            __stcg(fr + 0, pe);
-            __stcg(fr + 1, rs);
-            __stcg(fr + 2, (uint32_t)S);
-            __stcg(fr + 3, (uint32_t)(S >> 32));
-        }
-        __threadfence();
-    }
-    __syncwarp();
-    if (got && g.leader()) st_release(&prm.seq[ticket & qmask], ticket + 1u);
-    return got != 0u;
-}
-
 // ---------------------------------------------------------------------------
-// The lane tier.  Most nodes of the search tree lie where few vertices are
-// left: once a frame's P u X has at most 32 vertices, nothing outside that
+// The warp tier.  Most nodes of the search tree lie where few vertices are
+// left: once a frame's P u X has at most 128 vertices, nothing outside that
 // set can ever enter a descendant's P or X (Alg. 4 only intersects them with
 // rows of vertices of P).  Such a frame is compressed: U = P u X in
 // increasing position is relabelled 0..u-1 -- order-preserving, so "first in
 // the order" is still the lowest set bit and every pivot rule (first of X or
 // P; the TX / TomitaBB argmax with ties to the earliest) picks the same
-// vertex -- its induced adjacency becomes u rows of 32 bits, and one lane
-// runs Alg. 4 on it alone with single-word sets, next to 31 other lanes doing
-// the same on their own subproblems.  The tree, the leaves and the hash terms
-// (through the positions of the local vertices) are exactly those of the
-// group search.
-
-struct T2Lane {
-    uint32_t P = 0, X = 0, L = 0, rs = 0;  // local sets of the current frame, |R|
-    uint64_t S = 0;                        // S(R)
-    int d = 0;                             // explicit-stack depth
-    bool busy = false;
+// vertex -- and its induced adjacency becomes u rows of W = ceil(u/32) words
+// in the warp's shared memory.  The whole warp then searches the subtree from
+// a stack of frames: a step hands the next 32 unexpanded children, counted
+// from the top of the stack down, to the 32 lanes, whatever frames they
+// belong to, and every lane computes its child from the frame's sets and
+// pushes it if it has children itself.  No lane keeps a frame between steps,
+// so a frame with many children that are leaves (most frames near the bottom)
+// takes as few steps as its children fill.  The tree, the leaves and the hash
+// terms are exactly those of the search by frames; only who expands which
+// node differs.
+//
+// What bounds it: issue slots.  A step of 29 nodes takes about 340
+// instructions with four-word sets, the SM issues on 60 to 70 % of its
+// cycles, and the rest waits on the step's chain of shared-memory loads (frame
+// -> pivot row -> child row -> pivot row).  Building a subproblem costs about
+// as much as 300 nodes.  Before, a warp searched 32 subproblems of at most 32
+// vertices, each by one lane with a stack of its own, and everything above 32
+// vertices a node per warp; now against then, ms: G(1000, 0.3) 3.2 / 5.8,
+// G(500, 0.5) 9.6 / 21.4, G(300, 0.5) 1.3 / 2.0, Moon-Moser 45 0.66 / 0.86,
+// G(45, 0.5) 0.052 / 0.10, G(100, 0.8) 1.1 / 2.6.  It loses where a search is
+// nothing but subproblems of ten nodes or so (G(700, 0.18) 0.49 / 0.45).
+//
+// Graphs of at most 128 vertices need no compression: their rows (and hash
+// terms) are laid out once per block and every frame goes to the warp tier as
+// it is.
+//
+// The warp's region of shared memory: local rows | hash terms of the local
+// vertices | their positions | leaf buffer | stack of frames.
+// A frame on the stack: P and X as they were when it was pushed (W words each),
+// then meta = pivot (7 bits) | subproblem slot (3) | |R| less the start
+// frame's (7) | children |L| (7) | children already taken (7), then S(R) in two
+// words.  L = P \ N(pivot) is recomputed; child i is its i-th element v, with
+// the earlier ones moved from P to X (Alg. 4's loop).  Frames are an odd
+// number of words, so lanes on consecutive frames touch different banks.
+template <int W>
+struct PoolShape {
+    static constexpr unsigned kFields = 2 * W + 3;
+    static constexpr unsigned kStride = W == 3 ? 4u : (unsigned)W;         // words of a local row
+    static constexpr unsigned kSlots = W == 1 ? 8u : (W == 2 ? 4u : 1u);   // subproblems searched together
+    static constexpr unsigned kSlotRows = 32u * W * kStride;               // row words of one subproblem
+    static constexpr unsigned kSlotVerts = 32u * W;
+    // byte offsets in the warp's region
+    static constexpr unsigned kHashOff = kSlots * kSlotRows * 4u;
+    static constexpr unsigned kPosOff = kHashOff + kSlots * kSlotVerts * 8u;
+    static constexpr unsigned kLeafOff = kPosOff + kSlots * kSlotVerts * 2u;
+    static constexpr unsigned kRs0Off = kLeafOff + kPoolLeafBytes;   // |R| of every slot's start frame
+    static constexpr unsigned kScratchOff = kRs0Off + 32u;           // one frame
+    static constexpr unsigned kStackOff = kScratchOff + 48u;
+    static_assert(kStackOff <= (unsigned)kPoolFixedBytes && kStackOff % 16u == 0u && kFields * 4u <= 48u,
+                  "the region's fixed part");
+    static_assert(kStackOff + 64u * kFields * 4u <= kPoolBytesMin, "a stack of at least 64 frames");
 };
-
-struct T2Warp {
-    uint32_t *A;    // [32 local rows][32 lanes]
-    uint16_t *pos;  // [32 local vertices][32 lanes]: position in the order
-    uint32_t *stk;  // [levels][kT2Fields][32 lanes]
-    uint32_t *piv;  // kPivotScratchWords: the lanes' words of P' (pivot scoring)
-    int levels;
+// The same for a size known at run time.
+struct PoolOffsets {
+    uint32_t hash, pos, leaf, rs0, stack;
 };
-
-// One node of every busy lane's subproblem: the child v = first of L of the
-// lane's current frame (the same step as the group search's section C, on
-// 32-bit sets).  Divergent by design: no warp collectives inside.
-template <int PIVOT>
-__device__ __forceinline__ void t2_step(T2Lane &t, const T2Warp &m, unsigned lane, const uint64_t *hv,
-                                        uint32_t *hist, uint64_t *out, uint32_t pivot_mode,
-                                        uint32_t (&spill)[32][kT2Fields], Counters &cn, unsigned *busy_lanes)
+template <int W>
+__device__ __forceinline__ PoolOffsets pool_offsets_of()
 {
-    if (!t.busy) return;
-    const int v = __ffs(t.L) - 1;
-    t.L &= t.L - 1u;
-    const uint32_t *A = m.A + lane;
-    const uint32_t a = A[v * 32];
-    const uint32_t Pc = t.P & a, Xc = t.X & a;  // P n N(v), X n N(v)
-    t.P &= ~(1u << v);                           // P <- P \ {v}
-    t.X |= 1u << v;                              // X <- X u {v}
-    const uint64_t Sc = t.S + hv[m.pos[v * 32 + lane]];
-    const unsigned k = t.rs + 1u;
-    if (Pc == 0u) {
-        if (Xc == 0u) {  // P u X empty: R u {v} is a maximal clique
-            ++cn.cnt;
-            cn.hash += mix64(Sc ^ mix64((uint64_t)k));
-            cn.max = k > cn.max ? k : cn.max;
-            const unsigned old = atomicAdd(&hist[k], 1u);
-            if (old == 0xffffffffu)
-                atomicAdd(reinterpret_cast<unsigned long long *>(out + MCE_OUT_HIST + k), 1ull << 32);
-        } else {
-            ++cn.dead;
-        }
+    using Sh = PoolShape<W>;
+    return {Sh::kHashOff, Sh::kPosOff, Sh::kLeafOff, Sh::kRs0Off, Sh::kStackOff};
+}
+__device__ __forceinline__ PoolOffsets pool_offsets(unsigned cls)
+{
+    return cls == 1u ? pool_offsets_of<1>()
+                     : (cls == 2u ? pool_offsets_of<2>() : (cls == 3u ? pool_offsets_of<3>() : pool_offsets_of<4>()));
+}
+
+// Flags beside the position (12 bits) of a vertex that is handed over.
+constexpr unsigned kPosInP = 0x8000u, kPosPivot = 0x4000u, kPosMask = 0x0fffu;
+
+// Where a warp's tier finds things (byte offsets in shared memory): the local
+// rows, hash terms and positions (the warp's own, or the block's when the
+// whole graph is small), the warp's region and the block ring.
+struct PoolAt {
+    uint32_t rows, hash, pos, region, lq, hist;
+};
+
+// Result counters of one warp-tier run (per lane).
+struct PoolCounters {
+    uint64_t hash = 0;
+    unsigned cnt = 0, intl = 0, dead = 0, max = 0;
+};
+
+template <int W>
+__device__ __forceinline__ void pool_row(uint32_t (&r)[W], const uint32_t *a)
+{
+    if constexpr (W == 1) {
+        r[0] = a[0];
+    } else if constexpr (W == 2) {
+        const uint2 t = *reinterpret_cast<const uint2 *>(a);
+        r[0] = t.x;
+        r[1] = t.y;
     } else {
-        ++cn.intl;
-    }
-    uint32_t Lc = 0u;
-    if (Pc != 0u) {
-        int p;
-        if (PIVOT == MCE_PIVOT_GREEDY) {
-            p = __ffs(Xc != 0u ? Xc : Pc) - 1;
-        } else {
-            // argmax |P' n N(u)| over X' (TX, NX) or P' u X' (TomitaBB),
-            // candidates in increasing position with '>' keeping the earliest
-            uint32_t cand = (PIVOT == MCE_PIVOT_GREEDY_TX) ? Xc : (Pc | Xc);
-            p = __ffs(Pc) - 1;  // TX with X' empty: first of P'
-            int best = -1;
-            const int all = __popc(Pc);
-            const bool nx = PIVOT == MCE_PIVOT_GREEDY_TX && pivot_mode == MCE_PIVOT_GREEDY_NX;
-            while (cand) {
-                const int u = __ffs(cand) - 1;
-                cand &= cand - 1u;
-                const int c = __popc(Pc & A[u * 32]);
-                if (c > best) {
-                    best = c;
-                    p = u;
-                }
-                if (nx && best == all) break;  // Naude's early exit: nothing later can beat it
-            }
-        }
-        Lc = Pc & ~A[p * 32];  // L' = P' \ N(p)
-    }
-    if (Lc != 0u) {
-        if (t.L != 0u) {  // the frame keeps children: push it
-            const uint32_t f[kT2Fields] = {t.P, t.X, t.L, t.rs, (uint32_t)t.S, (uint32_t)(t.S >> 32)};
-            if (t.d < m.levels) {
-                uint32_t *w = m.stk + (size_t)t.d * kT2Fields * 32 + lane;
-#pragma unroll
-                for (int i = 0; i < kT2Fields; ++i) w[i * 32] = f[i];
-            } else {
-#pragma unroll
-                for (int i = 0; i < kT2Fields; ++i) spill[t.d][i] = f[i];
-            }
-            ++t.d;
-        }
-        t.P = Pc;
-        t.X = Xc;
-        t.L = Lc;
-        t.rs = k;
-        t.S = Sc;
-    } else if (t.L == 0u) {  // the frame is exhausted: back to its parent
-        if (t.d == 0) {
-            t.busy = false;
-            atomicSub(busy_lanes, 1u);
-        } else {
-            --t.d;
-            uint32_t f[kT2Fields];
-            if (t.d < m.levels) {
-                const uint32_t *w = m.stk + (size_t)t.d * kT2Fields * 32 + lane;
-#pragma unroll
-                for (int i = 0; i < kT2Fields; ++i) f[i] = w[i * 32];
-            } else {
-#pragma unroll
-                for (int i = 0; i < kT2Fields; ++i) f[i] = spill[t.d][i];
-            }
-            t.P = f[0];
-            t.X = f[1];
-            t.L = f[2];
-            t.rs = f[3];
-            t.S = (uint64_t)f[4] | ((uint64_t)f[5] << 32);
-        }
+        const uint4 t = *reinterpret_cast<const uint4 *>(a);
+        r[0] = t.x;
+        r[1] = t.y;
+        r[2] = t.z;
+        if constexpr (W == 4) r[3] = t.w;
     }
 }
 
-// The search proper: the groups of this warp expand frames until the search
-// is over or aborts.  Work moves at two levels: idle groups take frames from
-// the block's shared-memory ring, which busy groups of the block refill by
-// giving away the front of their shallowest branching set; a block with idle
-// groups and an empty ring counts itself as starving, one of its idle warps
-// polls the global ring, and busy groups feed the global ring while starving
-// blocks outnumber its frames.  rows, hv, hist, lq are this block's staged
-// rows (or global rows), vertex hash terms, clique-size histogram and ring.
-// Called by all 32 lanes of every warp.
-template <int G, int K, bool SMEM, int PIVOT, bool LIST>
-__device__ __forceinline__ void search_loop(const SearchParams &prm, const uint32_t *rows, const uint64_t *hv,
-                                            uint32_t *hist, const LocalQ &lq, const Thresholds th,
-                                            uint32_t *stack_smem, int stack_smem_levels, unsigned char *t2_smem,
+template <int W>
+__device__ __forceinline__ bool pool_any(const uint32_t (&s)[W])
+{
+    uint32_t o = s[0];
+#pragma unroll
+    for (int k = 1; k < W; ++k) o |= s[k];
+    return o != 0u;
+}
+
+// Lowest element of a set (of an empty one: some value below 32 W after the
+// caller's mask).
+template <int W>
+__device__ __forceinline__ unsigned pool_first(const uint32_t (&s)[W])
+{
+    uint32_t w = s[W - 1];
+    unsigned base = 32u * (W - 1);
+#pragma unroll
+    for (int k = W - 2; k >= 0; --k)
+        if (s[k]) {
+            w = s[k];
+            base = 32u * (unsigned)k;
+        }
+    return base + (unsigned)__ffs(w) - 1u;
+}
+
+// Hand one subproblem to the warp's tier (all 32 lanes): `mine` are this
+// lane's words of U = P u X; the caller has written the positions of U with
+// their flags to the slot.  Lane i builds the local rows of U[i], U[i + 32],
+// ...: it walks its rows in word order, four words a load, and for every
+// vertex U[j] of a word (the same word and bit in every lane) rotates that
+// bit to place j of the row being assembled -- two instructions a column for
+// 32 rows, against a shuffle, a test and a ballot a row and 32 columns.  Rows
+// of more than 32 words (K > 1) would cost a sector of every lane's row for a
+// few bits (G(3000, 0.1): some 40 KB from L2 for 30 vertices); there the warp
+// reads one row at a time, lane i the word that holds U[i + 32 k], and a ballot
+// makes the local row.  The start frame goes on the stack as frame `slot`.
+template <int W, int K, bool SMEM>
+__device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const uint32_t *order, uint32_t region,
+                                        unsigned slot, uint32_t mine0, uint32_t mine1, uint32_t mine2, uint32_t mine3,
+                                        unsigned u, unsigned children, unsigned rs, uint64_t S)
+{
+    using Sh = PoolShape<W>;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const unsigned lane = threadIdx.x & 31u;
+    uint32_t *A = reinterpret_cast<uint32_t *>(smem_raw + region) + slot * Sh::kSlotRows;
+    uint64_t *lhv = reinterpret_cast<uint64_t *>(smem_raw + region + Sh::kHashOff) + slot * Sh::kSlotVerts;
+    const uint16_t *pos = reinterpret_cast<const uint16_t *>(smem_raw + region + Sh::kPosOff) + slot * Sh::kSlotVerts;
+    uint32_t *f = reinterpret_cast<uint32_t *>(smem_raw + region + Sh::kStackOff) + slot * Sh::kFields;
+    const uint32_t *srows = reinterpret_cast<const uint32_t *>(smem_raw);  // SMEM: the rows lead the block's shared memory
+    const uint32_t *row[W];
+    uint32_t qw[W], qm[W];  // word and bit of this lane's columns
+    unsigned pl = 0;
+#pragma unroll
+    for (int g = 0; g < W; ++g) {
+        const bool in = lane + 32u * g < u;
+        const unsigned e = in ? (unsigned)pos[lane + 32u * g] : 0u;
+        const unsigned q = e & kPosMask;
+        row[g] = (SMEM ? srows : rows) + (size_t)q * rw;
+        qw[g] = q >> 5;
+        qm[g] = in ? 1u << (q & 31u) : 0u;
+        if (in) lhv[lane + 32u * g] = mix64((uint64_t)order[q] + 1u);
+        const unsigned valid = __ballot_sync(FULL, in), p = __ballot_sync(FULL, (e & kPosInP) != 0u);
+        const unsigned pb = __ballot_sync(FULL, (e & kPosPivot) != 0u);
+        if (pb) pl = 32u * g + (unsigned)__ffs(pb) - 1u;
+        if (lane == 0) {
+            f[g] = p;
+            f[W + g] = valid & ~p;
+        }
+    }
+    if constexpr (K == 1) {
+        uint32_t acc[W];
+#pragma unroll
+        for (int g = 0; g < W; ++g) acc[g] = 0u;
+        unsigned j = 0;  // columns done
+        auto store = [&](unsigned kw) {
+#pragma unroll
+            for (int g = 0; g < W; ++g) {
+                A[(lane + 32u * g) * Sh::kStride + kw] = acc[g];
+                acc[g] = 0u;
+            }
+        };
+        const unsigned V = rw >= 4u ? 4u : rw;  // words of a load (rows are 1, 2 or a multiple of 4 words)
+        const unsigned sw = min(rw, 32u * K);
+#pragma unroll 1
+        for (unsigned w0 = 0; w0 < sw && j < u; w0 += 4u) {
+            // U's next four words (uniform), and the rows' (skipped where U has none)
+            uint32_t m[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const unsigned wi = w0 + t;
+                uint32_t x = mine0;
+                if (K > 1 && (wi % K) == 1u) x = mine1;
+                if (K > 2 && (wi % K) == 2u) x = mine2;
+                if (K > 2 && (wi % K) == 3u) x = mine3;
+                m[t] = __shfl_sync(FULL, x, (int)((wi / K) & 31u));
+                if (wi >= sw) m[t] = 0u;
+            }
+            if ((m[0] | m[1] | m[2] | m[3]) == 0u) continue;
+            uint32_t x[W][4];
+#pragma unroll
+            for (int g = 0; g < W; ++g) {
+                if (V == 4u) {
+                    const uint4 t = SMEM ? *reinterpret_cast<const uint4 *>(row[g] + w0)
+                                         : __ldg(reinterpret_cast<const uint4 *>(row[g] + w0));
+                    x[g][0] = t.x;
+                    x[g][1] = t.y;
+                    x[g][2] = t.z;
+                    x[g][3] = t.w;
+                } else {
+                    x[g][0] = SMEM ? row[g][0] : __ldg(row[g]);
+                    x[g][1] = V > 1u ? (SMEM ? row[g][1] : __ldg(row[g] + 1)) : 0u;
+                    x[g][2] = x[g][3] = 0u;
+                }
+            }
+#pragma unroll 1
+            for (int t = 0; t < 4; ++t) {
+                uint32_t mt = m[0];
+#pragma unroll 1
+                while (mt) {
+                    const unsigned rot = (j - (unsigned)__ffs(mt) + 1u) & 31u, bit = 1u << (j & 31u);
+                    mt &= mt - 1u;
+#pragma unroll
+                    for (int g = 0; g < W; ++g) acc[g] |= __funnelshift_l(x[g][0], x[g][0], rot) & bit;
+                    ++j;
+                    if ((j & 31u) == 0u) store(j / 32u - 1u);
+                }
+                m[0] = m[1];
+                m[1] = m[2];
+                m[2] = m[3];
+#pragma unroll
+                for (int g = 0; g < W; ++g) {
+                    x[g][0] = x[g][1];
+                    x[g][1] = x[g][2];
+                    x[g][2] = x[g][3];
+                }
+            }
+        }
+        if ((j & 31u) != 0u) store(j / 32u);
+        // words past the last column
+#pragma unroll 1
+        for (unsigned kw = (u + 31u) / 32u; kw < (unsigned)W; ++kw) store(kw);
+    } else {
+        constexpr int B = 4;  // rows at a time
+#pragma unroll 1
+        for (unsigned j0 = 0; j0 < u; j0 += B) {
+            uint32_t w[B][W];
+#pragma unroll
+            for (int t = 0; t < B; ++t) {
+                const unsigned qj = j0 + t < u ? pos[j0 + t] & kPosMask : 0u;
+#pragma unroll
+                for (int g = 0; g < W; ++g) w[t][g] = __ldg(rows + (size_t)qj * rw + qw[g]);
+            }
+#pragma unroll
+            for (int t = 0; t < B; ++t) {
+                uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                for (int g = 0; g < W; ++g) b[g] = __ballot_sync(FULL, (w[t][g] & qm[g]) != 0u);
+                if (lane == 0 && j0 + t < u) {
+                    uint32_t *a = A + (j0 + t) * Sh::kStride;
+                    if (W == 1) a[0] = b[0];
+                    else if (W == 2) *reinterpret_cast<uint2 *>(a) = make_uint2(b[0], b[1]);
+                    else *reinterpret_cast<uint4 *>(a) = make_uint4(b[0], b[1], b[2], b[3]);
+                }
+            }
+        }
+    }
+    if (lane == 0) {
+        f[2 * W] = pl | (slot << 7) | (children << 17);
+        f[2 * W + 1] = (uint32_t)S;
+        f[2 * W + 2] = (uint32_t)(S >> 32);
+        reinterpret_cast<uint32_t *>(smem_raw + region + Sh::kRs0Off)[slot] = rs;
+    }
+    __syncwarp();
+}
+
+// Position of the r-th (0-based) set bit of w, r < popc(w).
+__device__ __forceinline__ unsigned select_bit(uint32_t w, unsigned r)
+{
+    unsigned at = 0u;
+#pragma unroll
+    for (unsigned h = 16u; h != 0u; h >>= 1) {
+        const unsigned c = (unsigned)__popc((w >> at) & ((1u << h) - 1u));
+        const bool up = r >= c;
+        r -= up ? c : 0u;
+        at += up ? h : 0u;
+    }
+    return at;
+}
+
+// Give the frame at byte offset `frame`, as it stands, to the block ring
+// (`local`) or the device-wide ring as an ordinary frame over positions; the
+// copy there is left without children.  False when the ring is full.
+// Called by all 32 lanes; the warp holds a unit of block work.
+template <int W>
+__device__ __noinline__ bool pool_give(const PoolAt at, uint32_t frame, bool local)
+{
+    using Sh = PoolShape<W>;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const unsigned lane = threadIdx.x & 31u;
+    LocalHdr *h = reinterpret_cast<LocalHdr *>(smem_raw + at.lq);
+    const LocalQ lq = local_queue_at(smem_raw + at.lq, h->wp, h->slots);
+    uint32_t *f = reinterpret_cast<uint32_t *>(smem_raw + frame);
+    const uint32_t meta = f[2 * W];
+    const unsigned slot = (meta >> 7) & 7u, left = ((meta >> 17) & 127u) - (meta >> 24);
+    if (left == 0u) return true;  // nothing there
+    unsigned got = 0u, ticket = 0u;
+    if (lane == 0) {
+        if (local) {
+            atomicAdd(&h->bwork, 1u);
+            got = lq_reserve_push(h, lq.seq, lq.mask, ticket) ? 1u : 0u;
+            if (!got) atomicSub(&h->bwork, 1u);
+        } else {
+            atomicAdd(&h->ctl->pending, 1u);
+            got = q_reserve_push(h->ctl, h->gseq, h->qcap - 1u, ticket, h->margin) ? 1u : 0u;
+            if (!got) atomicSub(&h->ctl->pending, 1u);
+        }
+    }
+    got = __shfl_sync(FULL, got, 0);
+    ticket = __shfl_sync(FULL, ticket, 0);
+    if (!got) return false;
+    uint32_t *fr = local ? lq.frames + (size_t)(ticket & lq.mask) * frame_words(h->wp)
+                         : h->gframes + (size_t)(ticket & (h->qcap - 1u)) * h->fs;
+#pragma unroll 1
+    for (unsigned w = lane; w < 2u * h->wp; w += 32u) fr[kFrameHdr + w] = 0u;
+    __threadfence();
+    __syncwarp();
+    const uint16_t *pos = reinterpret_cast<const uint16_t *>(smem_raw + at.pos) + slot * Sh::kSlotVerts;
+    const uint32_t *a = reinterpret_cast<const uint32_t *>(smem_raw + at.rows) + slot * Sh::kSlotRows +
+                        (meta & 127u) * Sh::kStride;
+    unsigned taken = meta >> 24;  // the children already taken: from P to X
+    // The frame's own children end before its branching set does when it is
+    // the front of a set that was cut: `end` is the first position not its own.
+    unsigned ahead = left, end = h->n;
+#pragma unroll 1
+    for (int k = 0; k < W; ++k) {
+        uint32_t P = f[k], X = f[W + k];
+        uint32_t L = P & ~a[k], gone = 0u;
+        for (; taken != 0u && L != 0u; --taken) {
+            gone |= L & (0u - L);
+            L &= L - 1u;
+        }
+        P &= ~gone;
+        X |= gone;
+        const unsigned c = (unsigned)__popc(L);
+        if (ahead < c) {
+            end = pos[32 * k + select_bit(L, ahead)] & kPosMask;
+            ahead = 0xffffffffu;
+        } else if (ahead != 0xffffffffu) {
+            ahead -= c;
+        }
+        if (((P | X) >> lane) & 1u) {
+            const unsigned q = pos[32 * k + lane] & kPosMask;
+            atomicOr(fr + kFrameHdr + (((P >> lane) & 1u) ? 0u : h->wp) + (q >> 5), 1u << (q & 31u));
+        }
+    }
+    if (lane == 0) {
+        const uint32_t *rs0 = reinterpret_cast<const uint32_t *>(smem_raw + at.region + Sh::kRs0Off);
+        fr[0] = (uint32_t)(pos[meta & 127u] & kPosMask) | (end << 16);
+        fr[1] = rs0[slot] + ((meta >> 10) & 127u);
+        fr[2] = f[2 * W + 1];
+        fr[3] = f[2 * W + 2];
+        f[2 * W] = meta + (left << 24);
+    }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) {
+        if (local) {
+            vst(&lq.seq[ticket & lq.mask], ticket + 1u);
+        } else {
+            st_release(&h->gseq[ticket & (h->qcap - 1u)], ticket + 1u);
+            atomicAdd(&h->diag[kDiagGpush], 1ull);
+        }
+        atomicAdd(&h->diag[kDiagDonations], 1ull);
+    }
+    __syncwarp();
+    return true;
+}
+
+// Hash terms and sizes of up to 32 buffered leaves: lane i takes the entry at
+// e + 3 i; rs0 holds |R| of every slot's start frame.
+__device__ __forceinline__ void pool_leaves(const uint32_t *e, unsigned n, unsigned lane, const uint32_t *rs0,
+                                            uint32_t *hist, uint64_t *out, PoolCounters &c)
+{
+    const bool on = lane < n;
+    unsigned k = 0u;
+    if (on) {
+        const uint64_t S = (uint64_t)e[3 * lane] | ((uint64_t)e[3 * lane + 1] << 32);
+        const unsigned z = e[3 * lane + 2];
+        k = rs0[z >> 8] + (z & 255u);
+        ++c.cnt;
+        c.hash += mix64(S ^ mix64((uint64_t)k));
+        c.max = k > c.max ? k : c.max;
+    }
+    unsigned todo = __ballot_sync(FULL, on);
+#pragma unroll 1
+    while (todo) {  // one addition per size
+        const unsigned k0 = __shfl_sync(FULL, k, __ffs(todo) - 1);
+        const unsigned m = __ballot_sync(FULL, on && k == k0);
+        todo &= ~m;
+        if (lane == 0) {
+            const unsigned add = (unsigned)__popc(m), old = atomicAdd(&hist[k0], add);
+            if (old + add < old)
+                atomicAdd(reinterpret_cast<unsigned long long *>(out + MCE_OUT_HIST + k0), 1ull << 32);
+        }
+    }
+    __syncwarp();
+}
+
+// Pages of a warp's stack in local memory (32 frames each: a word per lane and
+// field); beyond kSoftPages a step takes one child at a time.
+constexpr unsigned kSoftPages = 8, kPages = kSoftPages + 128 / 32 + 1;
+
+// The bottom 32 frames of a full stack to a page, or the last page back to an
+// empty stack.
+template <int W>
+__device__ __noinline__ void pool_page(const PoolAt &at, uint32_t (*paged)[PoolShape<W>::kFields], unsigned &pages,
+                                       unsigned &cnt)
+{
+    constexpr unsigned F = PoolShape<W>::kFields;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const unsigned lane = threadIdx.x & 31u;
+    uint32_t *stk = reinterpret_cast<uint32_t *>(smem_raw + at.region + PoolShape<W>::kStackOff);
+    unsigned n = cnt, pg = pages;
+    if (n != 0u) {
+#pragma unroll 1
+        for (unsigned w = 0; w < F; ++w) paged[pg][w] = stk[w * 32u + lane];
+        ++pg;
+        n -= 32u;
+#pragma unroll 1
+        for (unsigned i = 0; i < n * F; i += 32u) {
+            __syncwarp();
+            const bool on = i + lane < n * F;
+            const uint32_t t = on ? stk[32u * F + i + lane] : 0u;
+            __syncwarp();
+            if (on) stk[i + lane] = t;
+        }
+    } else {
+        --pg;
+#pragma unroll 1
+        for (unsigned w = 0; w < F; ++w) stk[w * 32u + lane] = paged[pg][w];
+        n = 32u;
+    }
+    __syncwarp();
+    pages = pg;
+    cnt = n;
+}
+
+// What a long run looks at every few steps: it gives its oldest frames (of
+// the fullest subtrees; at most half of all it has) to idle warps -- the
+// block's own first, then any -- and watches for an abort and the search's
+// time limit.  True when the search has been aborted.
+template <int W>
+__device__ __noinline__ bool pool_watch(const PoolAt &at, uint32_t (*paged)[PoolShape<W>::kFields], unsigned pages,
+                                        unsigned cnt, unsigned &gave_io, uint64_t deadline, uint64_t *out)
+{
+    constexpr unsigned F = PoolShape<W>::kFields;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const unsigned lane = threadIdx.x & 31u;
+    LocalHdr *h = reinterpret_cast<LocalHdr *>(smem_raw + at.lq);
+    unsigned near = 0u, far = 0u;
+    if (lane == 0) {
+        Ctl *ctl = h->ctl;
+        const unsigned ab = ld_relaxed(&ctl->abort), gh = ld_relaxed(&ctl->head), gt = ld_relaxed(&ctl->tail);
+        const unsigned id = vld(&h->idle);
+        const bool shared_ring = h->total > blockDim.x / 32u;
+        const unsigned st = shared_ring ? ld_relaxed(&ctl->starving) : id;
+        const int l = (int)id - (int)(vld(&h->tail) - vld(&h->head));
+        const int g = (int)st - max((int)(gt - gh), 0) - max(l, 0);
+        near = (unsigned)min(max(l, 0), 4);
+        far = shared_ring ? (unsigned)min(max(g, 0), 4) : 0u;
+        if (4u * st > h->total) near |= 16u;  // draining (or filling): smaller frames too
+        if (deadline != ~0ull && global_ns() > deadline) set_status(out, ctl, MCE_ETIMEOUT);
+        if (ab) near = 32u;
+    }
+    near = __shfl_sync(FULL, near, 0);
+    far = __shfl_sync(FULL, far, 0);
+    if (near == 32u) return true;
+    const unsigned min_p = (near & 16u) != 0u ? h->give_p / 2u : h->give_p;
+    near &= 15u;
+    unsigned gave = gave_io;
+    const unsigned keep = (cnt + 32u * pages - gave + 1u) / 2u;  // frames this warp keeps
+#pragma unroll 1
+    for (; near + far != 0u && gave + keep < cnt + 32u * pages; ++gave) {
+        uint32_t frame = at.region + PoolShape<W>::kStackOff + (gave - 32u * pages) * F * 4u;
+        const bool out_page = gave < 32u * pages;
+        const unsigned pg = gave / 32u, q0 = (gave & 31u) * F;
+        if (out_page) {  // a frame that was paged out: through the scratch words
+            frame = at.region + PoolShape<W>::kScratchOff;
+            uint32_t *sc = reinterpret_cast<uint32_t *>(smem_raw + frame);
+#pragma unroll 1
+            for (unsigned w = 0; w < F; ++w) {
+                const unsigned q = w * 32u + lane - q0;
+                if (q < F) sc[q] = paged[pg][w];
+            }
+            __syncwarp();
+        }
+        const uint32_t *f = reinterpret_cast<const uint32_t *>(smem_raw + frame);
+        unsigned np = 0;
+#pragma unroll
+        for (int k = 0; k < W; ++k) np += (unsigned)__popc(f[k]);
+        const bool local = near != 0u;
+        if (np < min_p || !pool_give<W>(at, frame, local)) break;
+        near -= local ? 1u : 0u;
+        far -= local ? 0u : 1u;
+        if (out_page) {
+            const uint32_t m = f[2 * W];
+            __syncwarp();
+#pragma unroll 1
+            for (unsigned w = 0; w < F; ++w)
+                if (w * 32u + lane - q0 == 2u * W) paged[pg][w] = m;
+        }
+    }
+    gave_io = gave;
+    return false;
+}
+
+// Search the `cnt` start frames on the warp's stack to the end (all 32
+// lanes).  Leaves go to a buffer that is worked off 32 at a time, so that the
+// two 64-bit mixes of a clique's hash run on full warps.  cap = frames the
+// stack holds (at least 64).  Frames that would overflow it page out: the
+// bottom 32 go to local memory, a word per lane and field, and come back when
+// the stack is empty.  How many frames there can be: the frames pushed by one
+// step (at most 32) lie on top of the ones they are children of, so while
+// several steps' frames are on the stack their subtrees' heights fall from
+// step to step, and there are at most 32 per level of the tree.  Beyond
+// kSoftPages pages a step takes one child at a time, and the stack then grows
+// by less than one frame per level (at most 128), which the last pages hold.
+// Ends early, with the rest unsearched, only when the whole search has been
+// aborted.
+template <int W, int PIVOT>
+__device__ __noinline__ void pool_run(const PoolAt at, unsigned cnt, unsigned cap, uint64_t *out, uint64_t deadline,
+                                      PoolCounters &pc)
+{
+    using Sh = PoolShape<W>;
+    constexpr unsigned F = Sh::kFields;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned below = (1u << lane) - 1u;
+    const uint32_t *A0 = reinterpret_cast<const uint32_t *>(smem_raw + at.rows);
+    const uint64_t *lhv = reinterpret_cast<const uint64_t *>(smem_raw + at.hash);
+    uint32_t *leaf = reinterpret_cast<uint32_t *>(smem_raw + at.region + PoolShape<W>::kLeafOff);
+    const uint32_t *rs0 = reinterpret_cast<const uint32_t *>(smem_raw + at.region + Sh::kRs0Off);
+    uint32_t *stk = reinterpret_cast<uint32_t *>(smem_raw + at.region + PoolShape<W>::kStackOff);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + at.hist);
+    uint32_t paged[kPages][F];
+    unsigned pages = 0;
+    unsigned nleaf = 0;  // buffered leaves
+    unsigned gave = 0;   // frames at the bottom (of the first page, if any) that were given away
+    // (a step that scores pivots takes several times as long)
+    const unsigned give_mask = reinterpret_cast<const LocalHdr *>(smem_raw + at.lq)->give_mask >>
+                               (PIVOT == MCE_PIVOT_GREEDY ? 0 : 2);
+    PoolCounters c;
+
+#pragma unroll 1
+    for (unsigned step = 1;; ++step) {
+        if (cnt + 32u > cap || (cnt == 0u && pages != 0u)) pool_page<W>(at, paged, pages, cnt);
+        if (nleaf >= 32u || (cnt == 0u && nleaf != 0u)) {
+            const unsigned n = nleaf < 32u ? nleaf : 32u;
+            nleaf -= n;
+            pool_leaves(leaf + 3u * nleaf, n, lane, rs0, hist, out, c);
+        }
+        if (cnt == 0u) {
+            if (nleaf == 0u) break;
+            continue;
+        }
+        if ((step & give_mask) == 0u || (step <= 12u && (step & 3u) == 0u)) {
+            if (pool_watch<W>(at, paged, pages, cnt, gave, (step & 511u) == 0u ? deadline : ~0ull, out)) break;
+        }
+
+        // ---- hand out children: lane j looks at the j-th frame from the top
+        const uint32_t mj = lane < cnt ? stk[(cnt - 1u - lane) * F + 2 * W] : 0u;
+        const unsigned cj = ((mj >> 17) & 127u) - (mj >> 24);  // children left
+        unsigned incl = cj;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(FULL, incl, o);
+            incl += (int)lane >= o ? y : 0u;
+        }
+        const unsigned excl = incl - cj;
+        const unsigned most = pages < kSoftPages ? 32u : 1u;
+        // first lane of every frame's run of children
+        const unsigned firsts = __reduce_or_sync(FULL, cj != 0u && excl < most ? 1u << excl : 0u);
+        const unsigned total = min(most, __shfl_sync(FULL, incl, 31));
+        const unsigned upto = firsts & (below | (1u << lane));
+        const unsigned fi = (unsigned)__popc(upto) - 1u;  // this lane's frame from the top
+        const bool act = lane < total;
+        const unsigned gone_frames = (unsigned)__popc(__ballot_sync(FULL, lane < cnt && incl <= total));
+        const uint32_t *f = stk + (cnt - 1u - (act ? fi : 0u)) * F;
+        uint32_t P[W], X[W], L[W], a[W];
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            P[k] = f[k];
+            X[k] = f[W + k];
+        }
+        const uint32_t meta = f[2 * W];
+        const uint64_t S = (uint64_t)f[2 * W + 1] | ((uint64_t)f[2 * W + 2] << 32);
+        __syncwarp();
+        if (cj != 0u && excl < total && incl > total)  // the frame that keeps children
+            stk[(cnt - 1u - lane) * F + 2 * W] = mj + ((total - excl) << 24);
+        cnt -= gone_frames;
+        gave = min(gave, cnt + 32u * pages);
+
+        // ---- this lane's child v: element i of L, the earlier ones to X
+        // (lanes without one compute on the top frame, and none of it counts)
+        const unsigned slot = (meta >> 7) & 7u;
+        const uint32_t *A = A0 + slot * Sh::kSlotRows;
+        pool_row<W>(a, A + (meta & 127u) * Sh::kStride);
+        unsigned i = act ? (meta >> 24) + lane - (31u - (unsigned)__clz((int)upto)) : 0u;
+        // past[k]: the child lies past word k of L
+        bool past[W];
+        uint32_t lw;
+        unsigned vk = 0u;
+        {
+            unsigned run = 0u, skip = 0u;
+#pragma unroll
+            for (int k = 0; k < W; ++k) L[k] = P[k] & ~a[k];
+            lw = L[0];
+#pragma unroll
+            for (int k = 0; k < W - 1; ++k) {
+                run += (unsigned)__popc(L[k]);
+                past[k] = i >= run;
+                lw = past[k] ? L[k + 1] : lw;
+                skip = past[k] ? run : skip;
+                vk = past[k] ? 32u * (k + 1) : vk;
+            }
+            past[W - 1] = false;
+            i -= skip;
+        }
+        const unsigned vb = select_bit(lw, i) & 31u;
+        const unsigned v = vk + vb;
+        const uint32_t low = (1u << vb) - 1u;
+        pool_row<W>(a, A + v * Sh::kStride);
+        const uint64_t Sc = S + lhv[slot * Sh::kSlotVerts + v];
+        uint32_t op = 0u, ox = 0u;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const uint32_t g = L[k] & (past[k] ? FULL : (k == 0 || past[k > 0 ? k - 1 : 0] ? low : 0u));
+            P[k] = P[k] & ~g & a[k];    // (P minus the earlier children) n N(v)
+            X[k] = (X[k] | g) & a[k];   // (X and the earlier children) n N(v)
+            op |= P[k];
+            ox |= X[k];
+        }
+        const bool bp = act && op != 0u, bx = ox != 0u;
+        c.intl += bp ? 1u : 0u;
+        c.dead += act && !bp && bx ? 1u : 0u;
+        unsigned p = 0u;
+        if (PIVOT == MCE_PIVOT_GREEDY) {
+#pragma unroll
+            for (int k = 0; k < W; ++k) L[k] = bx ? X[k] : P[k];
+            p = bp ? pool_first<W>(L) : 0u;
+        } else if (bp) {
+            // argmax |P' n N(u)| over X' (TX, NX) or P' u X' (TomitaBB),
+            // candidates in increasing position with '>' keeping the earliest;
+            // one that covers all of P' cannot be beaten, which ends the scan
+            // under every rule (as Naude's early exit does)
+            p = pool_first<W>(P);  // TX with X' empty: first of P'
+            int best = -1, all = 0;
+#pragma unroll
+            for (int k = 0; k < W; ++k) all += __popc(P[k]);
+            bool open = true;
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                uint32_t cand = (PIVOT == MCE_PIVOT_GREEDY_TX) ? X[k] : (P[k] | X[k]);
+#pragma unroll 1
+                while (cand != 0u && open) {
+                    const unsigned w = 32u * k + (unsigned)__ffs(cand) - 1u;
+                    cand &= cand - 1u;
+                    uint32_t r[W];
+                    pool_row<W>(r, A + w * Sh::kStride);
+                    int n = 0;
+#pragma unroll
+                    for (int j = 0; j < W; ++j) n += __popc(P[j] & r[j]);
+                    if (n > best) {
+                        best = n;
+                        p = w;
+                    }
+                    open = best != all;
+                }
+            }
+        }
+        pool_row<W>(a, A + p * Sh::kStride);
+        unsigned n = 0;
+#pragma unroll
+        for (int k = 0; k < W; ++k) n += (unsigned)__popc(P[k] & ~a[k]);  // |L'|, L' = P' \ N(p)
+
+        // ---- P' u X' empty: R u {v} is a maximal clique
+        const unsigned rel = ((meta >> 10) & 127u) + 1u;
+        const bool lf = act && !bp && !bx;
+        const unsigned lm = __ballot_sync(FULL, lf);
+        if (lf) {
+            uint32_t *e = leaf + 3u * (nleaf + (unsigned)__popc(lm & below));
+            e[0] = (uint32_t)Sc;
+            e[1] = (uint32_t)(Sc >> 32);
+            e[2] = (slot << 8) | rel;
+        }
+        nleaf += (unsigned)__popc(lm);
+        // ---- a child with children of its own goes on the stack
+        const bool push = bp && n != 0u;
+        const unsigned pm = __ballot_sync(FULL, push);
+        if (push) {
+            uint32_t *fr = stk + (cnt + (unsigned)__popc(pm & below)) * F;
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                fr[k] = P[k];
+                fr[W + k] = X[k];
+            }
+            fr[2 * W] = p | (slot << 7) | (rel << 10) | (n << 17);
+            fr[2 * W + 1] = (uint32_t)Sc;
+            fr[2 * W + 2] = (uint32_t)(Sc >> 32);
+        }
+        cnt += (unsigned)__popc(pm);
+        __syncwarp();
+    }
+    pc = c;
+}
+
+// The warp tier with sets of `cls` words (the same for the whole search, so
+// that one instance of the code is in the instruction caches).
+template <int K, int PIVOT>
+__device__ __forceinline__ void pool_run_class(unsigned cls, const PoolAt &at, unsigned cnt, uint32_t bytes,
+                                               uint64_t *out, uint64_t deadline, PoolCounters &c)
+{
+    if (cls == 1u) pool_run<1, PIVOT>(at, cnt, (bytes - PoolShape<1>::kStackOff) / (4u * PoolShape<1>::kFields), out, deadline, c);
+    else if (cls == 2u) pool_run<2, PIVOT>(at, cnt, (bytes - PoolShape<2>::kStackOff) / (4u * PoolShape<2>::kFields), out, deadline, c);
+    else if (cls == 3u) pool_run<3, PIVOT>(at, cnt, (bytes - PoolShape<3>::kStackOff) / (4u * PoolShape<3>::kFields), out, deadline, c);
+    else pool_run<4, PIVOT>(at, cnt, (bytes - PoolShape<4>::kStackOff) / (4u * PoolShape<4>::kFields), out, deadline, c);
+}
+
+// The search proper: this warp expands frames until the search is over or
+// aborts.  rows, order: the renumbered adjacency (rows of prm.wp words, in
+// shared memory when SMEM) and the labels; hist, lq, region: this block's
+// clique-size histogram and ring and this warp's region of shared memory.
+// direct: the block holds the whole graph's rows, hash terms and positions in
+// the warp tier's layout (graphs of at most 128 vertices).  Called by all 32
+// lanes of every warp of the block.
+template <int K, bool SMEM, int PIVOT, bool LIST>
+__device__ __forceinline__ void search_loop(const SearchParams &prm, const uint32_t *rows, uint32_t *hist,
+                                            const LocalQ &lq, const Thresholds th, const PoolAt at, bool direct,
                                             Counters &cn)
 {
-    using Gp = Grp<G, K>;
-    constexpr int WP = G * K;
-    // the lane tier serves the counting kernels of groups of two or more
-    // lanes (one-lane groups already search with one or two words per lane)
-    constexpr bool T2 = !LIST && G >= 2;
-    constexpr unsigned GPW = 32u / G;  // groups per warp
-    const uint32_t n = prm.n;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr bool POOL = !LIST;
+    const uint32_t n = prm.n, rw = prm.wp;     // rw: words from row to row
+    const uint32_t sw = min(rw, 32u * K);      // words of a set
     Ctl *ctl = prm.ctl;
-    Gp g;
-    g.init();
+    LocalHdr *h = lq.h;
+    const unsigned lane = threadIdx.x & 31u;
+    const bool mine = lane * K < sw;  // this lane's words exist
+    const unsigned warps = blockDim.x >> 5;
+    const bool ring_shared = prm.total_groups > warps;
+    const unsigned qmask = prm.qcap - 1u;
     uint32_t P[K], X[K], L[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) P[k] = X[k] = L[k] = 0u;
@@ -1055,69 +1313,81 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
     uint64_t S = 0;
     int d = 0, dbase = 0;
     bool work = false;
-    bool lempty = true;  // the current frame's branching set is exhausted
-    bool poller = false;
-    unsigned gq = 0;  // global ring length last seen
-    // a claimed ticket of the device-wide ring whose frame this (idle) group
-    // takes once it is published
-    bool held = false;
+    bool lempty = true;     // the current frame's branching set is exhausted
+    bool fresh = false;     // the frame was just taken from a ring
+    bool open = true;       // the device-wide ring was short of frames when last seen
+    unsigned pslots = 0u;   // subproblems waiting on this warp's stack
+    // lane 0 only: the polling role, and a claimed ticket of the device-wide
+    // ring whose frame this (idle) warp takes once it is published
+    bool poller = false, held = false;
     unsigned hticket = 0;
-    // Clique listing (ListParams): this group's index, the |R| of the frame
-    // it took last, and (leader) the chunk it appends records to.
-    constexpr bool list = LIST;
-    const unsigned gidx = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32u / G) + g.lane / G;
+    // Clique listing (ListParams): this warp's index, the |R| of the frame it
+    // took last, and (lane 0) the chunk it appends records to.
+    const unsigned gidx = blockIdx.x * warps + (threadIdx.x >> 5);
     unsigned rsb = 0, cpos = 0, cend = 0;
     bool cfull = false;
 
-    using Stk = Stack<G, K>;
-    uint32_t stack_local[kStackDepth][Stk::LW];
-    Stk stk;
-    stk.SL = stack_smem_levels;
-    stk.sm = stack_smem + (size_t)(threadIdx.x >> 5) * (size_t)stack_smem_levels * Stk::LW * 32;
-    stk.ln = g.lane;
-    stk.lw = stack_local;
+    // ancestors of the current frame: P and X, and the scalars, one each in
+    // lanes 0..3 (pivot | end, |R|, S low, S high)
+    uint32_t stack[kStackDepth][2 * K + 1];
+    const PoolOffsets po = pool_offsets(th.cls);
+    uint16_t *ppos = reinterpret_cast<uint16_t *>(smem_raw + at.region + po.pos);
 
-    // lane tier: this lane's subproblem and the warp's region
-    T2Lane t2;
-    T2Warp t2m;
-    uint32_t t2_spill[32][kT2Fields];
-    const unsigned t2p = T2 ? min(prm.t2_max_p, th.share_local) : 0u;
-    {
-        unsigned char *wb = t2_smem + (size_t)(threadIdx.x >> 5) * t2_warp_bytes(prm.t2_levels, PIVOT != MCE_PIVOT_GREEDY);
-        t2m.A = reinterpret_cast<uint32_t *>(wb);
-        t2m.pos = reinterpret_cast<uint16_t *>(wb + 32 * 32 * 4);
-        t2m.stk = reinterpret_cast<uint32_t *>(wb + 32 * 32 * 4 + 32 * 32 * 2);
-        t2m.piv = t2m.stk + (size_t)prm.t2_levels * kT2Fields * 32;
-        t2m.levels = (int)prm.t2_levels;
-    }
-    unsigned t2it = 0;
-
-    uint64_t quiet_since = 0;
+    uint64_t quiet_since = 0, t_busy = 0;
     const uint64_t t_start = global_ns();
     unsigned last_pend = 0xffffffffu, last_head = 0xffffffffu;
-    unsigned backoff = 32;
-    const unsigned qmask = prm.qcap - 1u;
-    const size_t lfs = frame_words(WP, list);
+    unsigned backoff = 64;
 
-    auto rowp = [&](int v) -> const uint32_t * { return rows + (size_t)v * WP + g.gl * K; };
+    if (POOL && threadIdx.x == 0) {  // what the warp tier needs to give frames away
+        h->ctl = ctl;
+        h->gseq = prm.seq;
+        h->gframes = prm.frames;
+        h->qcap = prm.qcap;
+        h->fs = prm.fs;
+        h->margin = push_margin(prm);
+        h->wp = rw;
+        h->slots = lq.mask + 1u;
+        h->n = n;
+        h->give_p = prm.tune.give_p ? prm.tune.give_p : th.share;
+        h->total = ring_shared ? prm.total_groups : warps;
+        h->give_mask = prm.tune.give_steps - 1u;
+    }
+    __syncthreads();
 
-    // This lane's words of R for a frame of this group with |R| = r, plus
-    // vertex `extra` when it is >= 0 (listing only).
-    auto r_bits = [&](unsigned r, int extra, uint32_t (&out)[K]) {
-        const uint32_t *b = prm.lst.base + (size_t)gidx * WP + g.gl * K;
+    auto get_row = [&](uint32_t (&r)[K], unsigned v) {
+        if (mine) {
+            load_row<K, SMEM>(r, rows + (size_t)v * rw + lane * K);
+        } else {
 #pragma unroll
-        for (int k = 0; k < K; ++k) out[k] = b[k];
-        const uint16_t *pp = prm.lst.path + (size_t)gidx * n;
-        for (unsigned j = rsb; j < r; ++j) g.set(out, (int)pp[j]);
-        if (extra >= 0) g.set(out, extra);
+            for (int k = 0; k < K; ++k) r[k] = 0u;
+        }
+    };
+    auto scalars = [&]() -> uint32_t {
+        return lane == 0u ? pe : (lane == 1u ? rs : (lane == 2u ? (uint32_t)S : (uint32_t)(S >> 32)));
     };
 
-    // Append the maximal clique R u {v} (|R| = rs) as a record to this
-    // group's chunk.  Warp-uniform call; `emit` marks the groups reporting.
-    auto emit_clique = [&](bool emit, int v) {
+    // This lane's words of R for a frame of this warp with |R| = r, plus
+    // vertex `extra` when it is >= 0 (listing only).
+    auto r_bits = [&](unsigned r, int extra, uint32_t (&out)[K]) {
+        const uint32_t *b = prm.lst.base + (size_t)gidx * rw + lane * K;
+#pragma unroll
+        for (int k = 0; k < K; ++k) out[k] = mine ? b[k] : 0u;
+        const uint16_t *pp = prm.lst.path + (size_t)gidx * n;
+#pragma unroll 1
+        for (unsigned j = rsb; j < r; ++j)
+#pragma unroll
+            for (int k = 0; k < K; ++k) out[k] |= set_bit<K>(k, pp[j], lane);
+        if (extra >= 0)
+#pragma unroll
+            for (int k = 0; k < K; ++k) out[k] |= set_bit<K>(k, (unsigned)extra, lane);
+    };
+
+    // Append the maximal clique R u {v} (|R| = rs) as a record to this warp's
+    // chunk.
+    auto emit_clique = [&](int v) {
         const unsigned k = rs + 1u;
         unsigned ok = 0u, wpos = 0u;
-        if (emit && g.leader()) {
+        if (lane == 0) {
             const unsigned need = k + 1u, CW = prm.lst.chunk_words;
             if (cpos + need > cend && !cfull) {
                 if (cend) prm.lst.fill[cend / CW - 1u] = cpos - (cend - CW);  // retire the chunk
@@ -1137,78 +1407,113 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
                 cpos += need;
             }
         }
-        ok = g.from_leader(ok);
-        wpos = g.from_leader(wpos);
+        ok = __shfl_sync(FULL, ok, 0);
+        wpos = __shfl_sync(FULL, wpos, 0);
+        if (!ok) return;
         uint32_t rb[K];
-        const uint32_t *b = prm.lst.base + (size_t)gidx * WP + g.gl * K;
+        const uint32_t *b = prm.lst.base + (size_t)gidx * rw + lane * K;
 #pragma unroll
-        for (int kk = 0; kk < K; ++kk) rb[kk] = (emit && ok) ? b[kk] : 0u;
-        int c = 0;
+        for (int kk = 0; kk < K; ++kk) rb[kk] = mine ? b[kk] : 0u;
+        unsigned o = lanes_below_sum(set_count<K>(rb), lane);
+        // R of the taken frame fills slots [0, rsb), the path [rsb, rs), the
+        // leaf vertex slot rs
+        uint32_t *rec = prm.lst.rec + wpos + 1u;
 #pragma unroll
-        for (int kk = 0; kk < K; ++kk) c += __popc(rb[kk]);
-        int o = g.excl_scan(c);
-        if (emit && ok) {
-            // R of the taken frame fills slots [0, rsb), the path [rsb, rs),
-            // the leaf vertex slot rs
-            uint32_t *rec = prm.lst.rec + wpos + 1u;
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) {
-                uint32_t w = rb[kk];
-                while (w) {
-                    if (o < (int)rsb) rec[o] = (g.gl * K + kk) * 32u + (unsigned)(__ffs(w) - 1);
-                    ++o;
-                    w &= w - 1u;
-                }
+        for (int kk = 0; kk < K; ++kk) {
+            uint32_t w = rb[kk];
+            while (w) {
+                if (o < rsb) rec[o] = (lane * K + kk) * 32u + (unsigned)(__ffs(w) - 1);
+                ++o;
+                w &= w - 1u;
             }
-            const uint16_t *pp = prm.lst.path + (size_t)gidx * n;
-            for (unsigned j = rsb + g.gl; j < rs; j += G) rec[j] = pp[j];
-            if (g.leader()) {
-                rec[rs] = (uint32_t)v;
-                prm.lst.rec[wpos] = 0x80000000u | k;
-            }
+        }
+        const uint16_t *pp = prm.lst.path + (size_t)gidx * n;
+        for (unsigned j = rsb + lane; j < rs; j += 32u) rec[j] = pp[j];
+        if (lane == 0) {
+            rec[rs] = (uint32_t)v;
+            prm.lst.rec[wpos] = 0x80000000u | k;
         }
     };
 
-    // Take (P, X, pivot|end, |R|, S) as this group's frame.
-    uint64_t t_busy = 0;
-    auto start_frame = [&]() {
-        work = true;
-        lempty = false;
-        rsb = rs;
-        if (g.leader()) t_busy = global_ns();
-        d = dbase = 0;
-        uint32_t rp[K];
-        load_row<K, SMEM>(rp, rowp((int)(pe & 0xffffu)));
+    // Write a frame (and R when listing) to slot `ticket` of a ring and
+    // publish it.
+    auto publish = [&](bool local, unsigned ticket, const uint32_t (&fP)[K], const uint32_t (&fX)[K], unsigned fpe,
+                       unsigned frs, uint64_t fS, const uint32_t (&fR)[K]) {
+        uint32_t *fr = local ? lq.frames + (size_t)(ticket & lq.mask) * frame_words(rw, LIST)
+                             : prm.frames + (size_t)(ticket & qmask) * prm.fs;
+        if (mine) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) L[k] = P[k] & ~rp[k] & g.below(k, pe >> 16);
+            for (int k = 0; k < K; ++k) {
+                fr[kFrameHdr + lane * K + k] = fP[k];
+                fr[kFrameHdr + rw + lane * K + k] = fX[k];
+                if (LIST) fr[kFrameHdr + 2 * rw + lane * K + k] = fR[k];
+            }
+        }
+        if (lane == 0) {
+            fr[0] = fpe;
+            fr[1] = frs;
+            fr[2] = (uint32_t)fS;
+            fr[3] = (uint32_t)(fS >> 32);
+        }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) {
+            if (local) vst(&lq.seq[ticket & lq.mask], ticket + 1u);
+            else st_release(&prm.seq[ticket & qmask], ticket + 1u);
+            cn.note(kDiagDonations);
+        }
+        __syncwarp();
+    };
+    // A ticket of the block ring or the device-wide ring for a frame about to
+    // be published, or false.  A frame in the block ring is block work (the
+    // giver keeps the block active); one in the device-wide ring is a unit of
+    // global pending.
+    auto reserve = [&](bool local, unsigned &ticket) -> bool {
+        unsigned got = 0u;
+        ticket = 0u;
+        if (lane == 0) {
+            if (local) {
+                atomicAdd(&h->bwork, 1u);
+                got = lq_reserve_push(h, lq.seq, lq.mask, ticket) ? 1u : 0u;
+                if (!got) atomicSub(&h->bwork, 1u);
+            } else {
+                atomicAdd(&ctl->pending, 1u);
+                got = q_reserve_push(ctl, prm.seq, qmask, ticket, push_margin(prm)) ? 1u : 0u;
+                if (got) cn.note(kDiagGpush);
+                else atomicSub(&ctl->pending, 1u);
+            }
+        }
+        got = __shfl_sync(FULL, got, 0);
+        ticket = __shfl_sync(FULL, ticket, 0);
+        return got != 0u;
     };
 
-    // Share the shallowest frame this group owns (the stack bottom, else the
-    // current frame) through level LOCAL (true: block ring, false: global).
-    auto share = [&](bool want, bool local, int min_p) {
-        const bool from_stack = want && d > dbase;
-        uint32_t sP[K], sX[K], sL[K], l1[K];
-        uint32_t mr[Stk::M];
-#pragma unroll
-        for (int j = 0; j < Stk::M; ++j) mr[j] = 0u;
+    // Give away the front of the branching set of the shallowest frame this
+    // warp owns (the stack bottom, else the current frame): the taker gets
+    // the first half of L as the frame (P, X, pivot, end = first kept
+    // element), the giver keeps (P \ L1, X u L1).  Walking L1 then the rest is
+    // exactly the sequential loop of Alg. 4.  A stacked frame with one child
+    // left goes whole; a frame with |P| < min_p is kept.
+    auto share = [&](bool local, unsigned min_p) {
+        const bool from_stack = d > dbase;
+        uint32_t sP[K], sX[K], sL[K], sR[K];
         unsigned spe = pe, srs = rs;
         uint64_t sS = S;
-        if (from_stack) stk.get(dbase, sP, sX, mr);
-        {
-            unsigned pe2, rs2;
-            uint64_t S2;
-            meta_unpack<G, K>(g, mr, pe2, rs2, S2);
-            if (from_stack) {
-                spe = pe2;
-                srs = rs2;
-                sS = S2;
-            }
-        }
         if (from_stack) {
             uint32_t rp[K];
-            load_row<K, SMEM>(rp, rowp((int)(spe & 0xffffu)));
 #pragma unroll
-            for (int k = 0; k < K; ++k) sL[k] = sP[k] & ~rp[k] & g.below(k, spe >> 16);
+            for (int k = 0; k < K; ++k) {
+                sP[k] = stack[dbase][k];
+                sX[k] = stack[dbase][K + k];
+            }
+            const uint32_t m = stack[dbase][2 * K];
+            spe = __shfl_sync(FULL, m, 0);
+            srs = __shfl_sync(FULL, m, 1);
+            sS = (uint64_t)__shfl_sync(FULL, m, 2);
+            sS |= (uint64_t)__shfl_sync(FULL, m, 3) << 32;
+            get_row(rp, spe & 0xffffu);
+#pragma unroll
+            for (int k = 0; k < K; ++k) sL[k] = sP[k] & ~rp[k] & set_below<K>(k, spe >> 16, lane);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
@@ -1217,729 +1522,595 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
                 sL[k] = L[k];
             }
         }
-        uint32_t sR[K];
+        const unsigned cl = set_count<K>(sL);
+        const unsigned both = __reduce_add_sync(FULL, (set_count<K>(sP) << 16) | cl);
+        const unsigned c = both & 0xffffu;
+        const unsigned give = c >= 2u ? c / 2u : (c == 1u && from_stack ? 1u : 0u);
+        if (give == 0u || (both >> 16) < min_p) return;
+        // the position of element #give of L (the first one kept), or the
+        // frame's end when everything goes
+        unsigned split = spe >> 16;
+        if (give < c) {
+            const unsigned pre = lanes_below_sum(cl, lane);
+            unsigned at_pos = 0xffffffffu;
+            if (pre <= give && give < pre + cl) {
+                unsigned r = give - pre;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const unsigned cw = (unsigned)__popc(sL[k]);
+                    if (at_pos == 0xffffffffu) {
+                        if (r < cw) at_pos = (lane * K + k) * 32u + select_bit(sL[k], r);
+                        else r -= cw;
+                    }
+                }
+            }
+            split = __reduce_min_sync(FULL, at_pos);
+        }
+        unsigned ticket;
+        if (!reserve(local, ticket)) return;
 #pragma unroll
         for (int k = 0; k < K; ++k) sR[k] = 0u;
-        if (list && want) r_bits(srs, -1, sR);
-        bool whole = false, gave;
-        if (local)
-            gave = donate_front<G, K, true>(g, prm, lq, want, from_stack, min_p, sP, sX, sL, spe, srs, sS,
-                                            list, sR, l1, whole, cn);
-        else
-            gave = donate_front<G, K, false>(g, prm, lq, want, from_stack, min_p, sP, sX, sL, spe, srs, sS,
-                                             list, sR, l1, whole, cn);
-        if (gave) {
+        if (LIST) r_bits(srs, -1, sR);
+        publish(local, ticket, sP, sX, (spe & 0xffffu) | (split << 16), srs, sS, sR);
+        if (from_stack && give >= c) {
+            ++dbase;
+            return;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t l1 = sL[k] & set_below<K>(k, split, lane);
             if (from_stack) {
-                if (whole) {
-                    ++dbase;
-                } else {
-                    uint32_t nP[K], nX[K];
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        nP[k] = sP[k] & ~l1[k];
-                        nX[k] = sX[k] | l1[k];
-                    }
-                    stk.put_px(dbase, nP, nX);
-                }
+                stack[dbase][k] = sP[k] & ~l1;
+                stack[dbase][K + k] = sX[k] | l1;
             } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    P[k] &= ~l1[k];
-                    X[k] |= l1[k];
-                    L[k] &= ~l1[k];
-                }
+                P[k] &= ~l1;
+                X[k] |= l1;
+                L[k] &= ~l1;
             }
         }
     };
 
-    // Hand the child frames (Pc, Xc, Lc, |R| = rs1, S = Sc) of the groups
-    // with `comp` to free lanes of this warp as lane-tier subproblems (the
-    // first groups in lane order, as many as lanes are free).  Per group: the
-    // group's lanes list U = Pc u Xc in order into the slot's position column
-    // and form the local P, X, L words; then the whole warp builds the local
-    // rows, one ballot per row (lane i tests whether U[i] is adjacent to
-    // U[j]).  Warp-uniform call; true in the groups whose frame was taken.
-    auto t2_take = [&](bool comp, const uint32_t (&Pc)[K], const uint32_t (&Xc)[K], const uint32_t (&Lc)[K],
-                       unsigned rs1, uint64_t Sc) -> bool {
-        const unsigned freem = ~__ballot_sync(FULL, t2.busy);
-        const unsigned leads = __ballot_sync(FULL, comp && g.leader());
-        const unsigned rank = (unsigned)__popc(leads & ((1u << g.gbase) - 1u));
-        const bool ok = comp && rank < (unsigned)__popc(freem);
-        const unsigned okl = __ballot_sync(FULL, ok && g.leader());
-        if (okl == 0u) return false;
-        unsigned f = freem;
-        for (unsigned r = 0; r < rank && f; ++r) f &= f - 1u;
-        const unsigned slot = (ok && f) ? (unsigned)(__ffs(f) - 1) : 0u;
-        int cnt = 0;
-#pragma unroll
-        for (int k = 0; k < K; ++k) cnt += ok ? __popc(Pc[k] | Xc[k]) : 0;
-        const int off = g.excl_scan(cnt);
-        const int u_grp = g.sum(cnt);
-        uint32_t lp = 0u, lx = 0u, ll = 0u;
-        if (ok) {
-            unsigned i = (unsigned)off;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                uint32_t w = Pc[k] | Xc[k];
-                while (w) {
-                    const unsigned b = (unsigned)(__ffs(w) - 1);
-                    w &= w - 1u;
-                    t2m.pos[i * 32 + slot] = (uint16_t)((g.gl * K + k) * 32u + b);
-                    lp |= ((Pc[k] >> b) & 1u) << i;
-                    lx |= ((Xc[k] >> b) & 1u) << i;
-                    ll |= ((Lc[k] >> b) & 1u) << i;
-                    ++i;
-                }
-            }
+    // Search what waits on this warp's stack.
+    auto pool_flush = [&]() {
+        PoolCounters c;
+        PoolAt a = at;
+        if (!direct) {
+            a.rows = at.region;
+            a.hash = at.region + po.hash;
+            a.pos = at.region + po.pos;
         }
-        if (G > 1) {
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                lp |= __shfl_xor_sync(FULL, lp, o);
-                lx |= __shfl_xor_sync(FULL, lx, o);
-                ll |= __shfl_xor_sync(FULL, ll, o);
-            }
-        }
-        __syncwarp();
-        unsigned todo = okl;
-        while (todo) {
-            const int gb = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const unsigned s = __shfl_sync(FULL, slot, gb);
-            const unsigned u = (unsigned)__shfl_sync(FULL, u_grp, gb);
-            const uint32_t P0 = __shfl_sync(FULL, lp, gb), X0 = __shfl_sync(FULL, lx, gb);
-            const uint32_t L0 = __shfl_sync(FULL, ll, gb), r0 = __shfl_sync(FULL, rs1, gb);
-            const uint32_t s_lo = __shfl_sync(FULL, (uint32_t)Sc, gb), s_hi = __shfl_sync(FULL, (uint32_t)(Sc >> 32), gb);
-            const unsigned q = g.lane < u ? (unsigned)t2m.pos[g.lane * 32 + s] : 0u;
-            const uint32_t *rq = rows + (q >> 5);
-            const unsigned qb = q & 31u;
-            uint32_t row = 0u;
-#pragma unroll 4
-            for (unsigned j = 0; j < u; ++j) {
-                const unsigned qj = (unsigned)__shfl_sync(FULL, q, (int)j);
-                uint32_t w = 0u;
-                if (g.lane < u) w = SMEM ? rq[(size_t)qj * WP] : __ldg(rq + (size_t)qj * WP);
-                const unsigned b = __ballot_sync(FULL, (w >> qb) & 1u);
-                if (g.lane == j) row = b;
-            }
-            if (g.lane < u) t2m.A[g.lane * 32 + s] = row;
-            if (g.lane == s) {
-                t2.P = P0;
-                t2.X = X0;
-                t2.L = L0;
-                t2.rs = r0;
-                t2.S = (uint64_t)s_lo | ((uint64_t)s_hi << 32);
-                t2.d = 0;
-                t2.busy = true;
-            }
-        }
-        __syncwarp();
-        if (g.lane == 0) {
-            cn.note(kDiagLaneTasks, (unsigned long long)__popc(okl));
-            atomicAdd(&lq.h->t2_busy, (unsigned)__popc(okl));
-        }
-        return ok;
+        pool_run_class<K, PIVOT>(th.cls, a, pslots, prm.pool_bytes, prm.out, t_start + 10ull * prm.timeout_ns, c);
+        cn.cnt += c.cnt;
+        cn.intl += c.intl;
+        cn.dead += c.dead;
+        cn.hash += c.hash;
+        cn.max = c.max > cn.max ? c.max : cn.max;
+        pslots = 0u;
     };
 
-    for (unsigned it = 0;;) {
-        // ---- T: the lane tier.  While this warp's lanes hold subproblems,
-        // a lane step advances every one of them by a node.  It runs when
-        // fewer lanes are free than the warp has groups (room is made before
-        // the groups may hand over more), and when no group of the warp has a
-        // frame -- then every 4th iteration still goes through A and B so
-        // idle groups can take frames.
-        bool t2any = false;
-        if (T2) {
-            const unsigned busym = __ballot_sync(FULL, t2.busy);
-            t2any = busym != 0u;
-            if (t2any) {
-                const unsigned g1 = __ballot_sync(FULL, work);
-                if (32u - (unsigned)__popc(busym) < GPW || (g1 == 0u && (++t2it & 3u) != 0u)) {
-                    t2_step<PIVOT>(t2, t2m, g.lane, hv, hist, prm.out, prm.pivot_mode, t2_spill, cn,
-                                   &lq.h->t2_busy);
-                    continue;
-                }
+    // Hand the frame (tP, tX, tL, pivot tp, |R| = trs, S = tS) to the warp
+    // tier; what does not fit beside the subproblems already waiting has
+    // those searched first.
+    auto pool_take = [&](const uint32_t (&tP)[K], const uint32_t (&tX)[K], unsigned children, unsigned u, unsigned tp,
+                         unsigned trs, uint64_t tS) {
+        if (lane == 0) cn.note(kDiagLaneTasks);
+        if (direct) {
+            if (pslots != 0u) pool_flush();
+            uint32_t *f = reinterpret_cast<uint32_t *>(smem_raw + at.region + po.stack);
+            if (lane < th.cls) {
+                f[lane] = tP[0];
+                f[th.cls + lane] = tX[0];
             }
-        }
-        ++it;  // group-search iterations: the periodic ring checks below count these
-        // ---- A: a frame whose branching set is exhausted returns to its
-        // parent (a stacked level always has children left), or the group's
-        // work is done
-        const bool lpop = work && lempty && d > dbase;
-        const bool lfin = work && lempty && d <= dbase;
-        {
-            uint32_t mr[Stk::M];
-#pragma unroll
-            for (int j = 0; j < Stk::M; ++j) mr[j] = 0u;
-            if (lpop) {
-                --d;
-                stk.get(d, P, X, mr);
-            }
-            if (__ballot_sync(FULL, lpop) != 0u) {
-                unsigned pe2, rs2;
-                uint64_t S2;
-                meta_unpack<G, K>(g, mr, pe2, rs2, S2);
-                if (lpop) {
-                    pe = pe2;
-                    rs = rs2;
-                    S = S2;
-                    lempty = false;
-                    uint32_t rp[K];
-                    load_row<K, SMEM>(rp, rowp((int)(pe & 0xffffu)));
-#pragma unroll
-                    for (int k = 0; k < K; ++k) L[k] = P[k] & ~rp[k] & g.below(k, pe >> 16);
-                }
-            }
-        }
-        if (lfin) {
-            work = false;
-            lempty = false;
-            if (g.leader()) {
-                cn.note(kDiagBusyNs, global_ns() - t_busy);
-                atomicAdd(&lq.h->idle, 1u);
-                // the last work of the block gives back its unit
-                if (atomicSub(&lq.h->bwork, 1u) == 1u) atomicSub(&ctl->pending, 1u);
-            }
-        }
-
-        // ---- B1: the block ring (idle groups take, busy groups refill)
-        const unsigned busy_b = __ballot_sync(FULL, work);
-        if (busy_b != FULL || (it & (prm.tune.local_check - 1u)) == 0u) {
-            unsigned lh = 0, lt = 0, li = 0, ld = 0;
-            if (g.lane == 0) {
-                lh = vld(&lq.h->head);
-                lt = vld(&lq.h->tail);
-                li = vld(&lq.h->idle);
-                ld = vld(&lq.h->done);
-            }
-            lh = __shfl_sync(FULL, lh, 0);
-            lt = __shfl_sync(FULL, lt, 0);
-            li = __shfl_sync(FULL, li, 0);
-            ld = __shfl_sync(FULL, ld, 0);
-            if (busy_b == 0u && ld && !t2any) break;
-            const unsigned lqueued = lt - lh;
-            unsigned ticket = 0, got = 0;
-            if (!work && !held && lqueued != 0u && g.leader()) got = lq_reserve_pop(lq.h, lq.seq, lq.mask, ticket) ? 1u : 0u;
-            got = g.from_leader(got);
-            ticket = g.from_leader(ticket);
-            if (got) {
-                __threadfence_block();
-                const volatile uint32_t *fr = lq.frames + (size_t)(ticket & lq.mask) * lfs;
-                pe = fr[0];
-                rs = fr[1];
-                S = (uint64_t)fr[2] | ((uint64_t)fr[3] << 32);
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    P[k] = fr[kFrameHdr + g.gl * K + k];
-                    X[k] = fr[kFrameHdr + WP + g.gl * K + k];
-                }
-                if (list) {
-                    uint32_t *b = prm.lst.base + (size_t)gidx * WP + g.gl * K;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) b[k] = fr[kFrameHdr + 2 * WP + g.gl * K + k];
-                }
+            if (lane == 0) {
+                f[2 * th.cls] = tp | (trs << 10) | (children << 17);
+                f[2 * th.cls + 1] = (uint32_t)tS;
+                f[2 * th.cls + 2] = (uint32_t)(tS >> 32);
+                reinterpret_cast<uint32_t *>(smem_raw + at.region + po.rs0)[0] = 0u;
             }
             __syncwarp();
-            if (got) {
-                if (g.leader()) {
-                    __threadfence_block();
-                    vst(&lq.seq[ticket & lq.mask], ticket + lq.mask + 1u);
-                    atomicSub(&lq.h->idle, 1u);
-                    cn.note(kDiagSteals);
-                }
-                start_frame();
+            pslots = 1u;
+            return;
+        }
+        const unsigned slots = th.cls == 1u ? PoolShape<1>::kSlots : (th.cls == 2u ? PoolShape<2>::kSlots : 1u);
+        if (pslots >= slots) pool_flush();
+        const unsigned slot = pslots++;
+        uint32_t U[4] = {0u, 0u, 0u, 0u};
+        unsigned cnt = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            U[k] = tP[k] | tX[k];
+            cnt += (unsigned)__popc(U[k]);
+        }
+        unsigned i = slot * 32u * th.cls + lanes_below_sum(cnt, lane);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            uint32_t w = U[k];
+#pragma unroll 1
+            while (w) {
+                const unsigned b = (unsigned)(__ffs(w) - 1);
+                w &= w - 1u;
+                const unsigned q = (lane * K + k) * 32u + b;
+                ppos[i++] = (uint16_t)(q | (((tP[k] >> b) & 1u) ? kPosInP : 0u) | (q == tp ? kPosPivot : 0u));
             }
-            const bool hungry = work && !got && li > lqueued;
-            // with half the block's groups idle, smaller frames are worth moving
-            const unsigned bgroups = (blockDim.x >> 5) * (32u / G);
-            const int lmin = 2u * li > bgroups ? (int)min(th.share_local, prm.tune.share_tail) : (int)th.share_local;
-            if (__ballot_sync(FULL, hungry) != 0u) share(hungry, true, lmin);
+        }
+        __syncwarp();
+        const uint32_t *src = SMEM ? nullptr : rows;
+        if (th.cls == 1u)
+            pool_build<1, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+        else if (th.cls == 2u)
+            pool_build<2, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+        else if (th.cls == 3u)
+            pool_build<3, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+        else
+            pool_build<4, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+    };
+    // whether a frame of |P| = np, |P u X| = u and c children fits the tier
+    auto pool_fits = [&](unsigned np, unsigned u, unsigned c) -> bool {
+        return POOL && prm.t2_max_p != 0u && u <= 32u * th.cls && np <= min(prm.t2_max_p, th.task) && c <= 127u;
+    };
+
+#pragma unroll 1
+    for (unsigned it = 1;; ++it) {
+        // ---- A: a frame whose branching set is exhausted returns to its
+        // parent (a stacked level always has children left), or the warp's
+        // work is done.  (Subproblems of the warp tier are searched first: the
+        // frames they give away are block work, which this warp's unit keeps
+        // alive.)
+        if (work && lempty) {
+            if (d > dbase) {
+                --d;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    P[k] = stack[d][k];
+                    X[k] = stack[d][K + k];
+                }
+                const uint32_t m = stack[d][2 * K];
+                pe = __shfl_sync(FULL, m, 0);
+                rs = __shfl_sync(FULL, m, 1);
+                S = (uint64_t)__shfl_sync(FULL, m, 2);
+                S |= (uint64_t)__shfl_sync(FULL, m, 3) << 32;
+                uint32_t rp[K];
+                get_row(rp, pe & 0xffffu);
+#pragma unroll
+                for (int k = 0; k < K; ++k) L[k] = P[k] & ~rp[k] & set_below<K>(k, pe >> 16, lane);
+                lempty = false;
+            } else {
+                if (POOL && pslots != 0u) pool_flush();
+                work = false;
+                if (lane == 0) {
+                    cn.note(kDiagBusyNs, global_ns() - t_busy);
+                    atomicAdd(&h->idle, 1u);
+                    if (ring_shared) atomicAdd(&ctl->starving, 1u);
+                    // the last work of the block gives back its unit
+                    if (atomicSub(&h->bwork, 1u) == 1u) atomicSub(&ctl->pending, 1u);
+                }
+                backoff = 64;
+            }
         }
 
-        // ---- B2: the global ring and the end of the search.  Global state is
-        // read by the block's polling warp (an all-idle warp) or, at most
-        // every tune.refresh_ns, by one busy warp, and cached in shared memory.
-        const unsigned busy2 = __ballot_sync(FULL, work);
-        const bool anyheld = __ballot_sync(FULL, held) != 0u;
-        const bool periodic = busy2 == 0u || (it & (prm.tune.global_check - 1u)) == 0u;
-        // a held ticket is looked at every eighth iteration of a warp whose
-        // other groups are busy (each look is a round trip to L2)
-        if (periodic || (anyheld && (it & 7u) == 0u)) {
-            unsigned head = 0, tail = 0, pend = 1, starving = 0, ab = 0, lh = 0, lt = 0, done = 0;
-            bool pol = poller;
-            if (g.lane == 0) {
-                lh = vld(&lq.h->head);
-                lt = vld(&lq.h->tail);
-                // the polling warp is one with nothing at all to do (no frame and no
-                // lane-tier subproblem): it polls every iteration
-                if (busy2 == 0u && !pol && !t2any) pol = atomicCAS(&lq.h->poller, 0u, 1u) == 0u;
-                const uint64_t now = global_ns();
-                bool refresh = pol;
-                if (!refresh && now - *reinterpret_cast<volatile unsigned long long *>(&lq.h->stamp) > prm.tune.refresh_ns)
-                    refresh = atomicCAS(&lq.h->refreshing, 0u, 1u) == 0u;
-                if (refresh) {
-                    ab = ld_relaxed(&ctl->abort);
-                    pend = ld_relaxed(&ctl->pending);
-                    head = ld_relaxed(&ctl->head);
-                    tail = ld_relaxed(&ctl->tail);
-                    starving = ld_relaxed(&ctl->starving);
-                    // this block is starving while it has idle groups and an empty ring
-                    const bool st = vld(&lq.h->idle) != 0u && lt == lh;
-                    if (st != (vld(&lq.h->starving) != 0u)) {
-                        if (st) {
-                            if (atomicExch(&lq.h->starving, 1u) == 0u) atomicAdd(&ctl->starving, 1u);
-                        } else {
-                            if (atomicExch(&lq.h->starving, 0u) == 1u) atomicSub(&ctl->starving, 1u);
-                        }
-                    }
-                    vst(&lq.h->g_head, head);
-                    vst(&lq.h->g_tail, tail);
-                    vst(&lq.h->g_starving, starving);
-                    if (ab || pend == 0u) vst(&lq.h->done, ab ? 2u : 1u);
-                    *reinterpret_cast<volatile unsigned long long *>(&lq.h->stamp) = now;
-                    if (prm.trace) {
-                        const unsigned ti = atomicAdd(&lq.h->trace_n, 1u);
-                        if (ti < prm.trace_per_block) {
-                            const unsigned groups = prm.total_groups / gridDim.x;
-                            const unsigned busy = groups - min(groups, vld(&lq.h->idle));
-                            const unsigned qg = (int)(tail - head) > 0 ? min(tail - head, 65535u) : 0u;
-                            const unsigned sv = min(starving, 65535u);
-                            unsigned long long *rec = prm.trace + 2ull * ((size_t)blockIdx.x * prm.trace_per_block + ti);
-                            rec[0] = now;
-                            rec[1] = (unsigned long long)busy | ((unsigned long long)min(vld(&lq.h->t2_busy), 65535u) << 16) |
-                                     ((unsigned long long)qg << 32) | ((unsigned long long)sv << 48);
-                        }
-                    }
-                    if (now - t_start > 10ull * prm.timeout_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
-                    if (!pol) atomicExch(&lq.h->refreshing, 0u);
-                } else {
-                    head = vld(&lq.h->g_head);
-                    tail = vld(&lq.h->g_tail);
-                    starving = vld(&lq.h->g_starving);
-                    ab = vld(&lq.h->done) == 2u ? 1u : 0u;
+        // ---- B: idle warps take a frame (block ring first, then the
+        // device-wide ring), or end with the search; the block's polling warp
+        // refreshes the cached global state for the others
+        if (!work) {
+            unsigned code = 0u, ticket = 0u;  // 1: block ring, 2: device-wide ring, 3: the end
+            if (lane == 0) {
+                // (nothing to be seen: sleep on, in a loop of a few instructions)
+#pragma unroll 1
+                for (unsigned naps = 0; naps < 64u && !poller && !held; ++naps) {
+                    if (vld(&h->done) != 0u || vld(&h->tail) != vld(&h->head) || vld(&h->poller) == 0u ||
+                        (int)(vld(&h->g_tail) - vld(&h->g_head)) > 0)
+                        break;
+                    __nanosleep(backoff);
+                    backoff = backoff < prm.tune.idle_sleep_ns ? backoff * 2u : prm.tune.idle_sleep_ns;
                 }
-                done = vld(&lq.h->done);
-            }
-            pol = __shfl_sync(FULL, pol ? 1u : 0u, 0) != 0u;
-            poller = pol;
-            ab = __shfl_sync(FULL, ab, 0);
-            pend = __shfl_sync(FULL, pend, 0);
-            head = __shfl_sync(FULL, head, 0);
-            tail = __shfl_sync(FULL, tail, 0);
-            starving = __shfl_sync(FULL, starving, 0);
-            lh = __shfl_sync(FULL, lh, 0);
-            lt = __shfl_sync(FULL, lt, 0);
-            done = __shfl_sync(FULL, done, 0);
-            if (ab) break;
-            if (busy2 == 0u && done && !t2any) break;
-            // (claimed tickets can run ahead of the producers': nothing queued)
-            const unsigned queued = (int)(tail - head) > 0 ? tail - head : 0u;
-            gq = queued;
-
-            // An idle group takes a global frame when its block's ring is
-            // empty; only the block's polling warp asks, one group per try, so
-            // the ring's head sees one contender per block instead of one per
-            // idle group (the block's other groups get work from the taker
-            // through the block ring).
-            // (A block-private ring, as in the batched form, has no other
-            // contenders: there every idle group asks.)
-            // The polling warp's first asking group takes frames for up to four
-            // of the warp's asking groups with one ticket advance.
-            unsigned ticket = 0, got = 0;
-            const bool ring_shared = prm.total_groups > (blockDim.x >> 5) * (32u / G);
-            const bool ask = !work && !held && queued != 0u && lt == lh && (poller || !ring_shared) && g.leader();
-            const unsigned askers = __ballot_sync(FULL, ask);
-            if (!ring_shared) {
-                if (ask) {
-                    cn.note(kDiagGtry);
-                    got = q_reserve_pop(ctl, prm.seq, qmask, ticket, cn.diag + kDiagCasFail, prm.tune.pop_tries) ? 1u : 0u;
-                }
-            } else if (askers != 0u) {
-                const unsigned lead = (unsigned)(__ffs(askers) - 1);
-                unsigned first = 0u, k = 0u;
-                if (g.lane == lead) {
-                    cn.note(kDiagGtry);
-                    k = q_claim(ctl, min(4u, (unsigned)__popc(askers)), first);
-                }
-                k = __shfl_sync(FULL, k, (int)lead);
-                first = __shfl_sync(FULL, first, (int)lead);
-                const unsigned rank = (unsigned)__popc(askers & ((1u << g.lane) - 1u));
-                if (ask && rank < k) {
-                    held = true;
-                    hticket = first + rank;
-                }
-            }
-            got = g.from_leader(got);
-            ticket = g.from_leader(ticket);
-            held = g.from_leader(held ? 1u : 0u) != 0u;
-            hticket = g.from_leader(hticket);
-            if (ring_shared && __ballot_sync(FULL, held) != 0u) {
-                // a held ticket's frame, once its producer has published it
-                unsigned rdy = 0u;
-                if (held && g.leader()) rdy = ld_acquire(&prm.seq[hticket & qmask]) == hticket + 1u ? 1u : 0u;
-                rdy = g.from_leader(rdy);
-                if (rdy) {
-                    got = 1u;
+                if (vld(&h->done)) code = 3u;
+                if (code == 0u && held && ld_acquire(&prm.seq[hticket & qmask]) == hticket + 1u) {
+                    code = 2u;
                     ticket = hticket;
                     held = false;
                 }
+                if (code == 0u && !held && vld(&h->tail) != vld(&h->head) && lq_reserve_pop(h, lq.seq, lq.mask, ticket))
+                    code = 1u;
+                if (code == 0u && !poller) poller = atomicCAS(&h->poller, 0u, 1u) == 0u;
+                if (code == 0u && poller) {
+                    const uint64_t now = global_ns();
+                    const unsigned ab = ld_relaxed(&ctl->abort), pend = ld_relaxed(&ctl->pending);
+                    const unsigned gh = ld_relaxed(&ctl->head), gt = ld_relaxed(&ctl->tail);
+                    const unsigned st = ld_relaxed(&ctl->starving);
+                    vst(&h->g_head, gh);
+                    vst(&h->g_tail, gt);
+                    vst(&h->g_starving, st);
+                    *reinterpret_cast<volatile unsigned long long *>(&h->stamp) = now;
+                    if (ab || pend == 0u) {
+                        vst(&h->done, ab ? 2u : 1u);
+                        code = 3u;
+                    }
+                    // a stalled search: nothing moved for the whole budget
+                    if (pend != last_pend || gh != last_head || quiet_since == 0) {
+                        quiet_since = now;
+                        last_pend = pend;
+                        last_head = gh;
+                    } else if (now - quiet_since > prm.timeout_ns) {
+                        set_status(prm.out, ctl, MCE_ETIMEOUT);
+                    }
+                    if (now - t_start > 10ull * prm.timeout_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
+                    if (prm.trace) {
+                        const unsigned ti = atomicAdd(&h->trace_n, 1u);
+                        if (ti < prm.trace_per_block) {
+                            const unsigned busy = warps - min(warps, vld(&h->idle));
+                            const unsigned qg = (int)(gt - gh) > 0 ? min(gt - gh, 65535u) : 0u;
+                            unsigned long long *rec = prm.trace + 2ull * ((size_t)blockIdx.x * prm.trace_per_block + ti);
+                            rec[0] = now;
+                            rec[1] = (unsigned long long)busy | ((unsigned long long)qg << 32) |
+                                     ((unsigned long long)min(st, 65535u) << 48);
+                        }
+                    }
+                }
+                if (code == 0u && !held && (int)(vld(&h->g_tail) - vld(&h->g_head)) > 0) {
+                    cn.note(kDiagGtry);
+                    if (ring_shared) {
+                        if (q_claim(ctl, 1u, hticket) != 0u) {
+                            if (ld_acquire(&prm.seq[hticket & qmask]) == hticket + 1u) {
+                                code = 2u;
+                                ticket = hticket;
+                            } else {
+                                held = true;
+                            }
+                        } else {
+                            vst(&h->g_head, vld(&h->g_tail));  // (seen empty: wait for the next refresh)
+                        }
+                    } else if (q_reserve_pop(ctl, prm.seq, qmask, ticket, cn.diag + kDiagCasFail, prm.tune.pop_tries)) {
+                        code = 2u;
+                    }
+                }
             }
-            if (got) {
-                __threadfence();
-                const uint32_t *fr = prm.frames + (size_t)(ticket & qmask) * prm.fs;
+            code = __shfl_sync(FULL, code, 0);
+            ticket = __shfl_sync(FULL, ticket, 0);
+            if (code == 3u) break;
+            if (code == 0u) {
+                // the poller (or holder of a ticket) backs off too
+                if (lane == 0 && (poller || held)) {
+                    __nanosleep(backoff < 512u ? backoff : 512u);
+                    backoff = backoff < 512u ? backoff * 2u : 512u;
+                }
+                __syncwarp();
+                continue;
+            }
+            const bool local = code == 1u;
+            const uint32_t *fr = local ? lq.frames + (size_t)(ticket & lq.mask) * frame_words(rw, LIST)
+                                       : prm.frames + (size_t)(ticket & qmask) * prm.fs;
+            __threadfence();
+            if (local) {
+                const volatile uint32_t *v = fr;
+                pe = v[0];
+                rs = v[1];
+                S = (uint64_t)v[2] | ((uint64_t)v[3] << 32);
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    P[k] = mine ? v[kFrameHdr + lane * K + k] : 0u;
+                    X[k] = mine ? v[kFrameHdr + rw + lane * K + k] : 0u;
+                    if (LIST && mine)
+                        prm.lst.base[(size_t)gidx * rw + lane * K + k] = v[kFrameHdr + 2 * rw + lane * K + k];
+                }
+            } else {
                 pe = __ldcg(fr + 0);
                 rs = __ldcg(fr + 1);
                 S = (uint64_t)__ldcg(fr + 2) | ((uint64_t)__ldcg(fr + 3) << 32);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    P[k] = __ldcg(fr + kFrameHdr + g.gl * K + k);
-                    X[k] = __ldcg(fr + kFrameHdr + WP + g.gl * K + k);
-                }
-                if (list) {
-                    uint32_t *b = prm.lst.base + (size_t)gidx * WP + g.gl * K;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) b[k] = __ldcg(fr + kFrameHdr + 2 * WP + g.gl * K + k);
+                    P[k] = mine ? __ldcg(fr + kFrameHdr + lane * K + k) : 0u;
+                    X[k] = mine ? __ldcg(fr + kFrameHdr + rw + lane * K + k) : 0u;
+                    if (LIST && mine)
+                        prm.lst.base[(size_t)gidx * rw + lane * K + k] = __ldcg(fr + kFrameHdr + 2 * rw + lane * K + k);
                 }
             }
             __syncwarp();
-            if (got) {
-                if (g.leader()) {
+            if (lane == 0) {
+                if (local) {
+                    __threadfence_block();
+                    vst(&lq.seq[ticket & lq.mask], ticket + lq.mask + 1u);
+                } else {
                     st_release(&prm.seq[ticket & qmask], ticket + prm.qcap);
-                    atomicSub(&lq.h->idle, 1u);
                     // an already active block absorbs the frame's unit
-                    if (atomicAdd(&lq.h->bwork, 1u) != 0u) atomicSub(&ctl->pending, 1u);
-                    cn.note(kDiagSteals);
+                    if (atomicAdd(&h->bwork, 1u) != 0u) atomicSub(&ctl->pending, 1u);
                     cn.note(kDiagGlobal);
                 }
-                start_frame();
-            }
-            if (poller && __ballot_sync(FULL, work) != 0u) {
-                // busy now: hand the polling role to another idle warp
-                if (g.lane == 0) atomicExch(&lq.h->poller, 0u);
-                poller = false;
-            }
-
-            // busy groups feed starving blocks
-            const bool hungry = periodic && work && !got && starving > queued;
-            // with half the blocks starving (the search is draining), so are
-            // smaller frames
-            const int gmin = 2u * starving > gridDim.x ? (int)min(th.share_global, prm.tune.share_tail)
-                                                       : (int)th.share_global;
-            if (__ballot_sync(FULL, hungry) != 0u) share(hungry, false, gmin);
-
-            if (__ballot_sync(FULL, work) == 0u) {
-                if (T2 && t2any) continue;  // no frame, but subproblems: back to the lane tier
-                // nobody here has work: back off; the poller watches for a
-                // stalled search
-                if (g.lane == 0 && poller) {
-                    const uint64_t now = global_ns();
-                    if (pend != last_pend || head != last_head || quiet_since == 0) {
-                        quiet_since = now;
-                        last_pend = pend;
-                        last_head = head;
-                    } else if (now - quiet_since > prm.timeout_ns) {
-                        set_status(prm.out, ctl, MCE_ETIMEOUT);
-                    }
+                atomicSub(&h->idle, 1u);
+                if (ring_shared) atomicSub(&ctl->starving, 1u);
+                cn.note(kDiagSteals);
+                if (poller) {  // busy now: another idle warp polls
+                    atomicExch(&h->poller, 0u);
+                    poller = false;
                 }
-                // the poller backs off to 1 us; other idle warps only wait for
-                // the block ring and may sleep longer (fewer issue slots taken
-                // from the busy warps of the SM)
-                __nanosleep(backoff);
-                const unsigned cap = (poller || anyheld) ? 1024u : prm.tune.idle_sleep_ns;
-                backoff = backoff < cap ? backoff * 2u : cap;
+                t_busy = global_ns();
+            }
+            quiet_since = 0;
+            work = true;
+            fresh = true;
+            lempty = false;
+            rsb = rs;
+            d = dbase = 0;
+            uint32_t rp[K];
+            get_row(rp, pe & 0xffffu);
+#pragma unroll
+            for (int k = 0; k < K; ++k) L[k] = P[k] & ~rp[k] & set_below<K>(k, pe >> 16, lane);
+        }
+
+        // ---- a frame just taken that fits the warp tier goes there whole
+        if (fresh) {
+            fresh = false;
+            uint32_t u = 0;
+#pragma unroll
+            for (int k = 0; k < K; ++k) u += (unsigned)__popc(P[k] | X[k]);
+            const unsigned pu = __reduce_add_sync(FULL, (set_count<K>(P) << 16) | u);
+            const unsigned c = __reduce_add_sync(FULL, set_count<K>(L));
+            if (pool_fits(pu >> 16, pu & 0xffffu, c)) {
+                if (c != 0u) pool_take(P, X, c, pu & 0xffffu, pe & 0xffffu, rs, S);
+                lempty = true;
                 continue;
             }
-            backoff = 32;
         }
 
-        // ---- C: expand one child v = first(L) of every active frame.  After
-        // A and B every busy group has a non-empty branching set: pops and
-        // queued frames always carry children, and giving work away always
-        // leaves the giver at least one.
-        // (a frame without children would give v < 0; the group then just
-        // returns from it, reading no row)
-        const int v = g.first(L);
-        const bool act = work && v >= 0;
-        uint32_t Pc[K], Xc[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) Pc[k] = Xc[k] = 0u;
-        if (act) {
-            g.clear(L, v);
-            uint32_t r[K];
-            load_row<K, SMEM>(r, rowp(v));
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                Pc[k] = P[k] & r[k];  // P n N(v)
-                Xc[k] = X[k] & r[k];  // X n N(v)
+        // ---- busy warps refill the block ring while the block has more idle
+        // warps than queued frames, and the device-wide ring while the GPU has
+        if ((it & (prm.tune.local_check - 1u)) == 0u) {
+            unsigned want = 0u;
+            bool half = false;  // draining (or filling): smaller frames too
+            if (lane == 0) {
+                const int l = (int)vld(&h->idle) - (int)(vld(&h->tail) - vld(&h->head));
+                if (l > 0) {
+                    want = 1u;
+                    half = 4u * vld(&h->idle) > warps;
+                } else if ((it & (prm.tune.global_check - 1u)) == 0u) {
+                    const uint64_t now = global_ns();
+                    if (now - *reinterpret_cast<volatile unsigned long long *>(&h->stamp) > prm.tune.refresh_ns &&
+                        atomicCAS(&h->refreshing, 0u, 1u) == 0u) {
+                        const unsigned ab = ld_relaxed(&ctl->abort);
+                        vst(&h->g_head, ld_relaxed(&ctl->head));
+                        vst(&h->g_tail, ld_relaxed(&ctl->tail));
+                        vst(&h->g_starving, ld_relaxed(&ctl->starving));
+                        if (ab) vst(&h->done, 2u);
+                        if (now - t_start > 10ull * prm.timeout_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
+                        *reinterpret_cast<volatile unsigned long long *>(&h->stamp) = now;
+                        atomicExch(&h->refreshing, 0u);
+                    }
+                    if ((int)vld(&h->g_starving) > max((int)(vld(&h->g_tail) - vld(&h->g_head)), 0)) want = 2u;
+                    half = 4u * vld(&h->g_starving) > prm.total_groups;
+                }
+                if (vld(&h->done) == 2u) want = 3u;
+                if ((int)(vld(&h->g_tail) - vld(&h->g_head)) < (int)prm.split_target) want |= 4u;
+                if (half) want |= 8u;
             }
-            g.clear(P, v);  // P <- P \ {v}
-            g.set(X, v);    // X <- X u {v}
+            want = __shfl_sync(FULL, want, 0);
+            open = (want & 4u) != 0u;
+            half = (want & 8u) != 0u;
+            want &= 3u;
+            if (want == 3u) break;
+            if (want != 0u) share(want == 1u, (want == 1u ? th.share : th.share_far) >> (half ? 1 : 0));
         }
-        // first vertices of X' and P' (ChoosePivotOrdered's candidates) also
-        // answer the emptiness tests of the leaf test
-        bool bx, bp;
-        int fp = -1, pg = -1;
-        if (PIVOT == MCE_PIVOT_GREEDY) {
-            pg = g.first_either(Xc, Pc, bx, bp);
-        } else {
-            const int fx = g.first(Xc);
-            fp = g.first(Pc);
-            bx = fx >= 0;
-            bp = fp >= 0;
+
+        // ---- C: expand one child v = first(L).  (Pops and queued frames
+        // always carry children, and giving work away always leaves the giver
+        // at least one; a frame without would just be returned from.)
+        const int v = set_first<K>(L, lane);
+        if (v < 0) {
+            lempty = true;
+            continue;
         }
-        uint64_t Sc = 0;
-        if (act) Sc = S + hv[v];  // every lane keeps |R| and S
-        // every node is internal, a leaf or a dead end (nodes = their sum,
-        // formed when the counters are flushed)
-        const bool lead = act && g.leader();
-        cn.intl += (lead && bp) ? 1u : 0u;
-        cn.dead += (lead && !bp && bx) ? 1u : 0u;
-        if (lead && !bp && !bx) {  // P u X empty: R u {v} is a maximal clique
-            const unsigned k = rs + 1u;
-            ++cn.cnt;
-            cn.hash += mix64(Sc ^ mix64((uint64_t)k));
-            cn.max = k > cn.max ? k : cn.max;
-            const unsigned old = atomicAdd(&hist[k], 1u);
-            if (old == 0xffffffffu)
-                atomicAdd(reinterpret_cast<unsigned long long *>(prm.out + MCE_OUT_HIST + k), 1ull << 32);
+        uint32_t Pc[K], Xc[K], r[K];
+        get_row(r, (unsigned)v);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t b = set_bit<K>(k, (unsigned)v, lane);
+            Pc[k] = P[k] & r[k];  // P n N(v)
+            Xc[k] = X[k] & r[k];  // X n N(v)
+            L[k] &= ~b;
+            P[k] &= ~b;  // P <- P \ {v}
+            X[k] |= b;   // X <- X u {v}
         }
-        if (list) {
-            const bool emit = act && !bp && !bx;
-            if (__ballot_sync(FULL, emit) != 0u) emit_clique(emit, v);
+        const bool bp = __ballot_sync(FULL, set_or<K>(Pc) != 0u) != 0u;
+        const bool bx = __ballot_sync(FULL, set_or<K>(Xc) != 0u) != 0u;
+        const uint64_t Sc = S + mix64((uint64_t)prm.order[v] + 1u);
+        lempty = __ballot_sync(FULL, set_or<K>(L) != 0u) == 0u;
+        if (!bp) {
+            if (bx) {
+                cn.dead += lane == 0 ? 1u : 0u;
+            } else {  // P u X empty: R u {v} is a maximal clique
+                if (lane == 0) {
+                    const unsigned k = rs + 1u;
+                    ++cn.cnt;
+                    cn.hash += mix64(Sc ^ mix64((uint64_t)k));
+                    cn.max = k > cn.max ? k : cn.max;
+                    const unsigned old = atomicAdd(&hist[k], 1u);
+                    if (old == 0xffffffffu)
+                        atomicAdd(reinterpret_cast<unsigned long long *>(prm.out + MCE_OUT_HIST + k), 1ull << 32);
+                }
+                if (LIST) emit_clique(v);
+            }
+            continue;
         }
-        const bool inter = act && bp;
+        cn.intl += lane == 0 ? 1u : 0u;
 
         // ChoosePivotOrdered on the child (P', X')
-        int pc;
+        unsigned pc;
         if (PIVOT == MCE_PIVOT_GREEDY) {
-            pc = pg;
-        } else if (T2 && prm.t2_max_p != 0u) {
+            pc = (unsigned)(bx ? set_first<K>(Xc, lane) : set_first<K>(Pc, lane));
+        } else if (PIVOT == MCE_PIVOT_GREEDY_TX && !bx) {
+            pc = (unsigned)set_first<K>(Pc, lane);
+        } else {
             // argmax |P' n N(u)| over X' (TX, NX) or P' u X' (TomitaBB), all
             // candidates at once: the lanes' words of P' go to the warp's
-            // scratch, every lane scores the candidates in its own words
-            // against the whole of P' (16-byte loads starting at a chunk
-            // rotated by lane, so a phase of eight lanes hits distinct
-            // banks), and one packed max (score + 1, 0xffff - position) over
-            // the group keeps the highest score, earliest on ties.  NX has
-            // TX's pivot (its early exit only saves work).
-            Stk::st_vec(t2m.piv + g.lane * K, Pc);
+            // scratch (the leaf buffer, empty here), every lane scores the
+            // candidates in its own words against the whole of P' (16-byte
+            // loads starting at a chunk rotated by lane, so a phase of eight
+            // lanes hits distinct banks), and one packed max (score + 1,
+            // 0xffff - position) keeps the highest score, earliest on ties.
+            // NX has TX's pivot (its early exit only saves work).
+            uint32_t *pw = reinterpret_cast<uint32_t *>(smem_raw + at.region + po.leaf);
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (mine) pw[lane * K + k] = Pc[k];
             __syncwarp();
-            const uint32_t *pw = t2m.piv + g.gbase * K;  // this group's P' (WP words)
             unsigned best = 0u;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                uint32_t w = 0u;
-                if (inter) w = (PIVOT == MCE_PIVOT_GREEDY_TX) ? (bx ? Xc[k] : 0u) : (Pc[k] | Xc[k]);
+                uint32_t w = (PIVOT == MCE_PIVOT_GREEDY_TX) ? Xc[k] : (Pc[k] | Xc[k]);
+#pragma unroll 1
                 while (w) {
                     const unsigned b = (unsigned)(__ffs(w) - 1);
                     w &= w - 1u;
-                    const unsigned u = (g.gl * K + k) * 32u + b;
-                    const uint32_t *ru = rows + (size_t)u * WP;
-                    int c = 0;
-                    if (WP >= 4) {
-                        constexpr int NC = WP >= 4 ? WP / 4 : 1;
+                    const unsigned u = (lane * K + k) * 32u + b;
+                    const uint32_t *ru = rows + (size_t)u * rw;
+                    unsigned c = 0;
+                    if (sw >= 4u) {
+                        const unsigned nc = sw / 4u;
 #pragma unroll 4
-                        for (int j = 0; j < NC; ++j) {
-                            const int jj = ((j + (int)g.lane) & (NC - 1)) * 4;
+                        for (unsigned j = 0; j < nc; ++j) {
+                            const unsigned jj = ((j + lane) & (nc - 1u)) * 4u;
                             const uint4 a = *reinterpret_cast<const uint4 *>(pw + jj);
-                            const uint4 r = SMEM ? *reinterpret_cast<const uint4 *>(ru + jj)
+                            const uint4 q = SMEM ? *reinterpret_cast<const uint4 *>(ru + jj)
                                                  : __ldg(reinterpret_cast<const uint4 *>(ru + jj));
-                            c += __popc(a.x & r.x) + __popc(a.y & r.y) + __popc(a.z & r.z) + __popc(a.w & r.w);
+                            c += (unsigned)(__popc(a.x & q.x) + __popc(a.y & q.y) + __popc(a.z & q.z) + __popc(a.w & q.w));
                         }
                     } else {
-#pragma unroll
-                        for (int j = 0; j < WP; ++j) c += __popc(pw[j] & (SMEM ? ru[j] : __ldg(ru + j)));
+                        for (unsigned j = 0; j < sw; ++j) c += (unsigned)__popc(pw[j] & (SMEM ? ru[j] : __ldg(ru + j)));
                     }
-                    const unsigned key = ((unsigned)(c + 1) << 16) | (0xffffu - u);
+                    const unsigned key = ((c + 1u) << 16) | (0xffffu - u);
                     best = key > best ? key : best;
                 }
             }
-            if (G > 1) {
-#pragma unroll
-                for (int o = G / 2; o > 0; o >>= 1) {
-                    const unsigned y = __shfl_xor_sync(FULL, best, o);
-                    best = y > best ? y : best;
-                }
-            }
+            best = __reduce_max_sync(FULL, best);
             __syncwarp();
-            pc = best ? (int)(0xffffu - (best & 0xffffu)) : ((PIVOT == MCE_PIVOT_GREEDY_TX) ? fp : -1);
-        } else {
-            // argmax |P' n N(u)| over X' (TX) or P' u X' (TomitaBB); scanning
-            // candidates in increasing position with '>' keeps the earliest
-            uint32_t cand[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) cand[k] = (PIVOT == MCE_PIVOT_GREEDY_TX) ? (bx ? Xc[k] : 0u) : (Pc[k] | Xc[k]);
-            if (!inter) {
-#pragma unroll
-                for (int k = 0; k < K; ++k) cand[k] = 0u;
-            }
-            int best = -1;
-            pc = (PIVOT == MCE_PIVOT_GREEDY_TX) ? fp : -1;  // X' empty: first of P'
-            // GreedyBBNX (the TX kernel with pivot_mode NX): Naude's early exit.
-            // A candidate's count is one group-wide popcount here, so the
-            // exit is at candidate level: once a candidate covers all of P'
-            // (|P' n K(u)| = 0), no later one can beat it and the scan stops.
-            const bool nx = PIVOT == MCE_PIVOT_GREEDY_TX && prm.pivot_mode == MCE_PIVOT_GREEDY_NX;
-            int npc = 0;
-            if (nx) {
-#pragma unroll
-                for (int k = 0; k < K; ++k) npc += __popc(Pc[k]);
-                npc = g.sum(npc);
-            }
-            for (;;) {
-                uint32_t o = 0;
-#pragma unroll
-                for (int k = 0; k < K; ++k) o |= cand[k];
-                if (__ballot_sync(FULL, o != 0u) == 0u) break;
-                const int u = g.first(cand);
-                uint32_t r[K];
-#pragma unroll
-                for (int k = 0; k < K; ++k) r[k] = 0u;
-                if (u >= 0) load_row<K, SMEM>(r, rowp(u));
-                int cnt = 0;
-#pragma unroll
-                for (int k = 0; k < K; ++k) cnt += __popc(Pc[k] & r[k]);
-                cnt = g.sum(cnt);
-                if (u >= 0) {
-                    if (cnt > best) {
-                        best = cnt;
-                        pc = u;
-                    }
-                    g.clear(cand, u);
-                    if (nx && best == npc) {
-#pragma unroll
-                        for (int k = 0; k < K; ++k) cand[k] = 0u;
-                    }
-                }
-            }
+            pc = 0xffffu - (best & 0xffffu);
         }
-
         uint32_t Lc[K];
+        unsigned u = 0;
+        get_row(r, pc);
 #pragma unroll
-        for (int k = 0; k < K; ++k) Lc[k] = 0u;
-        if (inter) {
-            uint32_t r[K];
-            load_row<K, SMEM>(r, rowp(pc));
-#pragma unroll
-            for (int k = 0; k < K; ++k) Lc[k] = Pc[k] & ~r[k];  // L' = P' \ N(p)
+        for (int k = 0; k < K; ++k) {
+            Lc[k] = Pc[k] & ~r[k];  // L' = P' \ N(p)
+            u += (unsigned)__popc(Pc[k] | Xc[k]);
         }
-        bool hasLc, more;
-        g.any2(Lc, L, hasLc, more);
-        bool desc = inter && hasLc;
-        if (T2 && t2p != 0u) {
-            // a child whose P' u X' has at most 32 vertices and whose P' is
-            // small enough goes to a free lane of the warp instead
-            int cu = 0;
-#pragma unroll
-            for (int k = 0; k < K; ++k) cu += (__popc(Pc[k] | Xc[k]) << 16) | __popc(Pc[k]);
-            cu = g.sum(cu);
-            const bool comp = desc && (cu >> 16) <= 32 && (unsigned)(cu & 0xffff) <= t2p;
-            if (__ballot_sync(FULL, comp) != 0u) {
-                if (t2_take(comp, Pc, Xc, Lc, rs + 1u, Sc)) desc = false;
-            }
+        const unsigned c = __reduce_add_sync(FULL, set_count<K>(Lc));
+        if (c == 0u) continue;
+        const unsigned pu = __reduce_add_sync(FULL, (set_count<K>(Pc) << 16) | u);
+        if (pool_fits(pu >> 16, pu & 0xffffu, c)) {
+            pool_take(Pc, Xc, c, pu & 0xffffu, pc, rs + 1u, Sc);
+            continue;
         }
         // Breadth-first split of the top of the tree: a new subtree with a
-        // large candidate set goes to the global ring (while the ring is short
-        // of frames; gq is the same in every lane) instead of being descended
-        // into here.
-        const bool split_open = gq < prm.split_target;  // warp-uniform
-        const bool try_split = desc && split_open;
-        bool any_split = false;
-        if (split_open) any_split = __ballot_sync(FULL, try_split) != 0u;
-        if (any_split) {
-            int cp = 0;
-#pragma unroll
-            for (int k = 0; k < K; ++k) cp += __popc(Pc[k]);
-            const int np = g.sum(cp);
-            const bool sp = try_split && (unsigned)np >= th.split;
-            uint32_t sR[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) sR[k] = 0u;
-            if (list && sp) r_bits(rs, v, sR);
-            const bool pushed = push_global<G, K>(g, prm, sp, Pc, Xc, (unsigned)pc | (n << 16), rs + 1u, Sc, list, sR, cn);
-            if (pushed) {
-                desc = false;
-                if (g.leader()) cn.note(kDiagDonations);
-            }
-        }
-        bool spill = false;
-        if (desc && more) {
-            if (d < (int)prm.stack_levels) {
-                stk.put(d, g.gl, P, X, pe, rs, S);
-                ++d;
-            } else {
-                spill = true;
-            }
-        }
-        if (__ballot_sync(FULL, spill) != 0u) {
-            // stack full: the rest of this frame (L is non-empty) goes to the
-            // global ring as it stands, and the group descends without it
-            uint32_t sR[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) sR[k] = 0u;
-            if (list && spill) r_bits(rs, -1, sR);
-            const bool pushed = push_global<G, K>(g, prm, spill, P, X, pe, rs, S, list, sR, cn);
-            if (pushed && g.leader()) cn.note(kDiagDonations);
-            if (spill && !pushed && g.leader()) set_status(prm.out, ctl, MCE_EOVERFLOW);
-        }
-        lempty = (act && !desc && !more) || (work && v < 0);
-        if (desc) {
+        // large candidate set goes to the device-wide ring (while that is
+        // short of frames) instead of being descended into here.  With the
+        // stack full, the rest of this frame (L is non-empty) goes there as it
+        // stands, and the warp descends without it.
+        const bool split = open && (pu >> 16) >= th.split;
+        const bool spill = !split && !lempty && d >= (int)prm.stack_levels;
+        if (split || spill) {
+            uint32_t fP[K], fX[K], fR[K];
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                P[k] = Pc[k];
-                X[k] = Xc[k];
-                L[k] = Lc[k];
+                fP[k] = split ? Pc[k] : P[k];
+                fX[k] = split ? Xc[k] : X[k];
+                fR[k] = 0u;
             }
-            if (list) prm.lst.path[(size_t)gidx * n + rs] = (uint16_t)v;  // R grows by v at |R| = rs
-            pe = (unsigned)pc | (n << 16);
-            rs = rs + 1u;
-            S = Sc;
+            unsigned ticket;
+            const bool got = reserve(false, ticket);
+            if (got) {
+                if (LIST) r_bits(rs, split ? v : -1, fR);
+                publish(false, ticket, fP, fX, split ? (pc | (n << 16)) : pe, split ? rs + 1u : rs, split ? Sc : S, fR);
+            }
+            if (got && split) continue;
+            if (!got && !lempty && d >= (int)prm.stack_levels && lane == 0) set_status(prm.out, ctl, MCE_EOVERFLOW);
+            if (!got && !lempty && d >= (int)prm.stack_levels) lempty = true;
         }
+        if (!lempty && !spill) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                stack[d][k] = P[k];
+                stack[d][K + k] = X[k];
+            }
+            stack[d][2 * K] = scalars();
+            ++d;
+        }
+        if (LIST && lane == 0) prm.lst.path[(size_t)gidx * n + rs] = (uint16_t)v;  // R grows by v at |R| = rs
+        if (LIST) __syncwarp();
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            P[k] = Pc[k];
+            X[k] = Xc[k];
+            L[k] = Lc[k];
+        }
+        pe = pc | (n << 16);
+        rs = rs + 1u;
+        S = Sc;
+        lempty = false;
     }
-    if (list && g.leader() && cend)  // retire the last chunk
+    if (LIST && lane == 0 && cend)  // retire the last chunk
         prm.lst.fill[cend / prm.lst.chunk_words - 1u] = cpos - (cend - prm.lst.chunk_words);
 }
 
-template <int G, int K, bool SMEM, int PIVOT, bool LIST>
-__global__ void __launch_bounds__(512) search_kernel(const SearchParams prm)
+// Direct layout (n <= 128): rows of `cls` words (stride 4 for three), hash
+// terms and positions of the whole graph, once per block, in the order the
+// warp tier reads them.  Whole block; a barrier must follow.
+__device__ __forceinline__ void direct_layout(const uint32_t *rows, uint32_t rw, const uint32_t *order, uint32_t n,
+                                              unsigned cls, uint32_t *drows, uint64_t *dhash, uint16_t *dpos)
 {
-    constexpr int WP = G * K;
+    const unsigned stride = cls == 3u ? 4u : cls;
+    for (unsigned i = threadIdx.x; i < n * stride; i += blockDim.x) {
+        const unsigned v = i / stride, w = i % stride;
+        drows[i] = w < rw && w < cls ? rows[(size_t)v * rw + w] : 0u;
+    }
+    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+        dhash[i] = mix64((uint64_t)order[i] + 1u);
+        dpos[i] = (uint16_t)i;
+    }
+}
+
+template <int K, bool SMEM, int PIVOT, bool LIST>
+__global__ void __launch_bounds__(kLaunchThreads) search_kernel(const SearchParams prm)
+{
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t mbar;
 
     const uint32_t n = prm.n;
-    const size_t rbytes = smem_rows_bytes(n, WP, SMEM);
+    const size_t rbytes = smem_rows_bytes(n, prm.wp, SMEM);
     uint32_t *srows = reinterpret_cast<uint32_t *>(smem_raw);
-    uint64_t *hv = reinterpret_cast<uint64_t *>(smem_raw + rbytes);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(hv + n);
-    const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n, WP, SMEM), WP, prm.local_slots);
-    local_queue_reset(lq, (blockDim.x / 32u) * (32u / G));
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + rbytes);
+    const uint32_t lq_off = (uint32_t)smem_local_offset(n, prm.wp, SMEM);
+    const LocalQ lq = local_queue_at(smem_raw + lq_off, prm.wp, prm.local_slots);
+    local_queue_reset(lq, blockDim.x / 32u);
 
-    // ---- prologue: stage the rows (bulk copy), hash terms, histogram
+    // ---- prologue: stage the rows (bulk copy), histogram
     if (SMEM) {
         if (threadIdx.x == 0) mbar_init(&mbar);
         __syncthreads();
     }
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) hv[i] = mix64((uint64_t)prm.order[i] + 1u);
+#pragma unroll 1
     for (uint32_t i = threadIdx.x; i <= n; i += blockDim.x) hist[i] = 0u;
     bool staged = true;
     if (SMEM) staged = stage_rows(srows, prm.rows, (uint32_t)rbytes, (uint32_t)__cvta_generic_to_shared(&mbar), 0u);
     if (!staged && threadIdx.x == 0) set_status(prm.out, prm.ctl, MCE_ETIMEOUT);
+    const Thresholds th = density_thresholds(prm.ctl->pad3[0], n, prm.tune, prm.split_min_p);
+    const uint32_t *rows = SMEM ? srows : prm.rows;
+    const bool direct = !LIST && K == 1 && n <= 128u && prm.t2_max_p != 0u;
+    PoolAt at{};
+    at.rows = prm.direct_offset;
+    at.hash = at.rows + kDirectRows * 4;
+    at.pos = at.hash + kDirectVerts * 8;
+    at.region = prm.t2_offset + (threadIdx.x >> 5) * prm.pool_bytes;
+    at.lq = lq_off;
+    at.hist = (uint32_t)rbytes;
     const bool ok = __syncthreads_and(staged) != 0;
-
-    __shared__ unsigned deg_sum;
-    const Thresholds th = density_thresholds(SMEM ? srows : prm.rows, n, WP, prm.tune.share_local,
-                                             prm.tune.share_global, prm.split_min_p, &deg_sum,
-                                             prm.tune.small_split != 0u);
-    uint32_t *stack_smem = reinterpret_cast<uint32_t *>(smem_raw + prm.stack_offset);
+    if (direct && ok)
+        direct_layout(rows, prm.wp, prm.order, n, th.cls, reinterpret_cast<uint32_t *>(smem_raw + at.rows),
+                      reinterpret_cast<uint64_t *>(smem_raw + at.hash), reinterpret_cast<uint16_t *>(smem_raw + at.pos));
     Counters cn;
     cn.diag = lq.h->diag;
-    if (ok)
-        search_loop<G, K, SMEM, PIVOT, LIST>(prm, SMEM ? srows : prm.rows, hv, hist, lq, th, stack_smem,
-                                       (int)prm.stack_smem_levels, smem_raw + prm.t2_offset, cn);
+    if (ok) search_loop<K, SMEM, PIVOT, LIST>(prm, rows, hist, lq, th, at, direct, cn);
     flush_counters(cn, prm.out);
     __syncthreads();
     if (threadIdx.x == 0) flush_diag(lq.h->diag, prm.out);
+#pragma unroll 1
     for (uint32_t i = threadIdx.x; i <= n; i += blockDim.x)
         if (hist[i]) atomicAdd(reinterpret_cast<unsigned long long *>(prm.out + MCE_OUT_HIST + i), (unsigned long long)hist[i]);
 }
@@ -1950,10 +2121,9 @@ __global__ void __launch_bounds__(512) search_kernel(const SearchParams prm)
 // Per graph: output initialised with the root counted (status kept), rows
 // bulk-copied to shared memory, root frame queued, search, reduction into the
 // graph's own result array.
-template <int G, int K, bool SMEM, int PIVOT>
-__global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
+template <int K, bool SMEM, int PIVOT>
+__global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams bp)
 {
-    constexpr int WP = G * K;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t mbar;
     __shared__ unsigned cur, root_key;
@@ -1978,13 +2148,12 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         // the root's children t = part, part + parts, ... (independent
         // subtrees; the root node is counted by part 0)
         const unsigned item = bp.list[idx];
-        const unsigned part = (item >> 16) & 0xffu, parts = item >> 24;
+        const unsigned part = (item >> 16) & 0xffu, parts = max(item >> 24, 1u);
         const BatchGraph gd = bp.graphs[item & 0xffffu];
-        const uint32_t n = gd.n;
+        const uint32_t n = gd.n, WP = gd.wp;
         const size_t rbytes = smem_rows_bytes(n, WP, SMEM);
         uint32_t *srows = reinterpret_cast<uint32_t *>(smem_raw);
-        uint64_t *hv = reinterpret_cast<uint64_t *>(smem_raw + rbytes);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(hv + n);
+        uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + rbytes);
         const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n, WP, SMEM), WP);
         local_queue_reset(lq, bp.groups_per_block);
         const bool valid = gd.out[MCE_OUT_STATUS] == 0ull;
@@ -1993,7 +2162,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         // through the order, with R = {rv} already chosen.
         const bool sub = gd.root != nullptr;
         bool pne = false, xne = false;
-        for (uint32_t w = threadIdx.x; w < (uint32_t)WP; w += blockDim.x) {
+        for (uint32_t w = threadIdx.x; w < WP; w += blockDim.x) {
             uint32_t pw = 0u, xw = 0u;
             if (!sub) {
                 const uint32_t base = w * 32u;
@@ -2019,7 +2188,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         // the root is one node: internal, a leaf (R is maximal) or a dead end;
         // the graph's result array starts zeroed (cleared with the batch) and
         // every part adds to it
-        const bool split = parts >= 2u && !sub;
+        const bool split = !sub;  // every graph but an outer-loop subproblem starts from its root's children
         if (threadIdx.x == 0 && (!split || part == 0u)) {
             unsigned long long *o = reinterpret_cast<unsigned long long *>(gd.out);
             atomicAdd(o + MCE_OUT_NODES, 1ull);
@@ -2032,8 +2201,14 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
                 atomicMax(o + MCE_OUT_MAX_SIZE, (unsigned long long)r0);
             }
         }
-        for (uint32_t j = threadIdx.x; j < n; j += blockDim.x)
-            hv[j] = mix64((uint64_t)(sub ? gd.label[gd.order[j]] : gd.order[j]) + 1u);
+        // (a subproblem's order becomes the original labels: the search reads
+        // it for the hash terms alone)
+        if (sub) {
+            __syncthreads();
+#pragma unroll 1
+            for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) gd.order[j] = gd.label[gd.order[j]];
+        }
+#pragma unroll 1
         for (uint32_t j = threadIdx.x; j <= n; j += blockDim.x) hist[j] = 0u;
 
         // ChoosePivotOrdered at the root: the key (score + 1) << 12 | (4095 -
@@ -2051,7 +2226,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
                 if (!cand) continue;
                 unsigned score = 0;
                 if (PIVOT == MCE_PIVOT_TOMITA || (PIVOT == MCE_PIVOT_GREEDY_TX && xne))
-                    for (uint32_t w = 0; w < (uint32_t)WP; ++w)
+                    for (uint32_t w = 0; w < WP; ++w)
                         score += __popc(frames[kFrameHdr + w] & gd.ren[(size_t)u * WP + w]);
                 const unsigned key = ((score + 1u) << 12) | (4095u - u);
                 mine = key > mine ? key : mine;
@@ -2065,7 +2240,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         const unsigned p0 = root_key ? (4095u - (root_key & 4095u)) : 0u;
         bool lne = false;
         if (pne)
-            for (uint32_t w = threadIdx.x; w < (uint32_t)WP; w += blockDim.x)
+            for (uint32_t w = threadIdx.x; w < WP; w += blockDim.x)
                 lne = lne || (frames[kFrameHdr + w] & ~gd.ren[(size_t)p0 * WP + w]) != 0u;
         lne = __syncthreads_or(lne) != 0;
         const bool root = valid && pne && lne;
@@ -2080,7 +2255,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
             const uint32_t *rp0 = gd.ren + (size_t)p0 * WP;
             if (threadIdx.x == 0) {
                 unsigned acc = 0;
-                for (uint32_t w = 0; w < (uint32_t)WP; ++w) {
+                for (uint32_t w = 0; w < WP; ++w) {
                     lpre[w] = acc;
                     acc += (unsigned)__popc(frames[kFrameHdr + w] & ~rp0[w]);
                 }
@@ -2092,12 +2267,12 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
             for (unsigned j = threadIdx.x; j < mine && j + 1u < bp.qcap; j += blockDim.x) {
                 const unsigned t = part + j * parts;
                 unsigned w = 0;
-                while (w + 1u < (unsigned)WP && lpre[w + 1] <= t) ++w;
+                while (w + 1u < WP && lpre[w + 1] <= t) ++w;
                 uint32_t lw = frames[kFrameHdr + w] & ~rp0[w];
                 for (unsigned r = t - lpre[w]; r > 0u; --r) lw &= lw - 1u;
                 const unsigned v = w * 32u + (unsigned)(__ffs(lw) - 1);
                 uint32_t *fr = frames + (size_t)(j + 1u) * bp.fs;
-                for (uint32_t q = 0; q < (uint32_t)WP; ++q) {
+                for (uint32_t q = 0; q < WP; ++q) {
                     const uint32_t pw = frames[kFrameHdr + q];
                     uint32_t below = 0u;
                     if (v >= q * 32u + 32u) below = FULL;
@@ -2150,6 +2325,7 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         const bool ok = __syncthreads_and(staged) != 0;
 
         SearchParams prm;
+        prm = SearchParams{};
         prm.n = n;
         prm.wp = WP;
         prm.rows = gd.ren;
@@ -2166,29 +2342,37 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
         prm.stack_levels = bp.stack_levels;
         prm.split_min_p = bp.split_min_p;
         prm.split_target = bp.split_target;
-        prm.stack_smem_levels = bp.stack_smem_levels;
-        prm.stack_offset = bp.stack_offset;
-        prm.trace = nullptr;
-        prm.trace_per_block = 0;
         prm.tune = bp.tune;
-        prm.lst = ListParams{};
-        prm.part = nullptr;
-        prm.part_k = 0;
         prm.count_root = 1;
-        prm.seed_children = 0;
         prm.local_slots = kLocalSlots;
         prm.t2_offset = bp.t2_offset;
-        prm.t2_levels = bp.t2_levels;
+        prm.pool_bytes = bp.pool_bytes;
         prm.t2_max_p = bp.t2_max_p;
-        const Thresholds th = density_thresholds(SMEM ? srows : gd.ren, n, WP, bp.tune.share_local,
-                                                 bp.tune.share_global, bp.split_min_p, &root_key,
-                                                 bp.tune.small_split != 0u);
+        prm.direct_offset = bp.direct_offset;
+        const uint32_t *rows = SMEM ? srows : gd.ren;
+        if (threadIdx.x == 0) root_key = 0u;
+        __syncthreads();
+        {
+            unsigned mine = 0;
+            for (uint32_t i = threadIdx.x; i < n * WP; i += blockDim.x) mine += (unsigned)__popc(rows[i]);
+            atomicAdd(&root_key, mine);
+        }
+        __syncthreads();
+        const Thresholds th = density_thresholds(root_key, n, bp.tune, bp.split_min_p, bp.cls);
+        const bool direct = K == 1 && n <= 128u && bp.t2_max_p != 0u;
+        PoolAt at{};
+        at.rows = bp.direct_offset;
+        at.hash = at.rows + kDirectRows * 4;
+        at.pos = at.hash + kDirectVerts * 8;
+        at.region = bp.t2_offset + (threadIdx.x >> 5) * bp.pool_bytes;
+        at.lq = (uint32_t)smem_local_offset(n, WP, SMEM);
+        at.hist = (uint32_t)rbytes;
+        if (direct)
+            direct_layout(rows, WP, gd.order, n, th.cls, reinterpret_cast<uint32_t *>(smem_raw + at.rows),
+                          reinterpret_cast<uint64_t *>(smem_raw + at.hash), reinterpret_cast<uint16_t *>(smem_raw + at.pos));
         Counters cn;
         cn.diag = lq.h->diag;
-        if (ok)
-            search_loop<G, K, SMEM, PIVOT, false>(prm, SMEM ? srows : gd.ren, hv, hist, lq, th,
-                                           reinterpret_cast<uint32_t *>(smem_raw + bp.stack_offset),
-                                           (int)bp.stack_smem_levels, smem_raw + bp.t2_offset, cn);
+        if (ok) search_loop<K, SMEM, PIVOT, false>(prm, rows, hist, lq, th, at, direct, cn);
         flush_counters(cn, gd.out);
         __syncthreads();
         if (threadIdx.x == 0) flush_diag(lq.h->diag, gd.out);
@@ -2198,28 +2382,20 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchParams bp)
     }
 }
 
-// Root of Alg. 4 (P = V, X = R = {}) as the first queued frame, empty queue
-// otherwise, and the result array with the root already counted: one node,
-// internal when n > 0; for n = 0 the root is a leaf and the empty set is the
-// one maximal clique.  A non-zero status left by an earlier step (invalid
-// input) suppresses the root frame, so the search returns at once.
-// root_pivot (device, nullable = position 0) is the
-// root's pivot: with X empty every rule but TomitaBB takes the first vertex.
-template <int G, int K>
-__global__ void search_init_kernel(const SearchParams prm, const unsigned *root_pivot)
+// The result array with the root already counted: one node, internal when
+// n > 0; for n = 0 the root is a leaf and the empty set is the one maximal
+// clique; and an empty queue (the kernel that follows queues the root's
+// children, or a part of them).  A part counts the root only when asked to.
+// A non-zero status left by an earlier step (invalid input) suppresses the
+// frames, so the search returns at once.
+template <int D = 0>
+__global__ void search_init_kernel(const SearchParams prm)
 {
-    constexpr int WP = G * K;
     const uint32_t n = prm.n;
     const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned nth = gridDim.x * blockDim.x;
-    // a part of the root's branching queues part_k child frames (written by
-    // the part-frames kernel that follows) and counts the root only when
-    // asked to
     const bool part = prm.part != nullptr;
-    // seeded: the root's children are queued by the seeding kernel that
-    // follows, so the queue starts empty here
-    const bool seeded = part || prm.seed_children;
-    const unsigned queued = part ? prm.part_k : (prm.seed_children ? 0u : (n > 0u ? 1u : 0u));
+    const unsigned queued = part ? prm.part_k : 0u;
     const bool root = !part || prm.count_root;
     for (unsigned i = tid; i < prm.qcap; i += nth) prm.seq[i] = i < queued ? i + 1u : i;
     for (unsigned i = tid; i < MCE_OUT_WORDS(n); i += nth) {
@@ -2232,46 +2408,15 @@ __global__ void search_init_kernel(const SearchParams prm, const unsigned *root_
         if (i == MCE_OUT_GROUPS) v = prm.total_groups;
         prm.out[i] = v;
     }
-    if (seeded) {
-        if (tid == 0) {
-            Ctl *c = prm.ctl;
-            c->head = 0u;
-            c->abort = 0u;
-            const bool go = queued > 0u && prm.out[MCE_OUT_STATUS] == 0ull;
-            c->tail = go ? queued : 0u;
-            c->pending = go ? queued : 0u;
-            c->starving = 0u;
-        }
-        return;
-    }
-    if (n > 0u) {
-        for (unsigned w = tid; w < (unsigned)WP; w += nth) {
-            const unsigned base = w * 32u;
-            uint32_t pw = 0u;
-            if (n >= base + 32u) pw = FULL;
-            else if (n > base) pw = (1u << (n - base)) - 1u;
-            prm.frames[kFrameHdr + w] = pw;       // P = V
-            prm.frames[kFrameHdr + WP + w] = 0u;  // X = {}
-            if (prm.lst.rec) prm.frames[kFrameHdr + 2 * WP + w] = 0u;  // R = {}
-        }
-    }
     if (tid == 0) {
         Ctl *c = prm.ctl;
         c->head = 0u;
         c->abort = 0u;
-        if (n > 0u && prm.out[MCE_OUT_STATUS] == 0ull) {
-            const unsigned p0 = root_pivot ? *root_pivot : 0u;
-            prm.frames[0] = (p0 & 0xffffu) | (n << 16);
-            prm.frames[1] = 0u;
-            prm.frames[2] = 0u;
-            prm.frames[3] = 0u;
-            c->tail = 1u;
-            c->pending = 1u;
-        } else {
-            c->tail = 0u;
-            c->pending = 0u;
-        }
-        c->starving = 0u;
+        const bool go = queued > 0u && prm.out[MCE_OUT_STATUS] == 0ull;
+        c->tail = go ? queued : 0u;
+        c->pending = go ? queued : 0u;
+        c->starving = prm.total_groups;  // warps without a frame: all of them
+        c->pad3[0] = 0u;                 // degree sum, added by the kernel that follows
     }
 }
 

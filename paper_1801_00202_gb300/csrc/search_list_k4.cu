@@ -1,0 +1,3 @@
+// Clique-listing search kernels with 4 word(s) of every set per lane.
+#include "search_inst.cuh"
+MCE_DEFINE_SEARCH_LIST(4)

@@ -56,6 +56,16 @@ __device__ int select_child(const uint32_t *rows, uint32_t n, uint32_t wp, uint3
     return -1;
 }
 
+// Adds |N(v)| to the search's degree sum, which the search kernel reads its
+// density thresholds from (whole warps; every warp adds its share of the row).
+__device__ __forceinline__ void add_degree(const SearchParams &prm, uint32_t v)
+{
+    unsigned c = 0;
+    for (uint32_t w = threadIdx.x; w < prm.wp; w += blockDim.x) c += (unsigned)__popc(prm.rows[(size_t)v * prm.wp + w]);
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31u) == 0u && c != 0u) atomicAdd(&prm.ctl->pad3[0], c);
+}
+
 __global__ void root_children_kernel(const uint32_t *rows, uint32_t n, uint32_t wp, const unsigned *root_pivot,
                                      uint32_t *sizes, uint32_t cap, uint32_t *count)
 {
@@ -86,6 +96,7 @@ __global__ void part_frames_kernel(const SearchParams prm, const unsigned *root_
     __shared__ int v;
     const uint32_t j = blockIdx.x;
     const uint32_t n = prm.n, wp = prm.wp;
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) add_degree(prm, i);
     const uint32_t p0 = root_pivot ? *root_pivot : 0u;
     if (threadIdx.x == 0) {
         const uint32_t t = prm.part[j];
@@ -125,6 +136,7 @@ __global__ void seed_children_kernel(const SearchParams prm, const unsigned *roo
     const uint32_t n = prm.n, wp = prm.wp;
     const uint32_t p0 = root_pivot ? *root_pivot : 0u;
     const uint32_t *rp = prm.rows + (size_t)p0 * wp;
+    add_degree(prm, t);
     if (threadIdx.x == 0) {
         uint32_t cnt = 0;
         for (uint32_t w = 0; w * 32u < n; ++w) cnt += (uint32_t)__popc(valid_bits(w, n) & ~rp[w]);
