@@ -1860,7 +1860,7 @@ int enumerate_outer(mce_graph *g, const mce_options &o, mce_result *res, std::ch
     rc = dalloc(ctx, (void **)&d_ord, ((size_t)n * 2 + 64) * 4, s);
     if (rc != MCE_OK) return rc;
     uint32_t *d_pos = d_ord + n + 32;
-    e = outer_degeneracy(n, g->d_off, g->d_adj, d_ord, d_pos, s);
+    e = outer_degeneracy(n, off[n], g->d_off, g->d_adj, d_ord, d_pos, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(order.data(), d_ord, (size_t)n * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
