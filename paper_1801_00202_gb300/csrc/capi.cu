@@ -1184,10 +1184,16 @@ int list_deliver(mce_ctx *ctx, uint32_t n, const ListArea &la, const uint32_t *d
     return e == cudaSuccess ? MCE_OK : MCE_ECUDA;
 }
 
-int enumerate_once(mce_graph *g, const mce_options &o, mce_result *res, std::chrono::steady_clock::time_point t0,
+int enumerate_once(mce_graph *g, const mce_options &opts, mce_result *res, std::chrono::steady_clock::time_point t0,
                    const uint32_t *children, uint32_t k, uint32_t count_root, const Sink *sink)
 {
     mce_ctx *ctx = g->ctx;
+    mce_options o = opts;
+    // A listing without room for a single offset fits no result: the call
+    // asks for the sizes, which the counting search gives (G(700, 0.3), three
+    // million cliques: 1.3 ms against the listing search's 4.5).
+    const bool sizes_only = (o.flags & kListFlags) != 0u && !sink && (!res->list_off || res->list_off_cap == 0);
+    if (sizes_only) o.flags &= ~kListFlags;
     const bool listing = (o.flags & kListFlags) != 0u;
     Config c;
     int rc = choose(g->n, o, c);
@@ -1236,6 +1242,11 @@ int enumerate_once(mce_graph *g, const mce_options &o, mce_result *res, std::chr
             const uint32_t *d_order = reinterpret_cast<const uint32_t *>(static_cast<unsigned char *>(scr) + L.order);
             rc = list_deliver(ctx, g->n, la, d_order, h, (o.flags & MCE_LIST_SORTED) != 0u, res, ctx->stream,
                               sink ? *sink : Sink{});
+        }
+        if (sizes_only && rc == MCE_OK) {
+            res->list_ids_needed = 0;
+            for (uint32_t j = 0; j <= g->n; ++j) res->list_ids_needed += (uint64_t)j * h[MCE_OUT_HIST + j];
+            rc = MCE_ETRUNC;
         }
     }
     if (la.mem) dfree(ctx, la.mem, la.bytes, ctx->stream);
