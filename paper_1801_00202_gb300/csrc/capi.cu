@@ -475,6 +475,13 @@ int enumerate_device_impl(uint32_t n, uint32_t words_per_row, const uint32_t *d_
 {
     uint32_t *order = reinterpret_cast<uint32_t *>(scr + L.order);
     uint32_t *rows = reinterpret_cast<uint32_t *>(scr + L.rows);
+    if (!part && !(o.flags & MCE_ORDER_IDENTITY) && small_prep_fits(n, words_per_row, c.wp)) {
+        SearchParams p = params(n, c, L, scr, rows, order, d_out, o, lp);
+        p.prepared = 1u;
+        const cudaError_t e = launch_small_prep(p, words_per_row, d_rows, order, rows, s);
+        if (e != cudaSuccess) return cuda_code(e);
+        return cuda_code(c.impl.run(p, LaunchShape{c.blocks, c.threads, c.smem_bytes, c.smem}, s));
+    }
     cudaError_t e = cudaMemsetAsync(d_out + MCE_OUT_STATUS, 0, sizeof(uint64_t), s);
     if (e == cudaSuccess) e = launch_validate_rows(n, words_per_row, d_rows, d_out, s);
     if (e == cudaSuccess)

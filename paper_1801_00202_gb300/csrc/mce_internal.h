@@ -166,6 +166,7 @@ struct SearchParams {
     uint32_t t2_offset, pool_bytes, t2_max_p;
     uint32_t direct_offset;  // byte offset of the whole-graph layout (n <= 128)
     uint32_t local_slots;   // slots of the block ring (kLocalSlots or kLocalSlotsSmall)
+    uint32_t prepared;      // result array, queue and root frames are in place: the search alone is launched
 };
 
 // One graph of a batch (device table entry; pointers into library memory).
@@ -274,6 +275,12 @@ cudaError_t launch_root_children(const uint32_t *rows, uint32_t n, uint32_t wp, 
 cudaError_t launch_part_frames(const SearchParams &prm, const unsigned *root_pivot, cudaStream_t s);
 // Queue every root child as its own frame (after search_init_kernel left the
 // queue empty): frame t in slot t, tail = pending = |L|.  prm.qcap >= n.
+// Everything before the search (see small_prep_kernel), for graphs and rows
+// that small_prep_fits accepts: order and rows receive the order and the
+// renumbered rows.
+bool small_prep_fits(uint32_t n, uint32_t w, uint32_t wp);
+cudaError_t launch_small_prep(const SearchParams &prm, uint32_t w, const uint32_t *rows_in, uint32_t *order,
+                              uint32_t *rows, cudaStream_t s);
 cudaError_t launch_seed_children(const SearchParams &prm, const unsigned *root_pivot, cudaStream_t s);
 // TomitaBB's root pivot (the earliest vertex of maximum degree) to *dst.
 cudaError_t launch_root_degree_pivot(const uint32_t *rows, uint32_t n, uint32_t wp, unsigned *dst, cudaStream_t s);

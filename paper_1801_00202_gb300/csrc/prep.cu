@@ -39,28 +39,34 @@ __global__ void edges_kernel(uint32_t n, uint64_t m, const uint32_t *__restrict_
     }
 }
 
-// Bitset checks: zero diagonal, zero bits at positions >= n, symmetry.
+// Bitset checks of one word: zero diagonal, zero bits at positions >= n,
+// symmetry.
+__device__ __forceinline__ bool valid_word(uint32_t n, uint32_t w, const uint32_t *rows, uint64_t idx)
+{
+    const uint32_t i = (uint32_t)(idx / w), j = (uint32_t)(idx % w);
+    uint32_t word = rows[idx];
+    if (word == 0u) return true;
+    const uint32_t base = j * 32u;
+    uint32_t valid = FULLM;
+    if (base >= n) valid = 0u;
+    else if (n - base < 32u) valid = (1u << (n - base)) - 1u;
+    if (word & ~valid) return false;
+    if (i >= base && i < base + 32u && ((word >> (i - base)) & 1u)) return false;
+    while (word) {
+        const uint32_t b = (uint32_t)__ffs(word) - 1u;
+        word &= word - 1u;
+        const uint32_t u = base + b;
+        if (!((rows[(size_t)u * w + (i >> 5)] >> (i & 31)) & 1u)) return false;
+    }
+    return true;
+}
+
 __global__ void validate_kernel(uint32_t n, uint32_t w, const uint32_t *__restrict__ rows, uint64_t *out)
 {
     const uint64_t total = (uint64_t)n * w;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride) {
-        const uint32_t i = (uint32_t)(idx / w), j = (uint32_t)(idx % w);
-        uint32_t word = rows[idx];
-        if (word == 0u) continue;
-        const uint32_t base = j * 32u;
-        uint32_t valid = FULLM;
-        if (base >= n) valid = 0u;
-        else if (n - base < 32u) valid = (1u << (n - base)) - 1u;
-        if (word & ~valid) { flag_invalid(out); continue; }
-        if (i >= base && i < base + 32u && ((word >> (i - base)) & 1u)) { flag_invalid(out); continue; }
-        while (word) {
-            const uint32_t b = (uint32_t)__ffs(word) - 1u;
-            word &= word - 1u;
-            const uint32_t u = base + b;
-            if (!((rows[(size_t)u * w + (i >> 5)] >> (i & 31)) & 1u)) { flag_invalid(out); break; }
-        }
-    }
+    for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride)
+        if (!valid_word(n, w, rows, idx)) flag_invalid(out);
 }
 
 // Maximum-degree-first order (Section 4.2) by one block of T threads: highest
@@ -85,6 +91,7 @@ __global__ void validate_kernel(uint32_t n, uint32_t w, const uint32_t *__restri
 // brackets): n = 100 24 us (16), 300 85 (57), 500 146 (121), 1000 383 (253),
 // 3000 4345 (756; rows in L2, two dependent reads a round).
 constexpr unsigned kOrderCand = 128;
+constexpr unsigned kSmallPrepThreads = 256, kSmallPrepVerts = 128, kSmallPrepWords = 4;
 
 struct OrderShared {
     uint32_t adj[kOrderCand][4];   // adjacency among the candidates
@@ -336,6 +343,101 @@ __global__ void __launch_bounds__(T) order_kernel(uint32_t n, uint32_t w, const 
     order_block<T>(n, w, rows, order, rows_in_smem != 0, osm);
 }
 
+// Everything before the search of a graph of at most 128 vertices, by one
+// block: validation, the order, the renumbered rows, the result array and the
+// queue as the search starts from them (the root counted, its children's
+// frames queued; nothing queued for rows that are not a simple graph's).  As
+// separate launches these were seven short kernels in a row, some 20 us of
+// launch gaps and of global memory written and read back: G(45, 0.5) 62 us
+// from rows to result, now 50; G(100, 0.5) 145 and 137.  TomitaBB's root
+// pivot is position 0, too: the order's first vertex has the largest degree.
+__global__ void __launch_bounds__(kSmallPrepThreads) small_prep_kernel(const SearchParams prm, uint32_t w,
+                                                                       const uint32_t *__restrict__ rows_in,
+                                                                       uint32_t *order, uint32_t *rows)
+{
+    extern __shared__ __align__(16) unsigned char osm[];
+    __shared__ uint32_t so[kSmallPrepVerts], nrows[kSmallPrepVerts * kSmallPrepWords], bad, degrees;
+    OrderShared &sh = *reinterpret_cast<OrderShared *>(osm);
+    uint16_t *deg = reinterpret_cast<uint16_t *>(osm + (sizeof(OrderShared) + 15) / 16 * 16);
+    uint32_t *srows = reinterpret_cast<uint32_t *>(osm + order_fixed_bytes(prm.n));
+    const uint32_t n = prm.n, wp = prm.wp, t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    constexpr uint32_t T = kSmallPrepThreads;
+    if (t == 0) bad = degrees = 0u;
+    for (uint32_t i = t; i < n * w; i += T) srows[i] = rows_in[i];
+    // the ticket words past the queued frames
+    for (uint32_t i = t; i < prm.qcap; i += T)
+        if (i >= kSmallPrepVerts) prm.seq[i] = i;
+    __syncthreads();
+    for (uint32_t i = t; i < n * w; i += T)
+        if (!valid_word(n, w, srows, i)) bad = 1u;
+    order_rounds<T>(n, w, srows, order, deg, sh);
+    for (uint32_t i = t; i < n; i += T) so[i] = order[i];
+    __syncthreads();
+    for (uint32_t x = warp; x < n * wp; x += T / 32u) {
+        const uint32_t i = x / wp, j = x % wp * 32u + lane;
+        bool bit = false;
+        if (j < n) {
+            const uint32_t col = so[j];
+            bit = (srows[so[i] * w + (col >> 5)] >> (col & 31u)) & 1u;
+        }
+        const uint32_t word = __ballot_sync(FULLM, bit);
+        if (lane == 0) {
+            rows[x] = word;
+            nrows[x] = word;
+        }
+    }
+    __syncthreads();
+    uint32_t sum = 0u;
+    for (uint32_t x = t; x < n * wp; x += T) sum += (uint32_t)__popc(nrows[x]);
+    sum = __reduce_add_sync(FULLM, sum);
+    if (lane == 0 && sum != 0u) atomicAdd(&degrees, sum);
+    __syncthreads();
+    // L = V \ N(position 0): child k branches on its k-th vertex v, the ones
+    // before in X
+    const bool go = bad == 0u;
+    auto all_of = [&](uint32_t q) -> uint32_t { return n >= q * 32u + 32u ? FULLM : (n > q * 32u ? (1u << (n - q * 32u)) - 1u : 0u); };
+    uint32_t c = 0u;
+    for (uint32_t q = 0; q < wp; ++q) c += (uint32_t)__popc(all_of(q) & ~nrows[q]);
+    for (uint32_t k = t; k < kSmallPrepVerts && k < prm.qcap; k += T) prm.seq[k] = go && k < c ? k + 1u : k;
+    for (uint32_t k = t; k < c && go; k += T) {
+        uint32_t v = 0u;
+        for (uint32_t q = 0, before = 0; q < wp; ++q) {
+            uint32_t l = all_of(q) & ~nrows[q];
+            const uint32_t here = (uint32_t)__popc(l);
+            if (k >= before && k < before + here) {
+                for (uint32_t r = k - before; r > 0u; --r) l &= l - 1u;
+                v = q * 32u + (uint32_t)__ffs(l) - 1u;
+            }
+            before += here;
+        }
+        uint32_t *fr = prm.frames + (size_t)k * prm.fs;
+        for (uint32_t q = 0; q < wp; ++q) {
+            const uint32_t below = v >= q * 32u + 32u ? FULLM : (v > q * 32u ? (1u << (v - q * 32u)) - 1u : 0u);
+            const uint32_t X = all_of(q) & ~nrows[q] & below;
+            fr[kFrameHdr + q] = all_of(q) & ~X;
+            fr[kFrameHdr + wp + q] = X;
+            if (prm.lst.rec) fr[kFrameHdr + 2u * wp + q] = 0u;
+        }
+        fr[0] = (v + 1u) << 16;
+        fr[1] = fr[2] = fr[3] = fr[4] = 0u;
+    }
+    for (uint32_t i = t; i < MCE_OUT_WORDS(n); i += T) {
+        uint64_t x = 0ull;
+        if (i == MCE_OUT_NODES || i == MCE_OUT_INTERNAL) x = 1ull;
+        if (i == MCE_OUT_GROUPS) x = prm.total_groups;
+        if (i == MCE_OUT_STATUS && !go) x = static_cast<uint64_t>(static_cast<int64_t>(MCE_EINVAL));
+        prm.out[i] = x;
+    }
+    if (t == 0) {
+        Ctl *ctl = prm.ctl;
+        ctl->head = 0u;
+        ctl->abort = 0u;
+        ctl->tail = ctl->pending = go ? c : 0u;
+        ctl->starving = prm.total_groups;
+        ctl->pad3[0] = degrees;
+    }
+}
+
 // One block per graph of a batch; the rows go to shared memory when they fit
 // in the launch's dynamic shared memory.
 __global__ void __launch_bounds__(256) order_batch_kernel(const BatchGraph *__restrict__ graphs, size_t smem_bytes)
@@ -435,6 +537,19 @@ cudaError_t launch_order(uint32_t n, uint32_t w, const uint32_t *rows, uint32_t 
     cudaError_t e = kernel_smem_setup((const void *)f);
     if (e != cudaSuccess) return e;
     f<<<1, threads, smem, s>>>(n, w, rows, order, in_smem);
+    return cudaGetLastError();
+}
+
+bool small_prep_fits(uint32_t n, uint32_t w, uint32_t wp)
+{
+    return n >= 1u && n <= kSmallPrepVerts && wp <= kSmallPrepWords && order_fixed_bytes(n) + (size_t)n * w * 4 <= 40u * 1024u;
+}
+
+cudaError_t launch_small_prep(const SearchParams &prm, uint32_t w, const uint32_t *rows_in, uint32_t *order,
+                              uint32_t *rows, cudaStream_t s)
+{
+    small_prep_kernel<<<1, kSmallPrepThreads, order_fixed_bytes(prm.n) + (size_t)prm.n * w * 4, s>>>(prm, w, rows_in,
+                                                                                                order, rows);
     return cudaGetLastError();
 }
 

@@ -9,17 +9,20 @@ namespace mce {
 template <int K, bool SMEM, int PIVOT, bool LIST>
 cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStream_t s)
 {
-    const unsigned *rp = nullptr;
-    if (PIVOT == MCE_PIVOT_TOMITA && prm.n > 0) {
-        unsigned *dst = &prm.ctl->pad4[0];
-        root_tomita_pivot_kernel<0><<<1, 1024, 0, s>>>(prm.rows, prm.n, prm.wp, dst);
-        rp = dst;
+    cudaError_t e = cudaSuccess;
+    if (!prm.prepared) {
+        const unsigned *rp = nullptr;
+        if (PIVOT == MCE_PIVOT_TOMITA && prm.n > 0) {
+            unsigned *dst = &prm.ctl->pad4[0];
+            root_tomita_pivot_kernel<0><<<1, 1024, 0, s>>>(prm.rows, prm.n, prm.wp, dst);
+            rp = dst;
+        }
+        search_init_kernel<0><<<64, 256, 0, s>>>(prm);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        e = prm.part ? launch_part_frames(prm, rp, s) : launch_seed_children(prm, rp, s);
+        if (e != cudaSuccess) return e;
     }
-    search_init_kernel<0><<<64, 256, 0, s>>>(prm);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = prm.part ? launch_part_frames(prm, rp, s) : launch_seed_children(prm, rp, s);
-    if (e != cudaSuccess) return e;
     e = kernel_smem_setup((const void *)search_kernel<K, SMEM, PIVOT, LIST>);
     if (e != cudaSuccess) return e;
     search_kernel<K, SMEM, PIVOT, LIST><<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
