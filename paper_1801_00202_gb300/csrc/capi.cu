@@ -82,7 +82,6 @@ __attribute__((constructor)) void fault_from_env()
 
 struct Config {
     int G = 32, K = 1;  // the caller's shape: rows of G * K words
-    bool smem = false;
     unsigned threads = 0, blocks = 0;
     size_t smem_bytes = 0;
     uint32_t wp = 32;
@@ -108,12 +107,12 @@ mce_options defaults(const mce_options *o)
 
 // The search kernels for sets of `words` 32-bit words: one, two or four words
 // per lane of a warp.
-SearchImpl impl_for(uint32_t words, bool smem, int pivot, bool list = false)
+SearchImpl impl_for(uint32_t words, int pivot, bool list = false)
 {
     if (pivot == MCE_PIVOT_GREEDY_NX) pivot = MCE_PIVOT_GREEDY_TX;  // the TX kernels, early exit on
-    if (words <= 32) return list ? search_list_impl_1(smem, pivot) : search_impl_1(smem, pivot);
-    if (words <= 64) return list ? search_list_impl_2(smem, pivot) : search_impl_2(smem, pivot);
-    if (words <= 128) return list ? search_list_impl_4(smem, pivot) : search_impl_4(smem, pivot);
+    if (words <= 32) return list ? search_list_impl_1(pivot) : search_impl_1(pivot);
+    if (words <= 64) return list ? search_list_impl_2(pivot) : search_impl_2(pivot);
+    if (words <= 128) return list ? search_list_impl_4(pivot) : search_impl_4(pivot);
     return {nullptr, nullptr, nullptr, nullptr};
 }
 
@@ -128,11 +127,6 @@ uint32_t next_pow2(uint64_t x)
     uint64_t p = 1;
     while (p < x) p <<= 1;
     return (uint32_t)p;
-}
-
-size_t search_smem(uint32_t n, uint32_t wp, bool rows_in_smem, bool list = false, uint32_t slots = kLocalSlots)
-{
-    return search_smem_bytes(n, wp, rows_in_smem, list, slots);
 }
 
 constexpr uint32_t kListFlags = MCE_LIST | MCE_LIST_SORTED;
@@ -204,22 +198,17 @@ int choose(uint32_t n, const mce_options &o, Config &c)
     c.threads = o.threads_per_block ? o.threads_per_block : kLaunchThreads;
     if (c.threads % 32 || (o.threads_per_block && c.threads > kMaxThreads)) return MCE_EINVAL;
 
-    // Shared memory: rows of up to t2_smem_words words, and a region per warp
-    // for the warp tier; fewer warps where the regions do not fit.
+    // Shared memory: a region per warp for the warp tier; fewer warps where
+    // the regions do not fit.
     const Tuning tu = default_tuning();
     const uint32_t direct = n <= 128u ? kDirectBytes : 0u;
-    auto base_of = [&](bool rows_smem) {
-        return round_up(search_smem(n, c.wp, rows_smem, c.list, c.local_slots), 16) + direct;
-    };
-    auto fits = [&](bool rows_smem, unsigned threads) {
-        return base_of(rows_smem) + (size_t)(threads / 32) * kPoolBytesMin <= limit;
-    };
-    c.smem = W <= 32 && c.wp <= tu.t2_smem_words && fits(true, c.threads);
-    while (c.threads > 32 && !fits(c.smem, c.threads)) c.threads -= 32;
-    if (!fits(c.smem, c.threads)) return MCE_EINVAL;
-    c.impl = impl_for(W, c.smem, (int)o.pivot_mode, c.list);
+    const size_t base = round_up(search_smem_bytes(n, c.wp, c.list, c.local_slots), 16) + direct;
+    auto fits = [&](unsigned threads) { return base + (size_t)(threads / 32) * kPoolBytesMin <= limit; };
+    while (c.threads > 32 && !fits(c.threads)) c.threads -= 32;
+    if (!fits(c.threads)) return MCE_EINVAL;
+    c.impl = impl_for(W, (int)o.pivot_mode, c.list);
     if (!c.impl.run) return MCE_EINVAL;
-    c.t2_offset = (uint32_t)base_of(c.smem);
+    c.t2_offset = (uint32_t)base;
     c.direct_offset = c.t2_offset - direct;
     c.pool_bytes = plan_pool(c.t2_offset, c.threads, limit);
     c.t2_max_p = c.list ? 0u : tu.t2_p;
@@ -289,7 +278,6 @@ Tuning mce::default_tuning()
         // 0.472 -> 0.456 ms, and nothing off longer ones)
         d.idle_sleep_ns = 1024u;
         d.t2_p = (uint32_t)kPoolMaxP;
-        d.t2_smem_words = 0u;
         d.batch_split = 4u;
         d.give_steps = 16u;
         if (const char *env = std::getenv("MCE_TUNE")) {
@@ -308,7 +296,6 @@ Tuning mce::default_tuning()
                 else if (!std::strcmp(key, "pop_tries") && val) d.pop_tries = val;
                 else if (!std::strcmp(key, "idle_sleep_ns") && val) d.idle_sleep_ns = val;
                 else if (!std::strcmp(key, "t2_p")) d.t2_p = std::min(val, (uint32_t)kPoolMaxP);
-                else if (!std::strcmp(key, "t2_smem_words")) d.t2_smem_words = val;
                 else if (!std::strcmp(key, "batch_split")) d.batch_split = val;
                 else if (!std::strcmp(key, "serve_bcost")) d.serve_bcost = val;
                 else if (!std::strcmp(key, "t2_task")) d.t2_task = val;
@@ -389,7 +376,7 @@ int run_search(uint32_t n, const Config &c, const Layout &L, unsigned char *scra
         p.part_k = part->k;
         p.count_root = part->count_root;
     }
-    LaunchShape sh{c.blocks, c.threads, c.smem_bytes, c.smem};
+    LaunchShape sh{c.blocks, c.threads, c.smem_bytes};
     return cuda_code(c.impl.run(p, sh, s));
 }
 
@@ -480,7 +467,7 @@ int enumerate_device_impl(uint32_t n, uint32_t words_per_row, const uint32_t *d_
         p.prepared = 1u;
         const cudaError_t e = launch_small_prep(p, words_per_row, d_rows, order, rows, s);
         if (e != cudaSuccess) return cuda_code(e);
-        return cuda_code(c.impl.run(p, LaunchShape{c.blocks, c.threads, c.smem_bytes, c.smem}, s));
+        return cuda_code(c.impl.run(p, LaunchShape{c.blocks, c.threads, c.smem_bytes}, s));
     }
     cudaError_t e = cudaMemsetAsync(d_out + MCE_OUT_STATUS, 0, sizeof(uint64_t), s);
     if (e == cudaSuccess) e = launch_validate_rows(n, words_per_row, d_rows, d_out, s);
@@ -1363,7 +1350,6 @@ struct Bucket {
     uint32_t split = 0, wclass = 0;
     bool tuned = false;
     double tuned_ms = 0.0;
-    bool smem = false;
     std::vector<uint32_t> graphs;
     std::vector<uint32_t> items;  // work items: graph | part << 16 | parts << 24
     uint32_t split_graphs = 0;
@@ -1619,11 +1605,10 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         auto it = choice.find(wc);
         const TuneChoice t = it != choice.end() ? it->second : default_choice(g->n, o, !subproblems);
         const int G = t.G, K = t.K;
-        const SearchImpl plain = impl_for(W, false, (int)o.pivot_mode);
+        const SearchImpl plain = impl_for(W, (int)o.pivot_mode);
         if ((uint32_t)(G * K) < W || !shape_known(G, K) || !plain.run) { delete b; return MCE_EINVAL; }
-        const bool smem = W <= 32 && (uint32_t)(G * K) <= default_tuning().t2_smem_words;
         size_t bi = 0;
-        while (bi < buckets.size() && !(buckets[bi].plain.run == plain.run && buckets[bi].smem == smem &&
+        while (bi < buckets.size() && !(buckets[bi].plain.run == plain.run &&
                                         buckets[bi].threads == t.threads && buckets[bi].split == t.split))
             ++bi;
         if (bi == buckets.size()) {
@@ -1634,7 +1619,6 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
             nb.wclass = wc;
             nb.tuned = t.tuned;
             nb.tuned_ms = t.ms_per_graph;
-            nb.smem = smem;
             buckets.push_back(nb);
         }
         if (G * K > buckets[bi].G * buckets[bi].K) {  // the bucket reports its widest rows
@@ -1675,9 +1659,9 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         size_t base = 0;
         for (uint32_t i : bk.graphs) {
             words = std::max(words, (b->n[i] + 31) / 32);
-            base = std::max(base, search_smem(b->n[i], wp_of[i], bk.smem));
+            base = std::max(base, search_smem_bytes(b->n[i], wp_of[i]));
         }
-        bk.impl = impl_for(words, bk.smem, (int)o.pivot_mode);
+        bk.impl = impl_for(words, (int)o.pivot_mode);
         unsigned threads = bk.threads;
         if (threads % 32 || threads > (o.threads_per_block ? kMaxThreads : kLaunchThreads)) { rc = MCE_EINVAL; break; }
         // the whole-graph layout and the warp tier's regions; fewer warps where
@@ -1696,7 +1680,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         unsigned blocks = o.blocks ? o.blocks : (unsigned)(per_sm * sms);
         const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, blocks, default_tuning().batch_split);
         blocks = std::min<unsigned>(blocks, (unsigned)bk.items.size());
-        bk.shape = LaunchShape{blocks, threads, smem, bk.smem};
+        bk.shape = LaunchShape{blocks, threads, smem};
         bk.groups = threads / 32;
         bk.qcap = next_pow2(std::max<uint64_t>(256, 4ull * bk.groups + 64 + part_frames));
         if (o.queue_log2) bk.qcap = std::max<uint32_t>(bk.qcap, 1u << o.queue_log2);

@@ -102,7 +102,6 @@ struct Tuning {
     uint32_t pop_tries;     // ticket attempts of one take from the device-wide ring
     uint32_t idle_sleep_ns; // longest back-off of an idle warp that is not polling
     uint32_t t2_p;          // warp tier: largest |P| of a subproblem (0: off, at most kPoolMaxP)
-    uint32_t t2_smem_words; // warp tier on: rows of up to this many words are kept in shared memory
     uint32_t batch_split;   // batched form: parts of about 1/(blocks * batch_split) of a bucket's cost (0: no split)
     uint32_t serve_bcost;   // served form: largest expected maximal cliques (thousands) of a micro-batched request
     uint32_t t2_task;       // largest |P u X| of a subproblem (0: by density and size)
@@ -239,7 +238,6 @@ __host__ __device__ inline size_t batch_region_bytes(uint32_t qcap, uint32_t fs)
 struct LaunchShape {
     unsigned blocks, threads;
     size_t smem;
-    bool rows_in_smem;
 };
 
 // One search: init kernel (root frame, queue, zeroed output) + persistent
@@ -253,13 +251,13 @@ struct SearchImpl {
     cudaError_t (*run_batch)(const BatchParams &, const LaunchShape &, cudaStream_t);
     cudaError_t (*batch_occupancy)(int threads, size_t smem, int *blocks_per_sm);
 };
-SearchImpl search_impl_1(bool smem, int pivot);
-SearchImpl search_impl_2(bool smem, int pivot);
-SearchImpl search_impl_4(bool smem, int pivot);
+SearchImpl search_impl_1(int pivot);
+SearchImpl search_impl_2(int pivot);
+SearchImpl search_impl_4(int pivot);
 // Listing variants (run/occupancy only; no batched form).
-SearchImpl search_list_impl_1(bool smem, int pivot);
-SearchImpl search_list_impl_2(bool smem, int pivot);
-SearchImpl search_list_impl_4(bool smem, int pivot);
+SearchImpl search_list_impl_1(int pivot);
+SearchImpl search_list_impl_2(int pivot);
+SearchImpl search_list_impl_4(int pivot);
 
 
 // The root's children as independent subtrees (split.cu).  The root's
@@ -334,19 +332,12 @@ cudaError_t list_build(const ListJob &j, cudaStream_t s);
 Tuning default_tuning();
 
 // Shared-memory layout of the search kernels:
-//   [rows (when staged), padded to 16 B][hist: (n + 1) x u32, padded to 16 B]
-//   [local frame ring][whole-graph layout (n <= 128)][warp regions]
-__host__ __device__ inline size_t smem_rows_bytes(uint32_t n, uint32_t wp, bool rows_in_smem)
-{
-    return rows_in_smem ? ((size_t)n * wp * 4 + 15) / 16 * 16 : 0;
-}
-__host__ __device__ inline size_t smem_local_offset(uint32_t n, uint32_t wp, bool rows_in_smem)
-{
-    return smem_rows_bytes(n, wp, rows_in_smem) + (((size_t)n + 1) * 4 + 15) / 16 * 16;
-}
-__host__ __device__ inline size_t search_smem_bytes(uint32_t n, uint32_t wp, bool rows_in_smem, bool list = false,
+//   [hist: (n + 1) x u32, padded to 16 B][local frame ring]
+//   [whole-graph layout (n <= 128)][warp regions]
+__host__ __device__ inline size_t smem_local_offset(uint32_t n) { return (((size_t)n + 1) * 4 + 15) / 16 * 16; }
+__host__ __device__ inline size_t search_smem_bytes(uint32_t n, uint32_t wp, bool list = false,
                                                    uint32_t slots = kLocalSlots)
 {
-    return smem_local_offset(n, wp, rows_in_smem) + local_queue_bytes(wp, list, slots);
+    return smem_local_offset(n) + local_queue_bytes(wp, list, slots);
 }
 }  // namespace mce

@@ -12,8 +12,9 @@
 //  * The warp tier, where nearly all nodes are: subtrees of at most 128
 //    vertices, compressed to small sets and searched a child per lane (see
 //    "The warp tier" below).
-//  * The renumbered adjacency (Section 4.2) is staged in shared memory by a
-//    1-D bulk-copy (TMA) when it is small, else read from L2.
+//  * The renumbered adjacency (Section 4.2) is read from L2 above the warp
+//    tier, which leaves the shared memory to that tier (staging rows of up to
+//    32 words there gained 5 % on G(700, 0.18) and nothing elsewhere).
 //  * Work moves at two levels.  Idle warps take frames from their block's
 //    ring in shared memory or from the device-wide ring (a bounded MPMC ring
 //    in global memory whose tickets are taken by fetch-and-add at both ends);
@@ -27,7 +28,7 @@
 //    histogram; everything is integer arithmetic modulo 2^64, so the
 //    reduction order does not matter and results are bit-exact.
 //
-// Every spin (queue tickets, idle wait, the bulk-copy barrier) is bounded and
+// Every spin (queue tickets, idle wait) is bounded and
 // ends in an error status plus a global abort flag, never a hang or a trap.
 #pragma once
 
@@ -335,17 +336,17 @@ __device__ __forceinline__ unsigned lanes_below_sum(unsigned x, unsigned lane)
     return incl - x;
 }
 
-template <int K, bool SMEM>
+template <int K>
 __device__ __forceinline__ void load_row(uint32_t (&r)[K], const uint32_t *p)
 {
     if (K == 1) {
-        r[0] = SMEM ? p[0] : __ldg(p);
+        r[0] = __ldg(p);
     } else if (K == 2) {
-        uint2 t = SMEM ? *reinterpret_cast<const uint2 *>(p) : __ldg(reinterpret_cast<const uint2 *>(p));
+        uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
         r[0] = t.x;
         r[1] = t.y;
     } else {
-        uint4 t = SMEM ? *reinterpret_cast<const uint4 *>(p) : __ldg(reinterpret_cast<const uint4 *>(p));
+        uint4 t = __ldg(reinterpret_cast<const uint4 *>(p));
         r[0] = t.x;
         r[1] = t.y;
         r[2] = t.z;
@@ -485,64 +486,6 @@ __device__ __forceinline__ void flush_diag(const unsigned long long *diag, uint6
 #pragma unroll
     for (int i = 0; i < kDiagCount; ++i)
         if (diag[i]) atomicAdd(o + word[i], diag[i]);
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t mb, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(mb), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for phase `parity` of the barrier at mb: ~2 s, then false.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t mb, uint32_t parity)
-{
-    const uint64_t t0 = global_ns();
-#pragma unroll 1
-    for (unsigned t = 0;; ++t) {
-        if (mbar_try_wait(mb, parity)) return true;
-        if ((t & 63u) == 63u && global_ns() - t0 > 2000000000ull) return false;
-    }
-}
-
-// Stage `bytes` (multiple of 16, 16-byte aligned ends) of rows from global to
-// shared memory with 1-D bulk copies completing on the barrier at mb.  Thread 0
-// issues; every thread waits (bounded) for phase `parity`.  Returns false on a
-// timeout, after a second bounded wait that lets copies in flight land before
-// the shared memory can be reused.  Must be called by the whole block.
-__device__ __forceinline__ bool stage_rows(uint32_t *sdst, const uint32_t *gsrc, uint32_t bytes, uint32_t mb,
-                                           uint32_t parity)
-{
-    if (threadIdx.x == 0) {
-        // order earlier generic-proxy reads of this shared memory before the
-        // async-proxy writes
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes) : "memory");
-        const uint32_t dst0 = (uint32_t)__cvta_generic_to_shared(sdst);
-        for (uint32_t off = 0; off < bytes; off += 65536u) {
-            const uint32_t len = (bytes - off) < 65536u ? (bytes - off) : 65536u;
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    dst0 + off),
-                "l"(reinterpret_cast<const unsigned char *>(gsrc) + off), "r"(len), "r"(mb)
-                : "memory");
-        }
-    }
-    if (mbar_wait_bounded(mb, parity)) return true;
-    mbar_wait_bounded(mb, parity);
-    return false;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar)
-{
-    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(bar);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -691,7 +634,7 @@ __device__ __forceinline__ unsigned pool_first(const uint32_t (&s)[W])
 // few bits (G(3000, 0.1): some 40 KB from L2 for 30 vertices); there the warp
 // reads one row at a time, lane i the word that holds U[i + 32 k], and a ballot
 // makes the local row.  The start frame goes on the stack as frame `slot`.
-template <int W, int K, bool SMEM>
+template <int W, int K>
 __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const uint32_t *order, uint32_t region,
                                         unsigned slot, uint32_t mine0, uint32_t mine1, uint32_t mine2, uint32_t mine3,
                                         unsigned u, unsigned children, unsigned rs, uint64_t S)
@@ -703,7 +646,6 @@ __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const
     uint64_t *lhv = reinterpret_cast<uint64_t *>(smem_raw + region + Sh::kHashOff) + slot * Sh::kSlotVerts;
     const uint16_t *pos = reinterpret_cast<const uint16_t *>(smem_raw + region + Sh::kPosOff) + slot * Sh::kSlotVerts;
     uint32_t *f = reinterpret_cast<uint32_t *>(smem_raw + region + Sh::kStackOff) + slot * Sh::kFields;
-    const uint32_t *srows = reinterpret_cast<const uint32_t *>(smem_raw);  // SMEM: the rows lead the block's shared memory
     const uint32_t *row[W];
     uint32_t qw[W], qm[W];  // word and bit of this lane's columns
     unsigned pl = 0;
@@ -712,7 +654,7 @@ __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const
         const bool in = lane + 32u * g < u;
         const unsigned e = in ? (unsigned)pos[lane + 32u * g] : 0u;
         const unsigned q = e & kPosMask;
-        row[g] = (SMEM ? srows : rows) + (size_t)q * rw;
+        row[g] = rows + (size_t)q * rw;
         qw[g] = q >> 5;
         qm[g] = in ? 1u << (q & 31u) : 0u;
         if (in) lhv[lane + 32u * g] = mix64((uint64_t)order[q] + 1u);
@@ -757,15 +699,14 @@ __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const
 #pragma unroll
             for (int g = 0; g < W; ++g) {
                 if (V == 4u) {
-                    const uint4 t = SMEM ? *reinterpret_cast<const uint4 *>(row[g] + w0)
-                                         : __ldg(reinterpret_cast<const uint4 *>(row[g] + w0));
+                    const uint4 t = __ldg(reinterpret_cast<const uint4 *>(row[g] + w0));
                     x[g][0] = t.x;
                     x[g][1] = t.y;
                     x[g][2] = t.z;
                     x[g][3] = t.w;
                 } else {
-                    x[g][0] = SMEM ? row[g][0] : __ldg(row[g]);
-                    x[g][1] = V > 1u ? (SMEM ? row[g][1] : __ldg(row[g] + 1)) : 0u;
+                    x[g][0] = __ldg(row[g]);
+                    x[g][1] = V > 1u ? __ldg(row[g] + 1) : 0u;
                     x[g][2] = x[g][3] = 0u;
                 }
             }
@@ -1284,13 +1225,13 @@ __device__ __forceinline__ void pool_run_class(unsigned cls, const PoolAt &at, u
 }
 
 // The search proper: this warp expands frames until the search is over or
-// aborts.  rows, order: the renumbered adjacency (rows of prm.wp words, in
-// shared memory when SMEM) and the labels; hist, lq, region: this block's
+// aborts.  rows, order: the renumbered adjacency (rows of prm.wp words) and
+// the labels; hist, lq, region: this block's
 // clique-size histogram and ring and this warp's region of shared memory.
 // direct: the block holds the whole graph's rows, hash terms and positions in
 // the warp tier's layout (graphs of at most 128 vertices).  Called by all 32
 // lanes of every warp of the block.
-template <int K, bool SMEM, int PIVOT, bool LIST>
+template <int K, int PIVOT, bool LIST>
 __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint32_t *rows, uint32_t *hist,
                                             const LocalQ &lq, const Thresholds th, const PoolAt at, bool direct,
                                             Counters &cn)
@@ -1356,7 +1297,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
 
     auto get_row = [&](uint32_t (&r)[K], unsigned v) {
         if (mine) {
-            load_row<K, SMEM>(r, rows + (size_t)v * rw + lane * K);
+            load_row<K>(r, rows + (size_t)v * rw + lane * K);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k) r[k] = 0u;
@@ -1634,15 +1575,14 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
             }
         }
         __syncwarp();
-        const uint32_t *src = SMEM ? nullptr : rows;
         if (th.cls == 1u)
-            pool_build<1, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<1, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
         else if (th.cls == 2u)
-            pool_build<2, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<2, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
         else if (th.cls == 3u)
-            pool_build<3, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<3, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
         else
-            pool_build<4, K, SMEM>(src, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<4, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
     };
     // whether a frame of |P| = np, |P u X| = u and c children fits the tier
     auto pool_fits = [&](unsigned np, unsigned u, unsigned c) -> bool {
@@ -1968,12 +1908,11 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
                         for (unsigned j = 0; j < nc; ++j) {
                             const unsigned jj = ((j + lane) & (nc - 1u)) * 4u;
                             const uint4 a = *reinterpret_cast<const uint4 *>(pw + jj);
-                            const uint4 q = SMEM ? *reinterpret_cast<const uint4 *>(ru + jj)
-                                                 : __ldg(reinterpret_cast<const uint4 *>(ru + jj));
+                            const uint4 q = __ldg(reinterpret_cast<const uint4 *>(ru + jj));
                             c += (unsigned)(__popc(a.x & q.x) + __popc(a.y & q.y) + __popc(a.z & q.z) + __popc(a.w & q.w));
                         }
                     } else {
-                        for (unsigned j = 0; j < sw; ++j) c += (unsigned)__popc(pw[j] & (SMEM ? ru[j] : __ldg(ru + j)));
+                        for (unsigned j = 0; j < sw; ++j) c += (unsigned)__popc(pw[j] & __ldg(ru + j));
                     }
                     const unsigned key = ((c + 1u) << 16) | (0xffffu - u);
                     best = key > best ? key : best;
@@ -2066,32 +2005,20 @@ __device__ __forceinline__ void direct_layout(const uint32_t *rows, uint32_t rw,
     }
 }
 
-template <int K, bool SMEM, int PIVOT, bool LIST>
+template <int K, int PIVOT, bool LIST>
 __global__ void __launch_bounds__(kLaunchThreads) search_kernel(const SearchParams prm)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t mbar;
-
     const uint32_t n = prm.n;
-    const size_t rbytes = smem_rows_bytes(n, prm.wp, SMEM);
-    uint32_t *srows = reinterpret_cast<uint32_t *>(smem_raw);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + rbytes);
-    const uint32_t lq_off = (uint32_t)smem_local_offset(n, prm.wp, SMEM);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw);
+    const uint32_t lq_off = (uint32_t)smem_local_offset(n);
     const LocalQ lq = local_queue_at(smem_raw + lq_off, prm.wp, prm.local_slots);
     local_queue_reset(lq, blockDim.x / 32u);
 
-    // ---- prologue: stage the rows (bulk copy), histogram
-    if (SMEM) {
-        if (threadIdx.x == 0) mbar_init(&mbar);
-        __syncthreads();
-    }
 #pragma unroll 1
     for (uint32_t i = threadIdx.x; i <= n; i += blockDim.x) hist[i] = 0u;
-    bool staged = true;
-    if (SMEM) staged = stage_rows(srows, prm.rows, (uint32_t)rbytes, (uint32_t)__cvta_generic_to_shared(&mbar), 0u);
-    if (!staged && threadIdx.x == 0) set_status(prm.out, prm.ctl, MCE_ETIMEOUT);
     const Thresholds th = density_thresholds(prm.ctl->pad3[0], n, prm.tune, prm.split_min_p);
-    const uint32_t *rows = SMEM ? srows : prm.rows;
+    const uint32_t *rows = prm.rows;
     const bool direct = !LIST && K == 1 && n <= 128u && prm.t2_max_p != 0u;
     PoolAt at{};
     at.rows = prm.direct_offset;
@@ -2099,14 +2026,14 @@ __global__ void __launch_bounds__(kLaunchThreads) search_kernel(const SearchPara
     at.pos = at.hash + kDirectVerts * 8;
     at.region = prm.t2_offset + (threadIdx.x >> 5) * prm.pool_bytes;
     at.lq = lq_off;
-    at.hist = (uint32_t)rbytes;
-    const bool ok = __syncthreads_and(staged) != 0;
-    if (direct && ok)
+    at.hist = 0u;
+    __syncthreads();
+    if (direct)
         direct_layout(rows, prm.wp, prm.order, n, th.cls, reinterpret_cast<uint32_t *>(smem_raw + at.rows),
                       reinterpret_cast<uint64_t *>(smem_raw + at.hash), reinterpret_cast<uint16_t *>(smem_raw + at.pos));
     Counters cn;
     cn.diag = lq.h->diag;
-    if (ok) search_loop<K, SMEM, PIVOT, LIST>(prm, rows, hist, lq, th, at, direct, cn);
+    search_loop<K, PIVOT, LIST>(prm, rows, hist, lq, th, at, direct, cn);
     flush_counters(cn, prm.out);
     __syncthreads();
     if (threadIdx.x == 0) flush_diag(lq.h->diag, prm.out);
@@ -2121,23 +2048,16 @@ __global__ void __launch_bounds__(kLaunchThreads) search_kernel(const SearchPara
 // Per graph: output initialised with the root counted (status kept), rows
 // bulk-copied to shared memory, root frame queued, search, reduction into the
 // graph's own result array.
-template <int K, bool SMEM, int PIVOT>
+template <int K, int PIVOT>
 __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams bp)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t mbar;
     __shared__ unsigned cur, root_key;
 
     unsigned char *region = bp.qbase + (size_t)blockIdx.x * bp.qstride;
     Ctl *ctl = reinterpret_cast<Ctl *>(region);
     unsigned *seq = reinterpret_cast<unsigned *>(region + batch_seq_offset());
     uint32_t *frames = reinterpret_cast<uint32_t *>(region + batch_frames_offset(bp.qcap));
-    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar);
-    if (SMEM) {
-        if (threadIdx.x == 0) mbar_init(&mbar);
-        __syncthreads();
-    }
-    uint32_t phase = 0;
     for (;;) {
         if (threadIdx.x == 0) cur = atomicAdd(bp.next, 1u);
         __syncthreads();
@@ -2151,10 +2071,8 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
         const unsigned part = (item >> 16) & 0xffu, parts = max(item >> 24, 1u);
         const BatchGraph gd = bp.graphs[item & 0xffffu];
         const uint32_t n = gd.n, WP = gd.wp;
-        const size_t rbytes = smem_rows_bytes(n, WP, SMEM);
-        uint32_t *srows = reinterpret_cast<uint32_t *>(smem_raw);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + rbytes);
-        const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n, WP, SMEM), WP);
+        uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw);
+        const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n), WP);
         local_queue_reset(lq, bp.groups_per_block);
         const bool valid = gd.out[MCE_OUT_STATUS] == 0ull;
         // The root's P and X over positions: all of V and nothing, or, for a
@@ -2302,9 +2220,6 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
             if (split && j >= 1u && j <= queued) sv = j + 1u;
             seq[j] = sv;
         }
-        bool staged = true;
-        if (SMEM) staged = stage_rows(srows, gd.ren, (uint32_t)rbytes, mb, phase & 1u);
-        ++phase;
         __syncthreads();
         if (threadIdx.x == 0) {
             frames[0] = (p0 & 0xffffu) | (n << 16);
@@ -2316,13 +2231,9 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
             ctl->tail = split ? queued + 1u : (root ? 1u : 0u);
             ctl->pending = split ? queued : (root ? 1u : 0u);
             ctl->starving = 0u;
-            if (!staged) {
-                atomicCAS(reinterpret_cast<unsigned long long *>(gd.out + MCE_OUT_STATUS), 0ull,
-                          static_cast<unsigned long long>(static_cast<long long>(MCE_ETIMEOUT)));
-            }
         }
         __threadfence();
-        const bool ok = __syncthreads_and(staged) != 0;
+        __syncthreads();
 
         SearchParams prm;
         prm = SearchParams{};
@@ -2349,7 +2260,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
         prm.pool_bytes = bp.pool_bytes;
         prm.t2_max_p = bp.t2_max_p;
         prm.direct_offset = bp.direct_offset;
-        const uint32_t *rows = SMEM ? srows : gd.ren;
+        const uint32_t *rows = gd.ren;
         if (threadIdx.x == 0) root_key = 0u;
         __syncthreads();
         {
@@ -2365,14 +2276,14 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
         at.hash = at.rows + kDirectRows * 4;
         at.pos = at.hash + kDirectVerts * 8;
         at.region = bp.t2_offset + (threadIdx.x >> 5) * bp.pool_bytes;
-        at.lq = (uint32_t)smem_local_offset(n, WP, SMEM);
-        at.hist = (uint32_t)rbytes;
+        at.lq = (uint32_t)smem_local_offset(n);
+        at.hist = 0u;
         if (direct)
             direct_layout(rows, WP, gd.order, n, th.cls, reinterpret_cast<uint32_t *>(smem_raw + at.rows),
                           reinterpret_cast<uint64_t *>(smem_raw + at.hash), reinterpret_cast<uint16_t *>(smem_raw + at.pos));
         Counters cn;
         cn.diag = lq.h->diag;
-        if (ok) search_loop<K, SMEM, PIVOT, false>(prm, rows, hist, lq, th, at, direct, cn);
+        search_loop<K, PIVOT, false>(prm, rows, hist, lq, th, at, direct, cn);
         flush_counters(cn, gd.out);
         __syncthreads();
         if (threadIdx.x == 0) flush_diag(lq.h->diag, gd.out);

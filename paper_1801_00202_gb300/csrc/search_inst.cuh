@@ -6,7 +6,7 @@
 
 namespace mce {
 
-template <int K, bool SMEM, int PIVOT, bool LIST>
+template <int K, int PIVOT, bool LIST>
 cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
@@ -23,72 +23,61 @@ cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStr
         e = prm.part ? launch_part_frames(prm, rp, s) : launch_seed_children(prm, rp, s);
         if (e != cudaSuccess) return e;
     }
-    e = kernel_smem_setup((const void *)search_kernel<K, SMEM, PIVOT, LIST>);
+    e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>);
     if (e != cudaSuccess) return e;
-    search_kernel<K, SMEM, PIVOT, LIST><<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
+    search_kernel<K, PIVOT, LIST><<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
     return cudaGetLastError();
 }
 
-template <int K, bool SMEM, int PIVOT, bool LIST>
+template <int K, int PIVOT, bool LIST>
 cudaError_t occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 {
-    cudaError_t e = kernel_smem_setup((const void *)search_kernel<K, SMEM, PIVOT, LIST>);
+    cudaError_t e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, search_kernel<K, SMEM, PIVOT, LIST>, threads,
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, search_kernel<K, PIVOT, LIST>, threads,
                                                          smem);
 }
 
-template <int K, bool SMEM, int PIVOT>
+template <int K, int PIVOT>
 cudaError_t run_batch_t(const BatchParams &bp, const LaunchShape &sh, cudaStream_t s)
 {
-    batch_kernel<K, SMEM, PIVOT><<<sh.blocks, sh.threads, sh.smem, s>>>(bp);
+    batch_kernel<K, PIVOT><<<sh.blocks, sh.threads, sh.smem, s>>>(bp);
     return cudaGetLastError();
 }
 
-template <int K, bool SMEM, int PIVOT>
+template <int K, int PIVOT>
 cudaError_t batch_occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 {
-    cudaError_t e = kernel_smem_setup((const void *)batch_kernel<K, SMEM, PIVOT>);
+    cudaError_t e = kernel_smem_setup((const void *)batch_kernel<K, PIVOT>);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<K, SMEM, PIVOT>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<K, PIVOT>, threads, smem);
 }
 
 // The listing variant (LIST) has no batched form.
-template <int K, bool SMEM, int PIVOT, bool LIST>
+template <int K, int PIVOT, bool LIST>
 SearchImpl impl_t()
 {
     if constexpr (LIST)
-        return {run_search_t<K, SMEM, PIVOT, true>, occupancy_t<K, SMEM, PIVOT, true>, nullptr, nullptr};
+        return {run_search_t<K, PIVOT, true>, occupancy_t<K, PIVOT, true>, nullptr, nullptr};
     else
-        return {run_search_t<K, SMEM, PIVOT, false>, occupancy_t<K, SMEM, PIVOT, false>, run_batch_t<K, SMEM, PIVOT>,
-                batch_occupancy_t<K, SMEM, PIVOT>};
+        return {run_search_t<K, PIVOT, false>, occupancy_t<K, PIVOT, false>, run_batch_t<K, PIVOT>,
+                batch_occupancy_t<K, PIVOT>};
 }
 
-template <int K, bool SMEM, bool LIST>
-SearchImpl pick_pivot(int pivot)
+template <int K, bool LIST>
+SearchImpl pick(int pivot)
 {
     switch (pivot) {
-    case MCE_PIVOT_GREEDY: return impl_t<K, SMEM, MCE_PIVOT_GREEDY, LIST>();
-    case MCE_PIVOT_GREEDY_TX: return impl_t<K, SMEM, MCE_PIVOT_GREEDY_TX, LIST>();
-    case MCE_PIVOT_TOMITA: return impl_t<K, SMEM, MCE_PIVOT_TOMITA, LIST>();
+    case MCE_PIVOT_GREEDY: return impl_t<K, MCE_PIVOT_GREEDY, LIST>();
+    case MCE_PIVOT_GREEDY_TX: return impl_t<K, MCE_PIVOT_GREEDY_TX, LIST>();
+    case MCE_PIVOT_TOMITA: return impl_t<K, MCE_PIVOT_TOMITA, LIST>();
     default: return {nullptr, nullptr, nullptr, nullptr};
     }
-}
-
-// Rows live in shared memory only for sets of at most 32 words.
-template <int K, bool LIST>
-SearchImpl pick(bool smem, int pivot)
-{
-    if constexpr (K == 1) {
-        if (smem) return pick_pivot<K, true, LIST>(pivot);
-    }
-    if (smem) return {nullptr, nullptr, nullptr, nullptr};
-    return pick_pivot<K, false, LIST>(pivot);
 }
 
 }  // namespace mce
 
 #define MCE_DEFINE_SEARCH(K) \
-    namespace mce { SearchImpl search_impl_##K(bool smem, int pivot) { return pick<K, false>(smem, pivot); } }
+    namespace mce { SearchImpl search_impl_##K(int pivot) { return pick<K, false>(pivot); } }
 #define MCE_DEFINE_SEARCH_LIST(K) \
-    namespace mce { SearchImpl search_list_impl_##K(bool smem, int pivot) { return pick<K, true>(smem, pivot); } }
+    namespace mce { SearchImpl search_list_impl_##K(int pivot) { return pick<K, true>(pivot); } }
