@@ -203,14 +203,16 @@ int choose(uint32_t n, const mce_options &o, Config &c)
     const Tuning tu = default_tuning();
     const uint32_t direct = n <= 128u ? kDirectBytes : 0u;
     const size_t base = round_up(search_smem_bytes(n, c.wp, c.list, c.local_slots), 16) + direct;
-    auto fits = [&](unsigned threads) { return base + (size_t)(threads / 32) * kPoolBytesMin <= limit; };
+    // (a listing search has no warp tier: a row of scratch for the pivot scores)
+    const size_t region = c.list ? round_up((size_t)c.wp * 4, 16) : kPoolBytesMin;
+    auto fits = [&](unsigned threads) { return base + (size_t)(threads / 32) * region <= limit; };
     while (c.threads > 32 && !fits(c.threads)) c.threads -= 32;
     if (!fits(c.threads)) return MCE_EINVAL;
     c.impl = impl_for(W, (int)o.pivot_mode, c.list);
     if (!c.impl.run) return MCE_EINVAL;
     c.t2_offset = (uint32_t)base;
     c.direct_offset = c.t2_offset - direct;
-    c.pool_bytes = plan_pool(c.t2_offset, c.threads, limit);
+    c.pool_bytes = c.list ? (uint32_t)region : plan_pool(c.t2_offset, c.threads, limit);
     c.t2_max_p = c.list ? 0u : tu.t2_p;
     c.smem_bytes = c.t2_offset + (size_t)(c.threads / 32) * c.pool_bytes;
     if (o.blocks) {

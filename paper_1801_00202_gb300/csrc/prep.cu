@@ -570,7 +570,7 @@ cudaError_t launch_renumber(uint32_t n, uint32_t w, const uint32_t *rows, const 
 }
 
 
-cudaError_t kernel_smem_setup(const void *func)
+cudaError_t kernel_smem_setup(const void *func, bool prefer_l1)
 {
     constexpr int kMaxDev = 64;
     static std::mutex mu;
@@ -587,7 +587,7 @@ cudaError_t kernel_smem_setup(const void *func)
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, func);
     if (e == cudaSuccess)  // static shared memory counts against the same limit
         e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !prefer_l1)
         e = cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess && (int)done.size() < kMaxDev * 256) done.emplace_back(func, dev);
     return e;

@@ -1886,7 +1886,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
             // lanes hits distinct banks), and one packed max (score + 1,
             // 0xffff - position) keeps the highest score, earliest on ties.
             // NX has TX's pivot (its early exit only saves work).
-            uint32_t *pw = reinterpret_cast<uint32_t *>(smem_raw + at.region + po.leaf);
+            uint32_t *pw = reinterpret_cast<uint32_t *>(smem_raw + at.region + (LIST ? 0u : po.leaf));
 #pragma unroll
             for (int k = 0; k < K; ++k)
                 if (mine) pw[lane * K + k] = Pc[k];

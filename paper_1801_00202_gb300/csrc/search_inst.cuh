@@ -23,7 +23,7 @@ cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStr
         e = prm.part ? launch_part_frames(prm, rp, s) : launch_seed_children(prm, rp, s);
         if (e != cudaSuccess) return e;
     }
-    e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>);
+    e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>, LIST);
     if (e != cudaSuccess) return e;
     search_kernel<K, PIVOT, LIST><<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
     return cudaGetLastError();
@@ -32,7 +32,7 @@ cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStr
 template <int K, int PIVOT, bool LIST>
 cudaError_t occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 {
-    cudaError_t e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>);
+    cudaError_t e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>, LIST);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, search_kernel<K, PIVOT, LIST>, threads,
                                                          smem);
