@@ -170,12 +170,35 @@ void pick_shape(uint32_t n, const mce_options &o, int &G, int &K)
     }
 }
 
-// Most threads per block a caller may ask for; the library's own choice is
-// kLaunchThreads (24 warps, 80 registers per thread: the warp tier's loop
-// needs no more, and more warps hide its shared-memory latencies).
+// Most threads per block a caller may ask for; the library's own choice for a
+// single graph is kShortThreads, and kLaunchThreads for a long search.
 constexpr unsigned kMaxThreads = 512u;
 
-int choose(uint32_t n, const mce_options &o, Config &c)
+// Whether G(n, m / C(n, 2)) has at least 4e7 maximal cliques in expectation:
+// between the last size at which 512 threads win (G(1000, 0.3), 1.5e7) and the
+// first at which 768 do (G(400, 0.5) 3.14 against 3.28 ms, G(700, 0.4) 5.07
+// against 5.17).  One logarithm a clique size, up to the sizes that no longer
+// count; nothing for graphs that are clearly short.
+bool long_search(uint32_t n, uint64_t m)
+{
+    if (n < 2) return false;
+    const double p = std::min(1.0, (double)m / (0.5 * n * (n - 1.0)));
+    if ((n <= 256 && p <= 0.5) || (n <= 64 && p <= 0.85) || p <= 0.0) return false;
+    const double lp = std::log(p);
+    double choose_k = 0.0, pk = 1.0, total = 0.0, best = -1e300;
+    for (uint32_t k = 1; k <= n; ++k) {
+        choose_k += std::log((n - k + 1.0) / k);
+        pk *= p;
+        const double t = choose_k + 0.5 * k * (k - 1.0) * lp + (pk < 1.0 ? (n - k) * std::log1p(-pk) : (k < n ? -1e9 : 0.0));
+        if (t > 17.6) return true;  // this size alone has 4e7
+        total += std::exp(t);
+        best = std::max(best, t);
+        if (t < best - 12.0 && t < 12.0 && pk * n < 1.0) break;
+    }
+    return total >= 4e7;
+}
+
+int choose(uint32_t n, const mce_options &o, Config &c, bool long_run = false)
 {
     if (o.pivot_mode > MCE_PIVOT_GREEDY_NX || o.stack_levels > (uint32_t)kStackDepth || o.queue_log2 > 24)
         return MCE_EINVAL;
@@ -195,7 +218,7 @@ int choose(uint32_t n, const mce_options &o, Config &c)
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return MCE_ECUDA;
     const size_t limit = (size_t)optin - 1024;  // static shared memory + slack
 
-    c.threads = o.threads_per_block ? o.threads_per_block : kLaunchThreads;
+    c.threads = o.threads_per_block ? o.threads_per_block : (long_run && !c.list ? kLaunchThreads : kShortThreads);
     if (c.threads % 32 || (o.threads_per_block && c.threads > kMaxThreads)) return MCE_EINVAL;
 
     // Shared memory: a region per warp for the warp tier; fewer warps where
@@ -213,6 +236,11 @@ int choose(uint32_t n, const mce_options &o, Config &c)
     c.t2_offset = (uint32_t)base;
     c.direct_offset = c.t2_offset - direct;
     c.pool_bytes = c.list ? (uint32_t)region : plan_pool(c.t2_offset, c.threads, limit);
+    // With 16 warps the stacks need not fill the shared memory, and what they
+    // leave is L1 for the rows (G(1000, 0.3) 3.05 -> 2.91 ms, G(700, 0.18) 0.477 ->
+    // 0.460).  Graphs of up to 128 vertices read no rows and keep the stacks
+    // (G(100, 0.8) 1.02 against 1.08).
+    if (c.threads <= kShortThreads && n > 128u) c.pool_bytes = std::min<uint32_t>(c.pool_bytes, kPoolBytesShort);
     c.t2_max_p = c.list ? 0u : tu.t2_p;
     c.smem_bytes = c.t2_offset + (size_t)(c.threads / 32) * c.pool_bytes;
     if (o.blocks) {
@@ -1192,7 +1220,7 @@ int enumerate_once(mce_graph *g, const mce_options &opts, mce_result *res, std::
     if (sizes_only) o.flags &= ~kListFlags;
     const bool listing = (o.flags & kListFlags) != 0u;
     Config c;
-    int rc = choose(g->n, o, c);
+    int rc = choose(g->n, o, c, long_search(g->n, g->m));
     if (rc) return rc;
     if (children && c.qcap < 2u * k) c.qcap = next_pow2(2ull * k);  // every child frame queued at once
     const Layout L = layout(g->n, c);

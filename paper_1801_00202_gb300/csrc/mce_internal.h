@@ -122,15 +122,23 @@ constexpr int kPoolMaxP = 128;          // largest |P| of a subproblem
 // A warp's region: at least 64 frames of any set size (a stack that is paged
 // out at fewer than 32 free frames must hold 32 to page), at most about 256 of
 // four words.
-constexpr uint32_t kPoolBytesMin = 7248, kPoolBytesMax = 15360;
+constexpr uint32_t kPoolBytesMin = 7248, kPoolBytesMax = 15360, kPoolBytesShort = 9216;
 
 // Graphs of at most 128 vertices: the whole graph in the warp tier's layout,
 // once per block (rows, hash terms, positions).
 constexpr int kDirectRows = 512, kDirectVerts = 128;
 constexpr uint32_t kDirectBytes = kDirectRows * 4 + kDirectVerts * 10;
 
-// Most threads of a search block (the register bound of the kernels).
-constexpr unsigned kLaunchThreads = 768u;
+// Most threads of a search block (the register bound of the kernels).  The
+// single-graph search is compiled for 768 threads (80 registers: the warp
+// tier's loop fits, the search by frames above it spills 200 words) and for
+// 512 (128 registers, nothing spilled).  Most searches spend enough of their
+// time above the warp tier for the latter, ms with 768 / 512 threads: G(100,
+// 0.5) 0.150 / 0.135, G(250, 0.4) 0.31 / 0.23, G(700, 0.18) 0.53 / 0.46,
+// G(1000, 0.3) 3.2 / 2.9, G(3000, 0.1) 3.0 / 2.6.  A long search is nearly all
+// warp tier and wants the warps: G(500, 0.5) 9.6 / 10.3, G(100, 0.9) 16.1 /
+// 18.4.  (576 and 608 threads: slower than the better of the two everywhere.)
+constexpr unsigned kLaunchThreads = 768u, kShortThreads = 512u;
 
 struct SearchParams {
     uint32_t n;             // vertices
@@ -307,9 +315,9 @@ inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // prefer the largest shared-memory carveout, once per (kernel, device).  Every
 // launch after that runs under the same settings, so kernels of different
 // requests on different streams never wait for one another to change them.
-// prefer_l1 (the listing search, which has no warp tier and needs little shared
-// memory): the carveout is left to the driver, and the rows stay in L1
-// (G(700, 0.3) 4.5 -> 4.1 ms, G(1000, 0.2) 1.9 -> 1.75).
+// prefer_l1 (the single-graph search of up to 512 threads): the carveout is
+// left to the driver, and the rows stay in L1 where the blocks leave room
+// (listing G(700, 0.3) 4.5 -> 4.1 ms, counting G(1000, 0.3) 3.11 -> 2.91).
 cudaError_t kernel_smem_setup(const void *func, bool prefer_l1 = false);
 
 // Listing post-pass (listing.cu): record chunks of a finished listing search

@@ -2005,8 +2005,8 @@ __device__ __forceinline__ void direct_layout(const uint32_t *rows, uint32_t rw,
     }
 }
 
-template <int K, int PIVOT, bool LIST>
-__global__ void __launch_bounds__(kLaunchThreads) search_kernel(const SearchParams prm)
+template <int K, int PIVOT, bool LIST, int T>
+__global__ void __launch_bounds__(T) search_kernel(const SearchParams prm)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const uint32_t n = prm.n;

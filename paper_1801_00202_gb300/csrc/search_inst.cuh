@@ -6,6 +6,16 @@
 
 namespace mce {
 
+// The instance for blocks of `threads` threads (listing has the short one).
+template <int K, int PIVOT, bool LIST>
+auto search_kernel_for(unsigned threads)
+{
+    if constexpr (LIST) return search_kernel<K, PIVOT, true, kShortThreads>;
+    else
+        return threads <= kShortThreads ? search_kernel<K, PIVOT, false, kShortThreads>
+                                        : search_kernel<K, PIVOT, false, kLaunchThreads>;
+}
+
 template <int K, int PIVOT, bool LIST>
 cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStream_t s)
 {
@@ -23,19 +33,20 @@ cudaError_t run_search_t(const SearchParams &prm, const LaunchShape &sh, cudaStr
         e = prm.part ? launch_part_frames(prm, rp, s) : launch_seed_children(prm, rp, s);
         if (e != cudaSuccess) return e;
     }
-    e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>, LIST);
+    auto kernel = search_kernel_for<K, PIVOT, LIST>(sh.threads);
+    e = kernel_smem_setup((const void *)kernel, sh.threads <= kShortThreads);
     if (e != cudaSuccess) return e;
-    search_kernel<K, PIVOT, LIST><<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
+    kernel<<<sh.blocks, sh.threads, sh.smem, s>>>(prm);
     return cudaGetLastError();
 }
 
 template <int K, int PIVOT, bool LIST>
 cudaError_t occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 {
-    cudaError_t e = kernel_smem_setup((const void *)search_kernel<K, PIVOT, LIST>, LIST);
+    auto kernel = search_kernel_for<K, PIVOT, LIST>((unsigned)threads);
+    cudaError_t e = kernel_smem_setup((const void *)kernel, (unsigned)threads <= kShortThreads);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, search_kernel<K, PIVOT, LIST>, threads,
-                                                         smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, threads, smem);
 }
 
 template <int K, int PIVOT>
