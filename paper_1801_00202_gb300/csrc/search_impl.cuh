@@ -2269,7 +2269,10 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
             atomicAdd(&root_key, mine);
         }
         __syncthreads();
-        const Thresholds th = density_thresholds(root_key, n, bp.tune, bp.split_min_p, bp.cls);
+        // (the outer loop's subproblems of more than 128 vertices are sparse and
+        // alike: the size that fits their children, several side by side.
+        // G(10000, 0.03): 18.5 -> 15.7 ms on the device)
+        const Thresholds th = density_thresholds(root_key, n, bp.tune, bp.split_min_p, sub && n > 128u ? 0u : bp.cls);
         const bool direct = K == 1 && n <= 128u && bp.t2_max_p != 0u;
         PoolAt at{};
         at.rows = bp.direct_offset;
