@@ -88,14 +88,16 @@ __global__ void validate_kernel(uint32_t n, uint32_t w, const uint32_t *__restri
 // picks, about 0.1 us each (max-reduction, one broadcast load, four
 // subtractions), and 3 to 5 us of gathering and barriers a round.  A search of
 // all vertices for one or two picks a round took, per launch (G(n, p), now in
-// brackets): n = 100 24 us (16), 300 85 (57), 500 146 (121), 1000 383 (253),
-// 3000 4345 (756; rows in L2, two dependent reads a round).
+// brackets): n = 100 24 us (16), 300 85 (55), 500 146 (94), 1000 383 (237),
+// 3000 4345 (915; rows in L2, two dependent reads a round).  The pass that
+// lowers the degrees counts them for the next round's classes as well: 4 % of
+// the launch against a pass and a barrier of its own (1000: 248, 3000: 952).
 constexpr unsigned kOrderCand = 128;
 constexpr unsigned kSmallPrepThreads = 256, kSmallPrepVerts = 128, kSmallPrepWords = 4;
 
 struct OrderShared {
     uint32_t adj[kOrderCand][4];   // adjacency among the candidates
-    uint32_t hist[kOrderCand];     // vertices by (maximum degree - degree)
+    uint32_t hist[2][kOrderCand];  // vertices by (base - degree), of this round and the next
     uint32_t chunk[4096 / 32];     // vertices of maximum degree by 32 labels (crowded rounds)
     uint16_t label[kOrderCand];    // the candidates
     uint16_t placed[kOrderCand];   // this round's picks
@@ -126,7 +128,7 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
     constexpr uint32_t NW = T / 32u;
     const uint32_t chunks = (n + 31u) / 32u;
     if (t == 0) sh.top = 0u;
-    for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[i] = 0u;
+    for (uint32_t i = t; i < 2u * kOrderCand; i += T) sh.hist[i / kOrderCand][i % kOrderCand] = 0u;
     __syncthreads();
     {
         uint32_t mx = 0u;
@@ -142,37 +144,48 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
         if (lane == 0) atomicMax(&sh.top, mx);
     }
     __syncthreads();
+    if (t == 0) {
+        sh.cands = 0u;
+        sh.beat = 0u;
+    }
+    uint32_t base = 0u, h = 0u;  // hist[h] counts vertices by (base - degree)
     for (uint32_t done = 0; done < n;) {
         const uint32_t M = sh.top;
-        if (t == 0) {
-            sh.cands = 0u;
-            sh.beat = 0u;
+        // The pass that lowers the degrees also counts them for the next
+        // round, by the distance from this round's maximum, which no degree
+        // exceeds; counted anew where the maximum has fallen too far below it.
+        if (done == 0u || base - M > kOrderCand / 2u) {
+            base = M;
+            for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[h][i] = 0u;
+            __syncthreads();
+            for (uint32_t u = t; u < n; u += T) {
+                const uint32_t d = deg[u];
+                if (d != 0u && base - d < kOrderCand) atomicAdd(&sh.hist[h][base - d], 1u);
+            }
+            __syncthreads();
         }
-        for (uint32_t u = t; u < n; u += T) {
-            const uint32_t d = deg[u];
-            if (d != 0u && M - d < kOrderCand) atomicAdd(&sh.hist[M - d], 1u);
-        }
-        __syncthreads();
-        // degree classes M, M - 1, ... that fit together (every warp computes
-        // the same number)
+        const uint32_t above = base - M;  // leading classes without a vertex
+        // degree classes base, base - 1, ... that fit together (every warp
+        // computes the same number)
         uint32_t classes;
         {
-            const uint4 h = *reinterpret_cast<const uint4 *>(&sh.hist[4u * lane]);
-            const uint32_t s4 = h.x + h.y + h.z + h.w;
+            const uint4 hc = *reinterpret_cast<const uint4 *>(&sh.hist[h][4u * lane]);
+            const uint32_t s4 = hc.x + hc.y + hc.z + hc.w;
             uint32_t incl = s4;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(FULLM, incl, o);
                 incl += (int)lane >= o ? y : 0u;
             }
-            const uint32_t e = incl - s4, c0 = e + h.x, c1 = c0 + h.y, c2 = c1 + h.z, c3 = c2 + h.w;
+            const uint32_t e = incl - s4, c0 = e + hc.x, c1 = c0 + hc.y, c2 = c1 + hc.z, c3 = c2 + hc.w;
             classes = (c0 <= kOrderCand) + (c1 <= kOrderCand) + (c2 <= kOrderCand) + (c3 <= kOrderCand);
             classes = __reduce_add_sync(FULLM, classes);
         }
-        if (classes != 0u) {
+        const bool whole = classes > above;
+        if (whole) {
             for (uint32_t c = warp; c < chunks; c += NW) {
                 const uint32_t u = c * 32u + lane, d = u < n ? deg[u] : 0u;
-                const uint32_t in = __ballot_sync(FULLM, d != 0u && M - d < classes);
+                const uint32_t in = __ballot_sync(FULLM, d != 0u && base - d < classes);
                 if (in == 0u) continue;
                 uint32_t at = 0u;
                 if (lane == 0) at = atomicAdd(&sh.cands, (uint32_t)__popc(in));
@@ -200,6 +213,7 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
         }
         __syncthreads();
         const uint32_t m = sh.cands;
+        for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[h ^ 1u][i] = 0u;
         // their adjacency, four rows a warp at a time (16 loads in flight)
         {
             uint32_t wd[4], sf[4];  // word and bit of this lane's columns
@@ -243,7 +257,7 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
             }
             // the (degree + 1, 4095 - label) to beat; whole classes: any
             // degree above the classes taken
-            const uint32_t beat = classes != 0u ? ((M - classes < M ? M - classes : 0u) << 12) | 4095u : sh.beat;
+            const uint32_t beat = whole ? ((base - classes < base ? base - classes : 0u) << 12) | 4095u : sh.beat;
             // (a row that is not a simple graph's can take a degree field below
             // zero: the candidate is then picked out of turn, and nothing else)
             uint32_t picks = 0u, floor_key = 0u;  // the first pick always stands
@@ -273,6 +287,8 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
             if (lane == 0) {
                 sh.picks = picks;
                 sh.top = 0u;
+                sh.cands = 0u;
+                sh.beat = 0u;
             }
         }
         __syncthreads();
@@ -300,13 +316,15 @@ __device__ __forceinline__ void order_rounds(uint32_t n, uint32_t w, const uint3
                 if (d != 0u) {
                     d = d > dec[q] + 1u ? d - dec[q] : 1u;
                     deg[u] = (uint16_t)d;
+                    if (M - d < kOrderCand) atomicAdd(&sh.hist[h ^ 1u][M - d], 1u);
                 }
                 mx = d > mx ? d : mx;
             }
         }
         mx = __reduce_max_sync(FULLM, mx);
         if (lane == 0) atomicMax(&sh.top, mx);
-        for (uint32_t i = t; i < kOrderCand; i += T) sh.hist[i] = 0u;
+        base = M;
+        h ^= 1u;
         __syncthreads();
     }
 }
