@@ -296,13 +296,15 @@ Tuning mce::default_tuning()
         Tuning d{};  // 0: thresholds by density
         d.local_check = d.global_check = 1u;
         d.refresh_ns = 2000u;
-        // Served form: a request alone gets a block per 20,000 expected
-        // maximal cliques, and requests expecting up to 10^6 share
-        // micro-batches (on the served workload, 10,400 -> 11,300 requests/s
-        // closed loop and p99 6.3 -> 3.9 ms at 0.7x that load, against one
-        // block per 50,000 and micro-batches up to 10^5)
-        d.serve_cpb = 20000u;
-        d.serve_bcost = 1000u;
+        // Served form: a request alone gets a block per 10,000 expected
+        // maximal cliques, and requests expecting up to 3 10^5 share
+        // micro-batches.  The single search gained more from the warp tier
+        // than a batch's blocks, so larger requests go alone now: 46 requests
+        // at once 7.3 -> 3.7 ms, 256 16.4 -> 15.9, p99 at 0.7x the capacity
+        // 3.6 -> 2.2 ms, closed loop 13,700 -> 13,300 requests/s, against one
+        // block per 20,000 and micro-batches up to 10^6.
+        d.serve_cpb = 10000u;
+        d.serve_bcost = 300u;
         d.pop_tries = 16384u;
         // (2 us -> 1 us took 1 to 3 % off searches of up to 2 ms, G(106, 0.7)
         // 0.472 -> 0.456 ms, and nothing off longer ones)
