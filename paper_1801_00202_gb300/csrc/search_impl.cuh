@@ -507,16 +507,17 @@ __device__ __forceinline__ void flush_diag(const unsigned long long *diag, uint6
 // terms are exactly those of the search by frames; only who expands which
 // node differs.
 //
-// What bounds it: issue slots.  A step of 29 nodes takes about 340
-// instructions with four-word sets, the SM issues on 60 to 70 % of its
-// cycles, and the rest waits on the step's chain of shared-memory loads (frame
-// -> pivot row -> child row -> pivot row).  Building a subproblem costs about
-// as much as 300 nodes.  Before, a warp searched 32 subproblems of at most 32
-// vertices, each by one lane with a stack of its own, and everything above 32
-// vertices a node per warp; now against then, ms: G(1000, 0.3) 3.2 / 5.8,
-// G(500, 0.5) 9.6 / 21.4, G(300, 0.5) 1.3 / 2.0, Moon-Moser 45 0.66 / 0.86,
-// G(45, 0.5) 0.052 / 0.10, G(100, 0.8) 1.1 / 2.6.  It loses where a search is
-// nothing but subproblems of ten nodes or so (G(700, 0.18) 0.49 / 0.45).
+// What bounds it: a step of 29 nodes takes about 340 instructions with
+// four-word sets, most of them in one chain (scan of the children counts,
+// frame -> pivot row -> child row -> pivot row from shared memory); the SM
+// issues on a third of its cycles, and the rest are that chain's latencies and
+// fetches of instructions.  Building a subproblem costs about as much as 300
+// nodes.  Before, a warp searched 32 subproblems of at most 32 vertices, each
+// by one lane with a stack of its own, and everything above 32 vertices a node
+// per warp; now against then, ms: G(1000, 0.3) 2.9 / 5.8, G(500, 0.5) 9.6 /
+// 21.4, G(300, 0.5) 1.2 / 2.0, Moon-Moser 45 0.63 / 0.85, G(45, 0.5) 0.045 /
+// 0.125, G(100, 0.8) 1.0 / 1.5.  It gains least where a search is nothing but
+// subproblems of ten nodes or so (G(700, 0.18) 0.46 / 0.45).
 //
 // Graphs of at most 128 vertices need no compression: their rows (and hash
 // terms) are laid out once per block and every frame goes to the warp tier as
