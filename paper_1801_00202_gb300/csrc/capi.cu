@@ -363,6 +363,7 @@ SearchParams params(uint32_t n, const Config &c, const Layout &L, unsigned char 
     p.fs = c.fs;
     p.out = out;
     p.timeout_ns = o.timeout_ns ? o.timeout_ns : 60ull * 1000000000ull;
+    p.limit_ns = total_limit(p.timeout_ns);
     p.total_groups = c.total_groups;
     p.pivot_mode = (uint32_t)c.pivot;
     p.stack_levels = o.stack_levels ? std::min<uint32_t>(o.stack_levels, kStackDepth) : kStackDepth;
@@ -1807,6 +1808,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
             bp.qcap = bk.qcap;
             bp.fs = bk.fs;
             bp.timeout_ns = o.timeout_ns ? o.timeout_ns : 60ull * 1000000000ull;
+            bp.limit_ns = total_limit(bp.timeout_ns);
             bp.pivot_mode = o.pivot_mode;
             bp.stack_levels = o.stack_levels ? std::min<uint32_t>(o.stack_levels, kStackDepth) : kStackDepth;
             bp.groups_per_block = bk.groups;

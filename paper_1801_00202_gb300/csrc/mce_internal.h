@@ -140,6 +140,13 @@ constexpr uint32_t kDirectBytes = kDirectRows * 4 + kDirectVerts * 10;
 // 18.4.  (576 and 608 threads: slower than the better of the two everywhere.)
 constexpr unsigned kLaunchThreads = 768u, kShortThreads = 512u;
 
+// Longest run of a search: ten times its wait budget (the largest value, no
+// limit, where that does not fit).
+inline uint64_t total_limit(uint64_t timeout_ns)
+{
+    return timeout_ns > UINT64_MAX / 10u ? UINT64_MAX : 10u * timeout_ns;
+}
+
 struct SearchParams {
     uint32_t n;             // vertices
     uint32_t wp;            // words per renumbered row (= lanes * words/lane)
@@ -151,7 +158,8 @@ struct SearchParams {
     uint32_t qcap;          // power of two
     uint32_t fs;            // frame stride in words
     uint64_t *out;          // MCE_OUT_WORDS(n) words
-    uint64_t timeout_ns;
+    uint64_t timeout_ns;    // longest time without progress
+    uint64_t limit_ns;      // longest time in all (total_limit)
     uint32_t total_groups;
     uint32_t pivot_mode;
     uint32_t stack_levels;  // <= kStackDepth
@@ -227,7 +235,7 @@ struct BatchParams {
     unsigned char *qbase;   // per-block queue regions
     size_t qstride;         // bytes per region
     uint32_t qcap, fs;      // slots per region, frame stride (words)
-    uint64_t timeout_ns;
+    uint64_t timeout_ns, limit_ns;
     uint32_t pivot_mode, stack_levels, groups_per_block;
     uint32_t split_min_p, split_target;
     Tuning tune;

@@ -1277,6 +1277,8 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
 
     uint64_t quiet_since = 0, t_busy = 0;
     const uint64_t t_start = global_ns();
+    // (~0: none, also where the sum does not fit)
+    const uint64_t deadline = prm.limit_ns < ~0ull - t_start ? t_start + prm.limit_ns : ~0ull;
     unsigned last_pend = 0xffffffffu, last_head = 0xffffffffu;
     unsigned backoff = 64;
 
@@ -1521,7 +1523,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
             a.hash = at.region + po.hash;
             a.pos = at.region + po.pos;
         }
-        pool_run_class<K, PIVOT>(th.cls, a, pslots, prm.pool_bytes, prm.out, t_start + 10ull * prm.timeout_ns, c);
+        pool_run_class<K, PIVOT>(th.cls, a, pslots, prm.pool_bytes, prm.out, deadline, c);
         cn.cnt += c.cnt;
         cn.intl += c.intl;
         cn.dead += c.dead;
@@ -1674,7 +1676,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
                     } else if (now - quiet_since > prm.timeout_ns) {
                         set_status(prm.out, ctl, MCE_ETIMEOUT);
                     }
-                    if (now - t_start > 10ull * prm.timeout_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
+                    if (now - t_start > prm.limit_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
                     if (prm.trace) {
                         const unsigned ti = atomicAdd(&h->trace_n, 1u);
                         if (ti < prm.trace_per_block) {
@@ -1811,7 +1813,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
                         vst(&h->g_tail, ld_relaxed(&ctl->tail));
                         vst(&h->g_starving, ld_relaxed(&ctl->starving));
                         if (ab) vst(&h->done, 2u);
-                        if (now - t_start > 10ull * prm.timeout_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
+                        if (now - t_start > prm.limit_ns) set_status(prm.out, ctl, MCE_ETIMEOUT);
                         *reinterpret_cast<volatile unsigned long long *>(&h->stamp) = now;
                         atomicExch(&h->refreshing, 0u);
                     }
@@ -2249,6 +2251,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
         prm.fs = bp.fs;
         prm.out = gd.out;
         prm.timeout_ns = bp.timeout_ns;
+        prm.limit_ns = bp.limit_ns;
         prm.total_groups = bp.groups_per_block;
         prm.pivot_mode = bp.pivot_mode;
         prm.stack_levels = bp.stack_levels;
