@@ -1388,7 +1388,7 @@ struct Bucket {
     uint32_t split_graphs = 0;
     SearchImpl plain{nullptr, nullptr, nullptr, nullptr}, impl{nullptr, nullptr, nullptr, nullptr};
     LaunchShape shape{};
-    uint32_t qcap = 0, fs = 0, groups = 0;
+    uint32_t qcap = 0, fs = 0, groups = 0, root_frames = 0;
     uint32_t t2_offset = 0, pool_bytes = 0, t2_max_p = 0, direct_offset = 0;  // warp tier (t2_max_p 0: off)
     uint32_t cls = 1;  // its words per set, for all graphs of the bucket
     size_t qstride = 0, list_off = 0, region_off = 0, next_off = 0;
@@ -1429,12 +1429,13 @@ uint32_t words_class(uint32_t n)
 // expected number of root children (|P \ N(pivot)| ~ n(1 - p)), by
 // kBatchMaxParts and by the kernel's prefix table (kBatchPartWords words per
 // row); subproblems of the outer loop are never split.  Items are sorted by
-// expected cost, largest first.  Returns the most child frames one part
-// queues at its start (0 when nothing is split), which the ring must hold.
+// expected cost, largest first.  Returns the most child frames one item
+// queues at its start, which the ring must hold: all of a part's, and of a
+// whole graph's at most `whole` (the last of them carries the other children).
 constexpr uint32_t kBatchMaxParts = 64;
 
 uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<double> &cost,
-                    const std::vector<uint32_t> &wp_of, unsigned blocks, uint32_t div)
+                    const std::vector<uint32_t> &wp_of, unsigned blocks, uint32_t div, uint32_t whole)
 {
     double total = 0.0;
     for (uint32_t i : bk.graphs) total += cost[i];
@@ -1451,10 +1452,8 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
             k = (uint32_t)std::min(cap, std::ceil(cost[i] / target));
         }
         for (uint32_t j = 0; j < k; ++j) items.push_back({cost[i] / k, i | (j << 16) | (k << 24)});
-        if (!g->root) frames = std::max(frames, (g->n + k - 1) / k + 1);
-        if (k >= 2) {
-            ++bk.split_graphs;
-        }
+        if (!g->root) frames = std::max(frames, k >= 2 ? (g->n + k - 1) / k + 1 : std::min(g->n + 1, whole));
+        if (k >= 2) ++bk.split_graphs;
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, uint32_t> &a, const std::pair<double, uint32_t> &c) {
@@ -1464,6 +1463,12 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
     for (auto &it : items) bk.items.push_back(it.second);
     return frames;
 }
+
+// Slots of a block's ring that may be there for the children of whole graphs'
+// roots.  Every block of the grid has a ring: one slot a child would take 1.3
+// GB on 152 blocks at 4,096 vertices, against 41 MB, and is slower (a batch of
+// 700 G(512, 0.3) 133.9 / 116.0 ms, 640 G(2000, 0.05) 56.0 / 30.1 ms).
+constexpr uint32_t kRootSlots = 256;
 
 // Launch choice of a batched graph without a tuned one: forced shapes as
 // given, otherwise the most threads a block can have (a batched graph has no
@@ -1711,11 +1716,16 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         int per_sm = 0;
         if (bk.impl.batch_occupancy((int)threads, smem, &per_sm) != cudaSuccess || per_sm < 1) { rc = MCE_EINVAL; break; }
         unsigned blocks = o.blocks ? o.blocks : (unsigned)(per_sm * sms);
-        const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, blocks, default_tuning().batch_split);
+        bk.groups = threads / 32;
+        // room for frames given away while the queued ones wait
+        const uint32_t slack = 4u * bk.groups + 64u;
+        static_assert(4u * (kLaunchThreads / 32u) + 64u < kRootSlots, "room for some children");
+        const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, blocks, default_tuning().batch_split,
+                                                kRootSlots - slack);
         blocks = std::min<unsigned>(blocks, (unsigned)bk.items.size());
         bk.shape = LaunchShape{blocks, threads, smem};
-        bk.groups = threads / 32;
-        bk.qcap = next_pow2(std::max<uint64_t>(256, 4ull * bk.groups + 64 + part_frames));
+        bk.qcap = next_pow2(std::max<uint32_t>(kRootSlots, slack + part_frames));
+        bk.root_frames = bk.qcap - slack;
         if (o.queue_log2) bk.qcap = std::max<uint32_t>(bk.qcap, 1u << o.queue_log2);
         bk.fs = (uint32_t)frame_words((uint32_t)(bk.G * bk.K));  // the widest rows' frames
         bk.qstride = batch_region_bytes(bk.qcap, bk.fs);
@@ -1806,6 +1816,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
             bp.qbase = base + bk.region_off;
             bp.qstride = bk.qstride;
             bp.qcap = bk.qcap;
+            bp.root_frames = bk.root_frames;
             bp.fs = bk.fs;
             bp.timeout_ns = o.timeout_ns ? o.timeout_ns : 60ull * 1000000000ull;
             bp.limit_ns = total_limit(bp.timeout_ns);

@@ -235,6 +235,7 @@ struct BatchParams {
     unsigned char *qbase;   // per-block queue regions
     size_t qstride;         // bytes per region
     uint32_t qcap, fs;      // slots per region, frame stride (words)
+    uint32_t root_frames;   // frames of a whole graph's root children, at most
     uint64_t timeout_ns, limit_ns;
     uint32_t pivot_mode, stack_levels, groups_per_block;
     uint32_t split_min_p, split_target;

@@ -2180,11 +2180,11 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
                 lne = lne || (frames[kFrameHdr + w] & ~gd.ren[(size_t)p0 * WP + w]) != 0u;
         lne = __syncthreads_or(lne) != 0;
         const bool root = valid && pne && lne;
-        // a part queues one frame per root child of the part instead of the
-        // root frame: child t branches on the t-th vertex v_t of L = P \ N(p0)
+        // one frame per root child of the part: child t branches on the t-th vertex v_t of L = P \ N(p0)
         // with v_1..v_{t-1} already in X, i.e. the frame (P minus those, X =
         // those, p0, end = v_t + 1); frames go to slots 1.. (slot 0 keeps the
-        // root frame's layout)
+        // root's P and X).  A whole graph with more children than the ring has
+        // room for queues the rest as one frame (end = n).
         unsigned queued = root ? 1u : 0u;
         if (split) {
             __shared__ unsigned lpre[kBatchPartWords + 1];
@@ -2199,7 +2199,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
             }
             __syncthreads();
             const unsigned nl = lpre[WP];
-            const unsigned mine = nl > part ? (nl - part + parts - 1u) / parts : 0u;
+            const unsigned mine = parts == 1u ? min(nl, bp.root_frames) : (nl > part ? (nl - part + parts - 1u) / parts : 0u);
             for (unsigned j = threadIdx.x; j < mine && j + 1u < bp.qcap; j += blockDim.x) {
                 const unsigned t = part + j * parts;
                 unsigned w = 0;
@@ -2217,7 +2217,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
                     fr[kFrameHdr + q] = pw & ~x;
                     fr[kFrameHdr + WP + q] = x;
                 }
-                fr[0] = (p0 & 0xffffu) | ((v + 1u) << 16);
+                fr[0] = (p0 & 0xffffu) | ((parts == 1u && j + 1u == mine ? n : v + 1u) << 16);
                 fr[1] = 0u;
                 fr[2] = 0u;
                 fr[3] = 0u;
@@ -2228,8 +2228,8 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
                 atomicCAS(reinterpret_cast<unsigned long long *>(gd.out + MCE_OUT_STATUS), 0ull,
                           static_cast<unsigned long long>(static_cast<long long>(MCE_EOVERFLOW)));
         }
-        // ring state: the root frame is consumer ticket 0 in slot 0; a part's
-        // frames are consumer tickets 1..queued in slots 1..queued (slot 0 is
+        // ring state: a subproblem's root frame is consumer ticket 0 in slot 0;
+        // root children are consumer tickets 1..queued in slots 1..queued (slot 0 is
         // then free for producer ticket qcap)
         for (uint32_t j = threadIdx.x; j < bp.qcap; j += blockDim.x) {
             unsigned sv = j;
