@@ -1427,15 +1427,17 @@ uint32_t words_class(uint32_t n)
 // subtrees of Alg. 4's root), so the heaviest graphs of a batch no longer run
 // on one block while the others idle.  k is capped by about half the
 // expected number of root children (|P \ N(pivot)| ~ n(1 - p)), by
-// kBatchMaxParts and by the kernel's prefix table (kBatchPartWords words per
+// kBatchMaxParts, by kPartCliques expected cliques a part and by the kernel's prefix table (kBatchPartWords words per
 // row); subproblems of the outer loop are never split.  Items are sorted by
 // expected cost, largest first.  Returns the most child frames one item
 // queues at its start, which the ring must hold: all of a part's, and of a
-// whole graph's at most `whole` (the last of them carries the other children).
+// whole graph's at most `whole` (a frame then carries several children).
 constexpr uint32_t kBatchMaxParts = 64;
+constexpr double kPartCliques = 2000.0;  // (a part takes some 20 us before its search: 160 G(850, 0.04) 2.8 -> 1.9 ms)
 
 uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<double> &cost,
-                    const std::vector<uint32_t> &wp_of, unsigned blocks, uint32_t div, uint32_t whole)
+                    const std::vector<uint32_t> &wp_of, std::vector<uint32_t> &parts_of, unsigned blocks, uint32_t div,
+                    uint32_t whole)
 {
     double total = 0.0;
     for (uint32_t i : bk.graphs) total += cost[i];
@@ -1448,12 +1450,13 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
         if (!g->root && target > 0.0 && cost[i] > 2.0 * target && wp_of[i] <= (uint32_t)kBatchPartWords && g->n > 1) {
             const double p = std::min(1.0, 2.0 * (double)g->m / ((double)g->n * (g->n - 1.0)));
             const double children = 0.5 * g->n * (1.0 - p);
-            const double cap = std::min<double>(kBatchMaxParts, std::max(1.0, children));
+            const double cap = std::min<double>(kBatchMaxParts, std::max(1.0, std::min(children, cost[i] / kPartCliques)));
             k = (uint32_t)std::min(cap, std::ceil(cost[i] / target));
         }
         for (uint32_t j = 0; j < k; ++j) items.push_back({cost[i] / k, i | (j << 16) | (k << 24)});
         if (!g->root) frames = std::max(frames, k >= 2 ? (g->n + k - 1) / k + 1 : std::min(g->n + 1, whole));
         if (k >= 2) ++bk.split_graphs;
+        parts_of[i] = k;
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, uint32_t> &a, const std::pair<double, uint32_t> &c) {
@@ -1469,6 +1472,47 @@ uint32_t plan_items(Bucket &bk, mce_graph *const *graphs, const std::vector<doub
 // GB on 152 blocks at 4,096 vertices, against 41 MB, and is slower (a batch of
 // 700 G(512, 0.3) 133.9 / 116.0 ms, 640 G(2000, 0.05) 56.0 / 30.1 ms).
 constexpr uint32_t kRootSlots = 256;
+
+// Words per set of the warp tier that a batched graph asks for: the first
+// level of the search tree whose P u X has at most 128 vertices in
+// expectation (n p^k at level k), with room for all of its frames; below the
+// root's children only in sparse graphs (p < 0.2), whose next level is far
+// smaller; elsewhere four words, which take subproblems higher up.  A bucket
+// has the largest of its graphs' sizes, so that one instance of the code stays
+// in the instruction caches (sizes mixed within a batch: 1 to 4 % slower).
+// Batches of alike sparse graphs with four words -> this, ms: 700 G(160, 0.04)
+// 1.73 -> 1.57, 160 G(1700, 0.1) 90.5 -> 60.9, 700 G(300, 0.1) 3.54 -> 3.16.
+uint32_t pool_words(uint32_t n, uint64_t m)
+{
+    if (n <= 128u) return std::max<uint32_t>(1u, (n + 31u) / 32u);
+    const double p = std::min(0.95, 2.0 * (double)m / ((double)n * (n - 1.0)));
+    double size = n, pk = 1.0;
+    int level = 0;
+    for (; size > 128.0; ++level) {
+        size *= p;
+        pk *= p;
+    }
+    if (level > 1 && p >= 0.2) return 4u;
+    size += (level > 1 ? 2.0 : 3.0) * std::sqrt(size * (1.0 - pk));
+    return (uint32_t)std::min(4.0, size / 32.0 + 1.0);
+}
+
+// Root children per frame of a batched graph that a block of `warps` warps
+// searches in `parts` parts.  A frame costs its warp some 10 us (a ticket, the
+// frame from L2, a subproblem searched by itself), so a frame holds children
+// of about kFrameCliques expected maximal cliques in all, whose subproblems
+// are searched side by side; but there is a frame for every warp.  A child a
+// frame -> this, ms: 700 G(160, 0.07) 1.91 -> 1.59, 700 G(300, 0.07) 3.0 -> 2.4,
+// 160 G(1700, 0.1) 57 -> 42, 512 mixed graphs 12.5 -> 11.6.
+constexpr double kFrameCliques = 4000.0;
+
+uint32_t children_per_frame(uint32_t n, uint64_t m, double cliques, uint32_t parts, uint32_t warps)
+{
+    const double children = n > 1 ? n - 2.0 * (double)m / n : 1.0;  // |V \ N(pivot)|, about
+    const double each = std::max(cliques / std::max(children, 1.0), 1e-3);
+    const double frames = (double)warps * parts;
+    return (uint32_t)std::max(1.0, std::floor(std::min(children / frames, kFrameCliques / each)));
+}
 
 // Launch choice of a batched graph without a tuned one: forced shapes as
 // given, otherwise the most threads a block can have (a batched graph has no
@@ -1629,7 +1673,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
     std::vector<Bucket> buckets;
     std::vector<double> cost(count);
     uint32_t max_n = 0, max_w = 0, max_wp = 0;
-    std::vector<uint32_t> wp_of(count);
+    std::vector<uint32_t> wp_of(count), parts_of(count, 1), groups_of(count, 1);
     for (uint32_t i = 0; i < count; ++i) {
         const mce_graph *g = graphs[i];
         if (!g || g->ctx != ctx || !g->d_rows) { delete b; return MCE_EINVAL; }
@@ -1711,16 +1755,18 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         bk.threads = threads;
         bk.pool_bytes = plan_pool(bk.t2_offset, threads, std::max<size_t>((slimit + 2048) * threads / kLaunchThreads - 2048, bk.t2_offset));
         bk.t2_max_p = default_tuning().t2_p;
-        bk.cls = std::min<uint32_t>(words, kPoolMaxP / 32);
+        bk.cls = 1;
+        for (uint32_t i : bk.graphs) bk.cls = std::max(bk.cls, pool_words(b->n[i], graphs[i]->m));
         const size_t smem = bk.t2_offset + (threads / 32) * bk.pool_bytes;
         int per_sm = 0;
         if (bk.impl.batch_occupancy((int)threads, smem, &per_sm) != cudaSuccess || per_sm < 1) { rc = MCE_EINVAL; break; }
         unsigned blocks = o.blocks ? o.blocks : (unsigned)(per_sm * sms);
         bk.groups = threads / 32;
+        for (uint32_t i : bk.graphs) groups_of[i] = bk.groups;
         // room for frames given away while the queued ones wait
         const uint32_t slack = 4u * bk.groups + 64u;
         static_assert(4u * (kLaunchThreads / 32u) + 64u < kRootSlots, "room for some children");
-        const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, blocks, default_tuning().batch_split,
+        const uint32_t part_frames = plan_items(bk, graphs, cost, wp_of, parts_of, blocks, default_tuning().batch_split,
                                                 kRootSlots - slack);
         blocks = std::min<unsigned>(blocks, (unsigned)bk.items.size());
         bk.shape = LaunchShape{blocks, threads, smem};
@@ -1766,7 +1812,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         t.n = b->n[i];
         t.w = graphs[i]->w;
         t.wp = wp_of[i];
-        t.pad = 0;
+        t.per = children_per_frame(t.n, graphs[i]->m, cost[i], parts_of[i], groups_of[i]);
         t.label = graphs[i]->label;
         t.root = graphs[i]->root;
         t.rv = graphs[i]->rv;

@@ -190,7 +190,8 @@ struct BatchGraph {
     uint32_t *order;        // n entries
     uint32_t *ren;          // n * wp renumbered words (+ pad to 16 B)
     uint64_t *out;          // MCE_OUT_WORDS(n) words
-    uint32_t n, w, wp, pad;
+    uint32_t n, w, wp;
+    uint32_t per;           // root children per queued frame (at least 1)
     // Subproblem of the outer loop (Alg. 3), else null / 0: label[i] is the
     // original label of local vertex i (hashes and sizes use it); root holds
     // the root's P then X as bitsets over local vertices (w words each); the

@@ -135,9 +135,13 @@ __device__ __forceinline__ Thresholds density_thresholds(unsigned deg_sum, uint3
         // code: 512 graphs of 32 to 512 vertices took 17.7 ms with the limits
         // of a graph searched alone, 13.0 with 128 vertices as the limit and
         // four words above 128 vertices, 12.5 with four words throughout.
+        // Dense graphs, two thirds of the vertices (a third, as alone / a half /
+        // two thirds / all, ms, 700 graphs: G(64, 0.8) 18.3 / 7.2 / 7.2 / 6.6,
+        // G(50, 0.9) 10.5 / 6.5 / 4.2 / 4.8, Moon-Moser 36 10.2 / 10.2 / 9.2 /
+        // 9.2, 160 G(130, 0.75) 178 / 145 / 145 / 146).
         if (batch_cls) {
             t.cls = batch_cls;
-            if (i < 30) t.task = 128u;
+            t.task = i < 30 ? 128u : max(20u, 2u * n / 3u);
         }
     }
     if (tune.share_local) t.share = tune.share_local;
@@ -2180,11 +2184,11 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
                 lne = lne || (frames[kFrameHdr + w] & ~gd.ren[(size_t)p0 * WP + w]) != 0u;
         lne = __syncthreads_or(lne) != 0;
         const bool root = valid && pne && lne;
-        // one frame per root child of the part: child t branches on the t-th vertex v_t of L = P \ N(p0)
-        // with v_1..v_{t-1} already in X, i.e. the frame (P minus those, X =
-        // those, p0, end = v_t + 1); frames go to slots 1.. (slot 0 keeps the
-        // root's P and X).  A whole graph with more children than the ring has
-        // room for queues the rest as one frame (end = n).
+        // frames of `per` consecutive root children each: with v_t the t-th
+        // vertex of L = P \ N(p0), children a..b-1 are the frame (P minus v_0
+        // ..v_{a-1}, X = those, p0, end = v_b); a part takes every parts-th of
+        // them.  Frames go to slots 1.. (slot 0 keeps the root's P and X).
+        // per: what makes a frame worth taking, and what the ring has room for.
         unsigned queued = root ? 1u : 0u;
         if (split) {
             __shared__ unsigned lpre[kBatchPartWords + 1];
@@ -2199,14 +2203,20 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
             }
             __syncthreads();
             const unsigned nl = lpre[WP];
-            const unsigned mine = parts == 1u ? min(nl, bp.root_frames) : (nl > part ? (nl - part + parts - 1u) / parts : 0u);
-            for (unsigned j = threadIdx.x; j < mine && j + 1u < bp.qcap; j += blockDim.x) {
-                const unsigned t = part + j * parts;
+            unsigned per = gd.per;
+            if (parts == 1u) per = max(per, (nl + bp.root_frames - 1u) / bp.root_frames);
+            const unsigned all = (nl + per - 1u) / per;
+            const unsigned mine = all > part ? (all - part + parts - 1u) / parts : 0u;
+            auto child = [&](unsigned t) -> unsigned {  // v_t
                 unsigned w = 0;
                 while (w + 1u < WP && lpre[w + 1] <= t) ++w;
                 uint32_t lw = frames[kFrameHdr + w] & ~rp0[w];
                 for (unsigned r = t - lpre[w]; r > 0u; --r) lw &= lw - 1u;
-                const unsigned v = w * 32u + (unsigned)(__ffs(lw) - 1);
+                return w * 32u + (unsigned)(__ffs(lw) - 1);
+            };
+            for (unsigned j = threadIdx.x; j < mine && j + 1u < bp.qcap; j += blockDim.x) {
+                const unsigned t = (part + j * parts) * per;
+                const unsigned v = child(t), end = t + per < nl ? child(t + per) : n;
                 uint32_t *fr = frames + (size_t)(j + 1u) * bp.fs;
                 for (uint32_t q = 0; q < WP; ++q) {
                     const uint32_t pw = frames[kFrameHdr + q];
@@ -2217,7 +2227,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
                     fr[kFrameHdr + q] = pw & ~x;
                     fr[kFrameHdr + WP + q] = x;
                 }
-                fr[0] = (p0 & 0xffffu) | ((parts == 1u && j + 1u == mine ? n : v + 1u) << 16);
+                fr[0] = (p0 & 0xffffu) | (end << 16);
                 fr[1] = 0u;
                 fr[2] = 0u;
                 fr[3] = 0u;
