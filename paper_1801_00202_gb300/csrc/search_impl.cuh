@@ -74,7 +74,7 @@ struct Thresholds {
 // non-zero caller values win.  batch_cls != 0: one of a batch's graphs, which
 // share sets of that size.
 __device__ __forceinline__ Thresholds density_thresholds(unsigned deg_sum, uint32_t n, const Tuning &tune,
-                                                         unsigned fixed_split, unsigned batch_cls = 0u)
+                                                         unsigned fixed_split, bool scores, unsigned batch_cls = 0u)
 {
     Thresholds t{0xffffffffu, 0xffffffffu, 0xffffffffu, 128u, max(batch_cls, 1u)};
     if (n >= 2u) {
@@ -107,10 +107,16 @@ __device__ __forceinline__ Thresholds density_thresholds(unsigned deg_sum, uint3
             t.task = size < 21.5f ? kShareLocalByDensity[i - 1]
                                   : (size < 24.5f ? kShareGlobalByDensity[i - 1] : kSplitByDensity[i - 1]);
         // Set size of the warp tier: k levels below the root P u X has about
-        // n p^k vertices.  The first level of at most 112 (128 in a long
+        // n p^k vertices.  The first level of at most 102 (128 in a long
         // search, which has frames enough beside the larger half) gets the tier, or
         // the one below where the children of the root would hold more than
-        // about 600 cliques each (then they are too few and too uneven).
+        // about 256 cliques each (then they are too few and too uneven).  (At
+        // n p = 97 / 99 / 101 the four words for all children beat the level
+        // below, G(750, 0.13) 0.34 / 0.37, G(660, 0.15) 0.28 / 0.36, G(560, 0.18)
+        // 0.25 / 0.33 ms; at 103 / 104 / 106 too many children do not fit them,
+        // G(622, 0.165) 0.42 / 0.35, G(600, 0.174) 0.39 / 0.35, G(640, 0.165) 0.51 /
+        // 0.36.  With 600 cliques in place of 256: G(260, 0.32) 0.27 / 0.21, G(190,
+        // 0.44) 0.26 / 0.22, G(310, 0.32) under TomitaBB 0.34 / 0.28.)
         // Room for all of the level's frames: three standard deviations for
         // the children of the root, two below; none in dense graphs, where
         // one level further down still holds enough work per frame.  One
@@ -120,14 +126,27 @@ __device__ __forceinline__ Thresholds density_thresholds(unsigned deg_sum, uint3
         float sz = (float)n, pk = 1.0f;
         const float pf = pd < 0.95f ? pd : 0.95f;
         int level = 0;
-        const float most = size < 22.5f ? 112.0f : 128.0f;
-        while (sz > most || (level == 1 && size - __log2f((float)n) > 9.3f)) {
+        const float most = size < 22.5f ? 102.0f : 128.0f;
+        while (sz > most || (level == 1 && size - __log2f((float)n) > 8.0f)) {
             sz *= pf;
             pk *= pf;
             ++level;
         }
         if (level <= 1) sz += 3.0f * sqrtf(sz * (1.0f - pk));
         else if (pf < 0.48f) sz += 2.0f * sqrtf(sz * (1.0f - pk));
+        // Below the root's children two words at least, where rows are short
+        // (one word builds eight subproblems side by side, but gives up a level
+        // more often: G(640, 0.165) 0.39 / 0.36 ms, G(1000, 0.14) 0.58 / 0.55);
+        // rows of more than 32 words cost the build a load per word (G(1600,
+        // 0.1): one word 0.78, two 0.83).
+        if (level > 1 && n <= 1024u) sz = fmaxf(sz, 32.0f);
+        // Just above 128 vertices a search of up to 2^19 cliques has fewer
+        // frames on that level than the GPU has warps; subproblems of at most
+        // 32 vertices, one level further down, spread it.  Under rules that
+        // score pivots a node takes longer, and it pays up to 2^21.  Two words /
+        // one, ms: G(129, 0.56) 0.28 / 0.20, under TomitaBB 0.34 / 0.23, G(140,
+        // 0.62) 0.44 / 0.45, under TomitaBB 0.65 / 0.47.
+        if (level > 1 && n <= 160u && size < (scores ? 21.0f : 19.0f)) sz = 1.0f;
         t.cls = n <= 128u ? (n + 31u) / 32u : (unsigned)((sz + 32.0f) * (1.0f / 32.0f));
         t.cls = min(max(t.cls, 1u), 4u);
         // A batch has work for every warp without cutting subtrees small, and
@@ -2039,7 +2058,7 @@ __global__ void __launch_bounds__(T) search_kernel(const SearchParams prm)
 
 #pragma unroll 1
     for (uint32_t i = threadIdx.x; i <= n; i += blockDim.x) hist[i] = 0u;
-    const Thresholds th = density_thresholds(prm.ctl->pad3[0], n, prm.tune, prm.split_min_p);
+    const Thresholds th = density_thresholds(prm.ctl->pad3[0], n, prm.tune, prm.split_min_p, PIVOT != MCE_PIVOT_GREEDY);
     const uint32_t *rows = prm.rows;
     const bool direct = !LIST && K == 1 && n <= 128u && prm.t2_max_p != 0u;
     PoolAt at{};
@@ -2301,7 +2320,7 @@ __global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams
         // (the outer loop's subproblems of more than 128 vertices are sparse and
         // alike: the size that fits their children, several side by side.
         // G(10000, 0.03): 18.5 -> 15.7 ms on the device)
-        const Thresholds th = density_thresholds(root_key, n, bp.tune, bp.split_min_p, sub && n > 128u ? 0u : bp.cls);
+        const Thresholds th = density_thresholds(root_key, n, bp.tune, bp.split_min_p, PIVOT != MCE_PIVOT_GREEDY, sub && n > 128u ? 0u : bp.cls);
         const bool direct = K == 1 && n <= 128u && bp.t2_max_p != 0u;
         PoolAt at{};
         at.rows = bp.direct_offset;
