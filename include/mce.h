@@ -395,13 +395,12 @@ int mce_batch_create(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count,
  * classed by words per row (1, 2, 4, ..., 128).  Classes with a choice cached
  * in the context (per class and pivot rule) take it; the others, if they hold
  * at least 16 graphs of the batch, are tuned by coordinate descent in
- * decreasing order of expected work: every candidate for the class -- 128 /
- * 256 / 512 threads per block, then the best with the breadth-first split
- * off -- is
- * timed as one captured launch of the whole batch (up to 4096 of its graphs,
- * sampled evenly) with the other classes at their current choice, and the
- * fastest is kept and cached.  Classes with fewer graphs use the built-in
- * defaults.  Tuning runs inside mce_batch_create (seconds for thousands of
+ * decreasing order of expected work: the library's own choice, then 128 /
+ * 256 / 512 threads per block, then the best of them with the breadth-first
+ * split off are each timed as one captured launch of the whole batch (up to
+ * 4096 of its graphs, sampled evenly) with the other classes at their current
+ * choice; one that is faster by more than the timing's noise is kept, and the
+ * result cached.  Classes with fewer graphs use the built-in defaults.  Tuning runs inside mce_batch_create (seconds for thousands of
  * graphs); mce_batch_launch replays the chosen plan. */
 typedef struct {
     uint32_t words_class;        /* rows of at most this many 32-bit words  */

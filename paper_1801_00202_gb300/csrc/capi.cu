@@ -1514,18 +1514,28 @@ uint32_t children_per_frame(uint32_t n, uint64_t m, double cliques, uint32_t par
     return (uint32_t)std::max(1.0, std::floor(std::min(children / frames, kFrameCliques / each)));
 }
 
+// Threads per block of a batch without a tuned or forced choice (a batched
+// graph has no device-wide ring to spread its work: one block with all of an
+// SM's registers): 512 threads of 128 registers spill nothing above the warp
+// tier, and 768 of 80 have more warps for the tier, which long searches are
+// nearly all of.  768 / 512 threads, ms, by expected cliques a block: 64 mixed
+// graphs (7e4) 2.21 / 1.99, 160 G(220, 0.2) (3e4) 0.82 / 0.74, 160 G(300, 0.33)
+// (1.6e5) 2.84 / 3.14, 700 G(96, 0.6) (2.4e5) 3.1 / 3.9, 160 G(96, 0.7) (3.1e5) 3.8 /
+// 4.2, 512 mixed (5e5) 11.8 / 12.0; against the line, 256 mixed (2.5e5) 6.3 / 6.2.
+unsigned batch_threads(double cliques, unsigned blocks)
+{
+    return cliques >= 1.5e5 * std::max(blocks, 1u) ? kLaunchThreads : kShortThreads;
+}
+
 // Launch choice of a batched graph without a tuned one: forced shapes as
-// given, otherwise the most threads a block can have (a batched graph has no
-// device-wide ring to spread its work: one block with all of the SM's warps);
-// 256 for the outer loop's subproblems, most of which have fewer children than
-// that block has warps.
-TuneChoice default_choice(uint32_t n, const mce_options &o, bool wide)
+// given, otherwise `threads` (batch_threads, or 256 for the outer loop's
+// subproblems, most of which have fewer children than a block of more has
+// warps).
+TuneChoice default_choice(uint32_t n, const mce_options &o, unsigned threads)
 {
     TuneChoice t;
     pick_shape(n, o, t.G, t.K);
-    t.threads = o.threads_per_block ? o.threads_per_block : 256u;
-    if (wide && !o.lanes_per_subtree && !o.words_per_lane && !o.threads_per_block)
-        t.threads = kLaunchThreads;
+    t.threads = o.threads_per_block ? o.threads_per_block : (o.lanes_per_subtree || o.words_per_lane ? 256u : threads);
     t.split = o.split_min_p;
     return t;
 }
@@ -1555,12 +1565,12 @@ double time_choices(mce_ctx *ctx, const std::vector<mce_graph *> &graphs, const 
 }
 
 // Coordinate descent over the words classes that have no cached choice:
-// classes in decreasing order of expected work; for each, every candidate
-// (1, 2 or 4 words per lane with the fewest lanes that hold a row; 128, 256
-// or 512 threads; then the best with breadth-first split off) is timed on
-// the whole batch (up to 4096 of its graphs, sampled evenly) with the other
-// classes at their current choice, and the fastest is kept.
-void tune_batch(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, const mce_options &o,
+// classes in decreasing order of expected work; for each, the library's own
+// choice (`own` threads), then 128, 256 and 512 threads, then the best of them
+// with the breadth-first split off are timed on the whole batch (up to 4096 of
+// its graphs, sampled evenly) with the other classes at their current choice,
+// and one that beats those before it by more than the timing's noise is kept.
+void tune_batch(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, const mce_options &o, unsigned own,
                 const std::vector<double> &cost, std::map<uint32_t, TuneChoice> &choice)
 {
     std::map<uint32_t, double> work;
@@ -1585,12 +1595,13 @@ void tune_batch(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, const mc
             auto trial = choice;
             trial[c] = t;
             const double ms = time_choices(ctx, sample, o, trial);
-            if (ms >= 0.0 && (best_ms < 0.0 || ms < best_ms)) {
+            if (ms >= 0.0 && (best_ms < 0.0 || ms < 0.985 * best_ms)) {
                 best_ms = ms;
                 best = t;
             }
         };
-        for (unsigned threads : {128u, 256u, 512u}) {
+        for (unsigned threads : {own, 128u, 256u, 512u}) {
+            if (best_ms >= 0.0 && threads == own) continue;
             TuneChoice t;
             default_shape(32u * W, t.G, t.K);
             t.threads = threads;
@@ -1636,14 +1647,18 @@ extern "C" int mce_batch_create(mce_ctx *ctx, mce_graph *const *graphs, uint32_t
     const bool forced = o.lanes_per_subtree || o.words_per_lane || o.threads_per_block || o.split_min_p;
     if ((o.flags & MCE_AUTOTUNE) && !forced) {
         std::vector<double> cost(count);
+        double total = 0.0;
+        int sms = 1;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return MCE_ECUDA;
         for (uint32_t i = 0; i < count; ++i) {
             cost[i] = expected_cliques(graphs[i]->n, graphs[i]->m);
+            total += cost[i];
             const uint32_t key = words_class(graphs[i]->n) * 4u + o.pivot_mode;
             std::lock_guard<std::mutex> lk(ctx->tune_mu);
             auto it = ctx->tuned.find(key);
             if (it != ctx->tuned.end()) choice[words_class(graphs[i]->n)] = it->second;
         }
-        tune_batch(ctx, graphs, count, o, cost, choice);
+        tune_batch(ctx, graphs, count, o, batch_threads(total, o.blocks ? o.blocks : (unsigned)sms), cost, choice);
     }
     return batch_create_impl(ctx, graphs, count, o, choice, out);
 }
@@ -1672,20 +1687,23 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
     // defaults), buckets of equal choice, most expensive first
     std::vector<Bucket> buckets;
     std::vector<double> cost(count);
+    double total = 0.0;
     uint32_t max_n = 0, max_w = 0, max_wp = 0;
     std::vector<uint32_t> wp_of(count), parts_of(count, 1), groups_of(count, 1);
     for (uint32_t i = 0; i < count; ++i) {
         const mce_graph *g = graphs[i];
         if (!g || g->ctx != ctx || !g->d_rows) { delete b; return MCE_EINVAL; }
         cost[i] = g->cost_hint > 0.0 ? g->cost_hint : expected_cliques(g->n, g->m);
+        total += cost[i];
     }
+    const unsigned own_threads = subproblems ? 256u : batch_threads(total, o.blocks ? o.blocks : (unsigned)sms);
     for (uint32_t i = 0; i < count; ++i) {
         const mce_graph *g = graphs[i];
         b->n[i] = g->n;
         const uint32_t W = std::max<uint32_t>(1, (g->n + 31) / 32);
         const uint32_t wc = words_class(g->n);
         auto it = choice.find(wc);
-        const TuneChoice t = it != choice.end() ? it->second : default_choice(g->n, o, !subproblems);
+        const TuneChoice t = it != choice.end() ? it->second : default_choice(g->n, o, own_threads);
         const int G = t.G, K = t.K;
         const SearchImpl plain = impl_for(W, (int)o.pivot_mode);
         if ((uint32_t)(G * K) < W || !shape_known(G, K) || !plain.run) { delete b; return MCE_EINVAL; }

@@ -2089,8 +2089,8 @@ __global__ void __launch_bounds__(T) search_kernel(const SearchParams prm)
 // Per graph: output initialised with the root counted (status kept), rows
 // bulk-copied to shared memory, root frame queued, search, reduction into the
 // graph's own result array.
-template <int K, int PIVOT>
-__global__ void __launch_bounds__(kLaunchThreads) batch_kernel(const BatchParams bp)
+template <int K, int PIVOT, int T>
+__global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ unsigned cur, root_key;

@@ -50,18 +50,25 @@ cudaError_t occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 }
 
 template <int K, int PIVOT>
+auto batch_kernel_for(unsigned threads)
+{
+    return threads <= kShortThreads ? batch_kernel<K, PIVOT, kShortThreads> : batch_kernel<K, PIVOT, kLaunchThreads>;
+}
+
+template <int K, int PIVOT>
 cudaError_t run_batch_t(const BatchParams &bp, const LaunchShape &sh, cudaStream_t s)
 {
-    batch_kernel<K, PIVOT><<<sh.blocks, sh.threads, sh.smem, s>>>(bp);
+    batch_kernel_for<K, PIVOT>(sh.threads)<<<sh.blocks, sh.threads, sh.smem, s>>>(bp);
     return cudaGetLastError();
 }
 
 template <int K, int PIVOT>
 cudaError_t batch_occupancy_t(int threads, size_t smem, int *blocks_per_sm)
 {
-    cudaError_t e = kernel_smem_setup((const void *)batch_kernel<K, PIVOT>);
+    auto kernel = batch_kernel_for<K, PIVOT>((unsigned)threads);
+    cudaError_t e = kernel_smem_setup((const void *)kernel);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<K, PIVOT>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, threads, smem);
 }
 
 // The listing variant (LIST) has no batched form.
