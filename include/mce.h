@@ -131,9 +131,10 @@ typedef struct {
     uint32_t words_per_lane;    /* 32-bit words of a row a lane holds:
                                    1,2,4; 0 = by n                            */
     uint32_t blocks;            /* persistent grid size; 0 = one wave         */
-    uint32_t threads_per_block; /* 0 = 512, or 768 for long searches and
-                                   batches; a multiple of 32, at most 512
-                                   (else MCE_EINVAL)                          */
+    uint32_t threads_per_block; /* 0 = 512, or 768 for long searches of
+                                   mce_enumerate and mce_enumerate_part and
+                                   for batches of much work; a multiple of
+                                   32, at most 512 (else MCE_EINVAL)          */
     uint64_t timeout_ns;        /* device-side wait budget: a search whose
                                    idle warps see no progress for this long
                                    stops with MCE_ETIMEOUT; 0 = 60 s          */
@@ -141,8 +142,9 @@ typedef struct {
                                    frames spill to the device work queue,
                                    1..64; 0 = 64                              */
     uint32_t queue_log2;        /* log2 of the device work-queue slots, <= 24;
-                                   0 = auto (at least four times the warps).  mce_enumerate retries a search
-                                   that overflowed with a 16x larger queue.   */
+                                   0 = auto (at least four times the warps).
+                                   mce_enumerate retries a search that
+                                   overflowed with a 16x larger queue.        */
     uint32_t split_min_p;       /* a new subtree whose candidate set P has at
                                    least this many vertices is published to
                                    the device work queue (breadth-first
@@ -171,7 +173,7 @@ typedef struct {
 #define MCE_OUT_GROUPS    11   /* warps of the launch                        */
 #define MCE_OUT_GPUSH     12   /* frames published to the device-wide queue  */
 #define MCE_OUT_GTRY      13   /* claims of frames from it (one fetch-and-add
-                                  each, for up to four frames)              */
+                                  each, for one frame)                      */
 #define MCE_OUT_CAS_FAIL  14   /* lost compare-and-swap races on ticket
                                   counters (block-private rings of the
                                   batched form; the device-wide queue

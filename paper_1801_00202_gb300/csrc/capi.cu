@@ -90,7 +90,6 @@ struct Config {
     int pivot = 0;
     bool list = false;  // frames carry R (clique listing)
     uint32_t t2_offset = 0, pool_bytes = 0, t2_max_p = 0, direct_offset = 0;  // warp tier (t2_max_p 0: off)
-    uint32_t local_slots = kLocalSlots;  // block ring slots
     SearchImpl impl{nullptr, nullptr, nullptr, nullptr};
 };
 
@@ -225,7 +224,7 @@ int choose(uint32_t n, const mce_options &o, Config &c, bool long_run = false)
     // the regions do not fit.
     const Tuning tu = default_tuning();
     const uint32_t direct = n <= 128u ? kDirectBytes : 0u;
-    const size_t base = round_up(search_smem_bytes(n, c.wp, c.list, c.local_slots), 16) + direct;
+    const size_t base = round_up(search_smem_bytes(n, c.wp, c.list), 16) + direct;
     // (a listing search has no warp tier: a row of scratch for the pivot scores)
     const size_t region = c.list ? round_up((size_t)c.wp * 4, 16) : kPoolBytesMin;
     auto fits = [&](unsigned threads) { return base + (size_t)(threads / 32) * region <= limit; };
@@ -370,9 +369,6 @@ SearchParams params(uint32_t n, const Config &c, const Layout &L, unsigned char 
     p.split_min_p = o.split_min_p;  // 0: by density
     p.split_target = c.qcap / 2;
     p.tune = default_tuning();
-    // the breadth-first split of small graphs from 20 vertices pays in a
-    // full-wave launch of one graph; a grid sized for one served request
-    // (o.blocks) ran slower with it (10,800 -> 10,300 requests/s)
     p.trace = nullptr;
     p.trace_per_block = 0;
     if (g_trace && c.blocks) {
@@ -387,7 +383,6 @@ SearchParams params(uint32_t n, const Config &c, const Layout &L, unsigned char 
     p.pool_bytes = c.pool_bytes;
     p.t2_max_p = c.t2_max_p;
     p.direct_offset = c.direct_offset;
-    p.local_slots = c.local_slots;
     return p;
 }
 
@@ -1867,7 +1862,7 @@ int batch_create_impl(mce_ctx *ctx, mce_graph *const *graphs, uint32_t count, co
         cudaError_t ce = cudaMemsetAsync(b->d_out, 0, b->out_words * 8, s);
         for (const Bucket &bk : buckets)
             if (ce == cudaSuccess) ce = cudaMemsetAsync(base + bk.next_off, 0, 4, s);
-        if (ce == cudaSuccess) ce = launch_order_batch(d_table, count, max_n, order_smem, s);
+        if (ce == cudaSuccess) ce = launch_order_batch(d_table, count, order_smem, s);
         if (ce == cudaSuccess) ce = launch_renumber_batch(d_table, count, max_n, max_wp, s);
         if (ce == cudaSuccess) ce = cudaEventRecord(b->events[0], s);
         for (size_t i = 0; ce == cudaSuccess && i < buckets.size(); ++i) {

@@ -33,22 +33,18 @@ struct Ctl {
 };
 
 // Per-block frame ring in shared memory (the first level of the work
-// distribution): header, `slots` sequence numbers and `slots` frames, with
-// slots = kLocalSlots, or kLocalSlotsSmall where halving the ring buys a
-// warp of a plain search block (the planner decides).
-constexpr int kLocalSlots = 32;
+// distribution): header, kLocalSlots sequence numbers and as many frames.
+constexpr uint32_t kLocalSlots = 32;
 struct LocalHdr {
     unsigned head, tail;  // ring tickets
     unsigned idle;        // warps of this block without a frame
     unsigned bwork;       // busy warps + frames in the ring; the block holds
                           // one unit of Ctl::pending while this is non-zero
-    unsigned spare0;      // unused
     unsigned poller;      // a warp of this block is polling the global ring
     unsigned done;        // the search is over (1) or aborted (2)
     unsigned refreshing;  // a warp is refreshing the cached global state
     // cached global state (refreshed every few microseconds)
     unsigned g_head, g_tail, g_starving;
-    unsigned spare;       // unused (keeps the stamp 8-byte aligned)
     unsigned long long stamp;
     unsigned trace_n;     // timeline records written by this block
     unsigned give_p;      // warp tier: smallest |P| of a frame that is given away
@@ -57,7 +53,7 @@ struct LocalHdr {
     Ctl *ctl;
     unsigned *gseq;
     uint32_t *gframes;
-    unsigned qcap, fs, margin, wp, slots, n;
+    unsigned qcap, fs, margin, wp, n;
     unsigned give_mask, total;
     // work-distribution diagnostics of the block (rare events, shared-memory
     // atomics; added to the result array once the block is done)
@@ -70,9 +66,9 @@ __host__ __device__ inline size_t frame_words(uint32_t wp, bool list = false)
 {
     return (8 + (list ? 3 : 2) * (size_t)wp + 3) / 4 * 4;
 }
-__host__ __device__ inline size_t local_queue_bytes(uint32_t wp, bool list = false, uint32_t slots = kLocalSlots)
+__host__ __device__ inline size_t local_queue_bytes(uint32_t wp, bool list = false)
 {
-    return sizeof(LocalHdr) + (size_t)slots * 4 + (size_t)slots * frame_words(wp, list) * 4;
+    return sizeof(LocalHdr) + (size_t)kLocalSlots * 4 + (size_t)kLocalSlots * frame_words(wp, list) * 4;
 }
 
 // Clique listing (MCE_LIST).  Every group appends, at each maximal clique it
@@ -130,13 +126,13 @@ constexpr int kDirectRows = 512, kDirectVerts = 128;
 constexpr uint32_t kDirectBytes = kDirectRows * 4 + kDirectVerts * 10;
 
 // Most threads of a search block (the register bound of the kernels).  The
-// single-graph search is compiled for 768 threads (80 registers: the warp
-// tier's loop fits, the search by frames above it spills 200 words) and for
-// 512 (128 registers, nothing spilled).  Most searches spend enough of their
-// time above the warp tier for the latter, ms with 768 / 512 threads: G(100,
-// 0.5) 0.150 / 0.135, G(250, 0.4) 0.31 / 0.23, G(700, 0.18) 0.53 / 0.46,
-// G(1000, 0.3) 3.2 / 2.9, G(3000, 0.1) 3.0 / 2.6.  A long search is nearly all
-// warp tier and wants the warps: G(500, 0.5) 9.6 / 10.3, G(100, 0.9) 16.1 /
+// single-graph search and the batch kernel are compiled for 768 threads (80
+// registers: the warp tier's loop fits, the search by frames above it spills
+// 200 words) and for 512 (128 registers, nothing spilled).  Most searches spend
+// enough of their time above the warp tier for the latter, ms with 768 / 512
+// threads: G(100, 0.5) 0.150 / 0.135, G(250, 0.4) 0.31 / 0.23, G(700, 0.18) 0.53 /
+// 0.46, G(1000, 0.3) 3.2 / 2.9, G(3000, 0.1) 3.0 / 2.6.  A long search is nearly
+// all warp tier and wants the warps: G(500, 0.5) 9.6 / 10.3, G(100, 0.9) 16.1 /
 // 18.4.  (576 and 608 threads: slower than the better of the two everywhere.)
 constexpr unsigned kLaunchThreads = 768u, kShortThreads = 512u;
 
@@ -180,7 +176,6 @@ struct SearchParams {
     // (a multiple of 16) and the largest |P| of a subproblem (0: the tier is off)
     uint32_t t2_offset, pool_bytes, t2_max_p;
     uint32_t direct_offset;  // byte offset of the whole-graph layout (n <= 128)
-    uint32_t local_slots;   // slots of the block ring (kLocalSlots or kLocalSlotsSmall)
     uint32_t prepared;      // result array, queue and root frames are in place: the search alone is launched
 };
 
@@ -259,8 +254,8 @@ struct LaunchShape {
 };
 
 // One search: init kernel (root frame, queue, zeroed output) + persistent
-// search kernel, and its occupancy query.  Defined per (lanes, words)
-// instantiation in search_gN.cu.
+// search kernel, and its occupancy query.  Defined per words of a lane in
+// search_kN.cu and search_list_kN.cu.
 struct SearchImpl {
     cudaError_t (*run)(const SearchParams &, const LaunchShape &, cudaStream_t);
     cudaError_t (*occupancy)(int threads, size_t smem, int *blocks_per_sm);
@@ -277,7 +272,6 @@ SearchImpl search_list_impl_1(int pivot);
 SearchImpl search_list_impl_2(int pivot);
 SearchImpl search_list_impl_4(int pivot);
 
-
 // The root's children as independent subtrees (split.cu).  The root's
 // branching set is L = V \ N(p0) (p0 = root_pivot, or position 0 when null)
 // over the renumbered rows; child t branches on its t-th vertex v_t with
@@ -291,13 +285,13 @@ cudaError_t launch_root_children(const uint32_t *rows, uint32_t n, uint32_t wp, 
 cudaError_t launch_part_frames(const SearchParams &prm, const unsigned *root_pivot, cudaStream_t s);
 // Queue every root child as its own frame (after search_init_kernel left the
 // queue empty): frame t in slot t, tail = pending = |L|.  prm.qcap >= n.
+cudaError_t launch_seed_children(const SearchParams &prm, const unsigned *root_pivot, cudaStream_t s);
 // Everything before the search (see small_prep_kernel), for graphs and rows
 // that small_prep_fits accepts: order and rows receive the order and the
 // renumbered rows.
 bool small_prep_fits(uint32_t n, uint32_t w, uint32_t wp);
 cudaError_t launch_small_prep(const SearchParams &prm, uint32_t w, const uint32_t *rows_in, uint32_t *order,
                               uint32_t *rows, cudaStream_t s);
-cudaError_t launch_seed_children(const SearchParams &prm, const unsigned *root_pivot, cudaStream_t s);
 // TomitaBB's root pivot (the earliest vertex of maximum degree) to *dst.
 cudaError_t launch_root_degree_pivot(const uint32_t *rows, uint32_t n, uint32_t wp, unsigned *dst, cudaStream_t s);
 
@@ -314,20 +308,20 @@ cudaError_t launch_renumber(uint32_t n, uint32_t w, const uint32_t *rows, const 
 // Batched preprocessing over a device table of graphs (max_n / max_w / max_wp
 // bound every entry).  prepare_* sets kernel attributes (call before capture).
 cudaError_t prepare_order_batch(uint32_t max_n, uint32_t max_w, size_t *smem);
-cudaError_t launch_order_batch(const BatchGraph *graphs, uint32_t count, uint32_t max_n, size_t smem,
-                               cudaStream_t s);
+cudaError_t launch_order_batch(const BatchGraph *graphs, uint32_t count, size_t smem, cudaStream_t s);
 cudaError_t launch_renumber_batch(const BatchGraph *graphs, uint32_t count, uint32_t max_n, uint32_t max_wp,
                                   cudaStream_t s);
 
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Raise a kernel's dynamic shared-memory limit to the device maximum and
-// prefer the largest shared-memory carveout, once per (kernel, device).  Every
-// launch after that runs under the same settings, so kernels of different
-// requests on different streams never wait for one another to change them.
+// prefer the largest shared-memory carveout, once per (kernel, device): kernels
+// that ask for the same carveout run beside one another without a change of it.
 // prefer_l1 (the single-graph search of up to 512 threads): the carveout is
 // left to the driver, and the rows stay in L1 where the blocks leave room
-// (listing G(700, 0.3) 4.5 -> 4.1 ms, counting G(1000, 0.3) 3.11 -> 2.91).
+// (listing G(700, 0.3) 4.5 -> 4.1 ms, counting G(1000, 0.3) 3.11 -> 2.91).  Served
+// requests searched alone then run beside micro-batches of another carveout;
+// the largest for both was slower all the same (24 to 256 requests: 0.97x).
 cudaError_t kernel_smem_setup(const void *func, bool prefer_l1 = false);
 
 // Listing post-pass (listing.cu): record chunks of a finished listing search
@@ -356,9 +350,8 @@ Tuning default_tuning();
 //   [hist: (n + 1) x u32, padded to 16 B][local frame ring]
 //   [whole-graph layout (n <= 128)][warp regions]
 __host__ __device__ inline size_t smem_local_offset(uint32_t n) { return (((size_t)n + 1) * 4 + 15) / 16 * 16; }
-__host__ __device__ inline size_t search_smem_bytes(uint32_t n, uint32_t wp, bool list = false,
-                                                   uint32_t slots = kLocalSlots)
+__host__ __device__ inline size_t search_smem_bytes(uint32_t n, uint32_t wp, bool list = false)
 {
-    return smem_local_offset(n) + local_queue_bytes(wp, list, slots);
+    return smem_local_offset(n) + local_queue_bytes(wp, list);
 }
 }  // namespace mce

@@ -618,9 +618,8 @@ cudaError_t prepare_order_batch(uint32_t max_n, uint32_t max_w, size_t *smem)
     return kernel_smem_setup((const void *)order_batch_kernel);
 }
 
-cudaError_t launch_order_batch(const BatchGraph *graphs, uint32_t count, uint32_t max_n, size_t smem, cudaStream_t s)
+cudaError_t launch_order_batch(const BatchGraph *graphs, uint32_t count, size_t smem, cudaStream_t s)
 {
-    (void)max_n;
     if (count == 0) return cudaSuccess;
     order_batch_kernel<<<count, 256, smem, s>>>(graphs, smem);
     return cudaGetLastError();

@@ -46,11 +46,10 @@ constexpr unsigned kCasTries = 1u << 14; // bound of one queue ticket loop
 // smallest candidate-set size k whose random subgraph G(k, p) has at least
 // 256, 2048 or 16384 maximal cliques in expectation
 // (sum_j C(k,j) p^C(j,2) (1-p^j)^(k-j)).  A frame is given to the block ring
-// when its candidate set reaches the first, to the device-wide ring when it
-// reaches the second, and a new subtree is published breadth-first when it
-// reaches the third: what moves must carry enough work to pay for the move,
-// and the further it moves the more work that takes.  The two sharing
-// thresholds are capped by a fraction of n (see density_thresholds).
+// or the device-wide ring when its candidate set reaches the first: what moves
+// must carry enough work to pay for the move.  The second and third bound the
+// warp tier's subproblems, and a new subtree of the third (at most half of the
+// vertices) is published breadth-first (see density_thresholds).
 __constant__ unsigned short kShareLocalByDensity[39] = {147, 111, 96, 87, 80, 73, 68, 63, 58, 55, 52, 49, 47,
                                                         44,  42,  41, 39, 37, 36, 35, 33, 32, 31, 30, 29, 29,
                                                         28,  27,  26, 26, 25, 25, 25, 25, 25, 25, 26, 28, 34};
@@ -431,14 +430,13 @@ struct LocalQ {
     unsigned mask;  // slots - 1
 };
 
-__device__ __forceinline__ LocalQ local_queue_at(unsigned char *base, uint32_t wp, uint32_t slots = kLocalSlots)
+__device__ __forceinline__ LocalQ local_queue_at(unsigned char *base)
 {
     LocalQ q;
     q.h = reinterpret_cast<LocalHdr *>(base);
     q.seq = reinterpret_cast<unsigned *>(base + sizeof(LocalHdr));
-    q.frames = reinterpret_cast<uint32_t *>(base + sizeof(LocalHdr) + (size_t)slots * 4);
-    q.mask = slots - 1u;
-    (void)wp;
+    q.frames = reinterpret_cast<uint32_t *>(base + sizeof(LocalHdr) + kLocalSlots * 4u);
+    q.mask = kLocalSlots - 1u;
     return q;
 }
 
@@ -651,8 +649,8 @@ __device__ __forceinline__ unsigned pool_first(const uint32_t (&s)[W])
     return base + (unsigned)__ffs(w) - 1u;
 }
 
-// Hand one subproblem to the warp's tier (all 32 lanes): `mine` are this
-// lane's words of U = P u X; the caller has written the positions of U with
+// Hand one subproblem to the warp's tier (all 32 lanes): `mine` is this
+// lane's (first) word of U = P u X; the caller has written the positions of U with
 // their flags to the slot.  Lane i builds the local rows of U[i], U[i + 32],
 // ...: it walks its rows in word order, four words a load, and for every
 // vertex U[j] of a word (the same word and bit in every lane) rotates that
@@ -664,8 +662,8 @@ __device__ __forceinline__ unsigned pool_first(const uint32_t (&s)[W])
 // makes the local row.  The start frame goes on the stack as frame `slot`.
 template <int W, int K>
 __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const uint32_t *order, uint32_t region,
-                                        unsigned slot, uint32_t mine0, uint32_t mine1, uint32_t mine2, uint32_t mine3,
-                                        unsigned u, unsigned children, unsigned rs, uint64_t S)
+                                        unsigned slot, uint32_t mine, unsigned u, unsigned children, unsigned rs,
+                                        uint64_t S)
 {
     using Sh = PoolShape<W>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -707,7 +705,7 @@ __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const
             }
         };
         const unsigned V = rw >= 4u ? 4u : rw;  // words of a load (rows are 1, 2 or a multiple of 4 words)
-        const unsigned sw = min(rw, 32u * K);
+        const unsigned sw = min(rw, 32u);
 #pragma unroll 1
         for (unsigned w0 = 0; w0 < sw && j < u; w0 += 4u) {
             // U's next four words (uniform), and the rows' (skipped where U has none)
@@ -715,11 +713,7 @@ __device__ __noinline__ void pool_build(const uint32_t *rows, uint32_t rw, const
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const unsigned wi = w0 + t;
-                uint32_t x = mine0;
-                if (K > 1 && (wi % K) == 1u) x = mine1;
-                if (K > 2 && (wi % K) == 2u) x = mine2;
-                if (K > 2 && (wi % K) == 3u) x = mine3;
-                m[t] = __shfl_sync(FULL, x, (int)((wi / K) & 31u));
+                m[t] = __shfl_sync(FULL, mine, (int)(wi & 31u));
                 if (wi >= sw) m[t] = 0u;
             }
             if ((m[0] | m[1] | m[2] | m[3]) == 0u) continue;
@@ -824,7 +818,7 @@ __device__ __noinline__ bool pool_give(const PoolAt at, uint32_t frame, bool loc
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const unsigned lane = threadIdx.x & 31u;
     LocalHdr *h = reinterpret_cast<LocalHdr *>(smem_raw + at.lq);
-    const LocalQ lq = local_queue_at(smem_raw + at.lq, h->wp, h->slots);
+    const LocalQ lq = local_queue_at(smem_raw + at.lq);
     uint32_t *f = reinterpret_cast<uint32_t *>(smem_raw + frame);
     const uint32_t meta = f[2 * W];
     const unsigned slot = (meta >> 7) & 7u, left = ((meta >> 17) & 127u) - (meta >> 24);
@@ -1328,7 +1322,6 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
         h->fs = prm.fs;
         h->margin = push_margin(prm);
         h->wp = rw;
-        h->slots = lq.mask + 1u;
         h->n = n;
         h->give_p = prm.tune.give_p ? prm.tune.give_p : th.share;
         h->total = ring_shared ? prm.total_groups : warps;
@@ -1596,7 +1589,7 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
         const unsigned slots = th.cls == 1u ? PoolShape<1>::kSlots : (th.cls == 2u ? PoolShape<2>::kSlots : 1u);
         if (pslots >= slots) pool_flush();
         const unsigned slot = pslots++;
-        uint32_t U[4] = {0u, 0u, 0u, 0u};
+        uint32_t U[K];
         unsigned cnt = 0;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -1617,13 +1610,13 @@ __device__ __forceinline__ void search_loop(const SearchParams &prm, const uint3
         }
         __syncwarp();
         if (th.cls == 1u)
-            pool_build<1, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<1, K>(rows, rw, prm.order, at.region, slot, U[0], u, children, trs, tS);
         else if (th.cls == 2u)
-            pool_build<2, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<2, K>(rows, rw, prm.order, at.region, slot, U[0], u, children, trs, tS);
         else if (th.cls == 3u)
-            pool_build<3, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<3, K>(rows, rw, prm.order, at.region, slot, U[0], u, children, trs, tS);
         else
-            pool_build<4, K>(rows, rw, prm.order, at.region, slot, U[0], U[1], U[2], U[3], u, children, trs, tS);
+            pool_build<4, K>(rows, rw, prm.order, at.region, slot, U[0], u, children, trs, tS);
     };
     // whether a frame of |P| = np, |P u X| = u and c children fits the tier
     auto pool_fits = [&](unsigned np, unsigned u, unsigned c) -> bool {
@@ -2053,7 +2046,7 @@ __global__ void __launch_bounds__(T) search_kernel(const SearchParams prm)
     const uint32_t n = prm.n;
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw);
     const uint32_t lq_off = (uint32_t)smem_local_offset(n);
-    const LocalQ lq = local_queue_at(smem_raw + lq_off, prm.wp, prm.local_slots);
+    const LocalQ lq = local_queue_at(smem_raw + lq_off);
     local_queue_reset(lq, blockDim.x / 32u);
 
 #pragma unroll 1
@@ -2086,9 +2079,9 @@ __global__ void __launch_bounds__(T) search_kernel(const SearchParams prm)
 // Batched form: each block takes graphs of its bucket one at a time, most
 // expensive first, and searches each with its own block-local queue region
 // (the same frame ring as the single-graph kernel, private to the block).
-// Per graph: output initialised with the root counted (status kept), rows
-// bulk-copied to shared memory, root frame queued, search, reduction into the
-// graph's own result array.
+// Per graph: the root counted (status kept), frames of its children (or a
+// subproblem's root) queued, search, reduction into the graph's own result
+// array.
 template <int K, int PIVOT, int T>
 __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
 {
@@ -2113,7 +2106,7 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
         const BatchGraph gd = bp.graphs[item & 0xffffu];
         const uint32_t n = gd.n, WP = gd.wp;
         uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw);
-        const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n), WP);
+        const LocalQ lq = local_queue_at(smem_raw + smem_local_offset(n));
         local_queue_reset(lq, bp.groups_per_block);
         const bool valid = gd.out[MCE_OUT_STATUS] == 0ull;
         // The root's P and X over positions: all of V and nothing, or, for a
@@ -2303,7 +2296,6 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
         prm.split_target = bp.split_target;
         prm.tune = bp.tune;
         prm.count_root = 1;
-        prm.local_slots = kLocalSlots;
         prm.t2_offset = bp.t2_offset;
         prm.pool_bytes = bp.pool_bytes;
         prm.t2_max_p = bp.t2_max_p;
