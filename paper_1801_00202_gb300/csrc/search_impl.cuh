@@ -2140,7 +2140,9 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
         // the root is one node: internal, a leaf (R is maximal) or a dead end;
         // the graph's result array starts zeroed (cleared with the batch) and
         // every part adds to it
-        const bool split = !sub;  // every graph but an outer-loop subproblem starts from its root's children
+        // every graph starts from its root's children, but the outer loop's
+        // subproblems of up to 128 vertices, which one warp takes whole
+        const bool split = !sub || n > 128u;
         if (threadIdx.x == 0 && (!split || part == 0u)) {
             unsigned long long *o = reinterpret_cast<unsigned long long *>(gd.out);
             atomicAdd(o + MCE_OUT_NODES, 1ull);
@@ -2198,7 +2200,7 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
         const bool root = valid && pne && lne;
         // frames of `per` consecutive root children each: with v_t the t-th
         // vertex of L = P \ N(p0), children a..b-1 are the frame (P minus v_0
-        // ..v_{a-1}, X = those, p0, end = v_b); a part takes every parts-th of
+        // ..v_{a-1}, X and those, p0, end = v_b); a part takes every parts-th of
         // them.  Frames go to slots 1.. (slot 0 keeps the root's P and X).
         // per: what makes a frame worth taking, and what the ring has room for.
         unsigned queued = root ? 1u : 0u;
@@ -2215,7 +2217,7 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
             }
             __syncthreads();
             const unsigned nl = lpre[WP];
-            unsigned per = gd.per;
+            unsigned per = sub ? max(1u, nl / bp.groups_per_block) : gd.per;
             if (parts == 1u) per = max(per, (nl + bp.root_frames - 1u) / bp.root_frames);
             const unsigned all = (nl + per - 1u) / per;
             const unsigned mine = all > part ? (all - part + parts - 1u) / parts : 0u;
@@ -2237,12 +2239,12 @@ __global__ void __launch_bounds__(T) batch_kernel(const BatchParams bp)
                     else if (v > q * 32u) below = (1u << (v - q * 32u)) - 1u;
                     const uint32_t x = pw & ~rp0[q] & below;
                     fr[kFrameHdr + q] = pw & ~x;
-                    fr[kFrameHdr + WP + q] = x;
+                    fr[kFrameHdr + WP + q] = frames[kFrameHdr + WP + q] | x;
                 }
                 fr[0] = (p0 & 0xffffu) | (end << 16);
-                fr[1] = 0u;
-                fr[2] = 0u;
-                fr[3] = 0u;
+                fr[1] = r0;
+                fr[2] = (uint32_t)s0;
+                fr[3] = (uint32_t)(s0 >> 32);
                 fr[4] = 0u;
             }
             queued = valid && pne ? min(mine, bp.qcap - 1u) : 0u;
