@@ -87,11 +87,11 @@ __global__ void validate_kernel(uint32_t n, uint32_t w, const uint32_t *__restri
 // 31, a graph of up to 128 vertices one round.  What bounds it is the chain of
 // picks, about 0.1 us each (max-reduction, one broadcast load, four
 // subtractions), and 3 to 5 us of gathering and barriers a round.  A search of
-// all vertices for one or two picks a round took, per launch (G(n, p), now in
-// brackets): n = 100 24 us (16), 300 85 (55), 500 146 (94), 1000 383 (237),
-// 3000 4345 (915; rows in L2, two dependent reads a round).  The pass that
-// lowers the degrees counts them for the next round's classes as well: 4 % of
-// the launch against a pass and a barrier of its own (1000: 248, 3000: 952).
+// all vertices for one or two picks a round took, per call by events (G(n, p),
+// now in brackets): n = 100 32 us (24), 300 96 (62), 500 152 (118), 1000 359
+// (238), 2000 1993 (452), 3000 4369 (843; rows in L2, two dependent reads a
+// round).  The pass that lowers the degrees counts them for the next round's
+// classes as well: 4 % of the launch against a pass and a barrier of its own.
 constexpr unsigned kOrderCand = 128;
 constexpr unsigned kSmallPrepThreads = 256, kSmallPrepVerts = 128, kSmallPrepWords = 4;
 
@@ -542,16 +542,15 @@ cudaError_t launch_validate_rows(uint32_t n, uint32_t w, const uint32_t *rows, u
 cudaError_t launch_order(uint32_t n, uint32_t w, const uint32_t *rows, uint32_t *order, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    // rows in shared memory up to 200 KB; more threads where there are more
-    // vertices to look at, fewer where barriers cost more than they save (256 /
-    // 512 / 1024 threads: n = 500 122 / 121 / 127 us, 1000 266 / 253 / 278, 3000
-    // 961 / 812 / 756)
+    // rows in shared memory up to 200 KB; 512 threads, fewer where barriers
+    // cost more than they save (256 / 512 / 1024 threads, us by events: n = 500
+    // 116 / 118 / 124, 1000 245 / 238 / 265, 2000 521 / 452 / 519, 3000 952 / 843 /
+    // 915; 512 / 1024: 4096 1346 / 1443)
     const size_t fixed = order_fixed_bytes(n), rbytes = (size_t)n * w * 4;
     const int in_smem = fixed + rbytes <= 200u * 1024u;
     const size_t smem = fixed + (in_smem ? rbytes : 0);
-    const unsigned threads = n <= 128 ? 128u : (n <= 1024 ? 512u : 1024u);
-    void (*f)(uint32_t, uint32_t, const uint32_t *, uint32_t *, int) =
-        threads == 128u ? order_kernel<128> : (threads == 512u ? order_kernel<512> : order_kernel<1024>);
+    const unsigned threads = n <= 128 ? 128u : 512u;
+    void (*f)(uint32_t, uint32_t, const uint32_t *, uint32_t *, int) = n <= 128 ? order_kernel<128> : order_kernel<512>;
     cudaError_t e = kernel_smem_setup((const void *)f);
     if (e != cudaSuccess) return e;
     f<<<1, threads, smem, s>>>(n, w, rows, order, in_smem);

@@ -223,7 +223,7 @@ __device__ __forceinline__ void set_status(uint64_t *out, Ctl *ctl, int code)
 // frame for consumer `ticket`).
 
 // Reserve a producer ticket: check the room left -- producer tickets at
-// most qcap - margin ahead of the consumers', margin = the groups that can
+// most qcap - margin ahead of the consumers', margin = the warps that can
 // reserve at once (one ticket each) -- and take the ticket with one
 // fetch-and-add, so producers race no compare-and-swap either.  The room
 // check puts the ticket's slot behind a consumer ticket already claimed, so
@@ -247,7 +247,7 @@ __device__ __forceinline__ bool q_reserve_push(Ctl *ctl, unsigned *seq, unsigned
 }
 
 // Take the oldest published frame of a block-private ring (batched form:
-// the only contenders are the block's own groups, so a compare-and-swap on
+// the only contenders are the block's own warps, so a compare-and-swap on
 // the head is cheap there).
 __device__ __forceinline__ bool q_reserve_pop(Ctl *ctl, unsigned *seq, unsigned mask, unsigned &ticket,
                                               unsigned long long *fails, unsigned tries = kCasTries)
